@@ -454,7 +454,7 @@ def dense_gemv(A: torch.Tensor, x: torch.Tensor, y: Optional[torch.Tensor] = Non
     need = dense_gemv_workspace(m, n, layout, s, cfg)
     ws_ptr, ws_bytes = None, 0
     if need > 0:
-        if workspace is None:
+        if workspace is None or layout == "row":      # the caller's serves column-major calls
             workspace = _workspace(need, sh, A.device)
         ws_ptr = _dev_ptr(workspace, "workspace")
         ws_bytes = workspace.numel() * workspace.element_size()
@@ -487,7 +487,7 @@ def dense_gemv_trans(A: torch.Tensor, x: torch.Tensor, y: Optional[torch.Tensor]
     need = dense_gemv_workspace(n, m, other, s, cfg)
     ws_ptr, ws_bytes = None, 0
     if need > 0:
-        if workspace is None:
+        if workspace is None or other == "row":
             workspace = _workspace(need, sh, A.device)
         ws_ptr, ws_bytes = _dev_ptr(workspace, "workspace"), workspace.numel()
     st = _lib.dense_gemv_trans(_vec_arg(y, "y"), _dev_ptr(A, "A"), _vec_arg(x, "x"), m, n, lda,

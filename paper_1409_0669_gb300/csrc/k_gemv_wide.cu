@@ -1,0 +1,366 @@
+// Dense products whose shape or alignment the one-group-per-row and the
+// tile-per-block kernels of k_gemv.cu serve badly:
+//
+//   gemv_rows_kernel   row-major: R rows of one alignment share every load of x,
+//                      their columns can be split over blocks, and x may start at
+//                      any offset against the rows
+//   gemv_tall_kernel   column-major with very many rows: a thread owns its rows
+//                      over all columns, no combine at all
+//
+// Both compute y = alpha * A x + beta * y (y is not read when beta == 0).
+#include "lak_internal.cuh"
+
+namespace lak {
+namespace {
+
+template <typename T>
+__device__ __forceinline__ T epilogue(typename Acc<T>::type t, typename Acc<T>::type alpha,
+                                      typename Acc<T>::type beta, typename Acc<T>::type yold) {
+    using Ac = typename Acc<T>::type;
+    if (beta == Ac(0)) return narrow<T>(alpha * t);
+    return narrow<T>(fma_acc(alpha, t, beta * yold));
+}
+
+// acc + <a, x> over one pack, as one FMA chain
+template <typename T, int V>
+__device__ __forceinline__ typename Acc<T>::type pack_dot(typename Acc<T>::type acc,
+                                                          const Pack<T, V> &a,
+                                                          const Pack<T, V> &x) {
+#pragma unroll
+    for (int v = 0; v < V; ++v) acc = fma_wide(a.e[v], x.e[v], acc);
+    return acc;
+}
+
+// ---- row-major: R rows per block, columns split over blocks ------------------------
+//
+// What bounds the shapes this serves: few long rows left the GPU idle (one block per
+// row: 30 rows of 2,097,152 FP64 ran as 30 warps), and rows whose length is not a
+// multiple of 16 bytes start at other offsets than x, so the one-row kernel loads x
+// one element at a time.
+//
+// Layout.  Rows r, r + P, ..., r + (R-1) P with P the smallest stride (a power of two,
+// at most 16 bytes / element) at which rows start at the same offset modulo 16 bytes:
+// a block takes one such set, so one head, one aligned body and ONE load of x serve R
+// rows, with R 16-byte loads of A in flight per lane and step.  x is read through two
+// aligned 16-byte loads whose 32 bytes are shifted in registers by the set's offset
+// (uniform over the block; the second load hits L1).  blockIdx.y is the column split:
+// with more than one, partial sums go to the workspace and the last block of a set to
+// arrive adds them in split order (deterministic).  No load leaves [x, x + n) or the
+// rows: packs whose window would are done one element at a time.
+//
+// Dependents may launch once every block is past its body, not at entry: a grid that
+// starts while SMs of this one are still busy puts most of its few blocks on the SMs
+// that are free first (4096 x 16384 FP64 by two rows: 208 us with the trigger at
+// entry, 127 us here).
+//
+// Measured (us, before -> with row sets): 30 x 2097152 FP64 12110 -> 121 (FP64 pipe: 100),
+// FP32 3780 -> 45 (5.6 TB/s); BF16 12007 x 11003 79 -> 45.6 (5.8 TB/s); FP32 16384 x
+// 16383 252 -> 155 (6.9 TB/s); FP64 4096 x 16384 150 -> 122.
+template <typename T, int R>
+__global__ void __launch_bounds__(256, R == 1 ? 4 : 2)
+gemv_rows_kernel(T *__restrict__ y, const T *__restrict__ A, const T *__restrict__ x, int64_t m,
+                 int64_t n, int64_t lda, int P, typename Acc<T>::type alpha,
+                 typename Acc<T>::type beta, typename Acc<T>::type *__restrict__ partials,
+                 unsigned int *__restrict__ tickets) {
+    LAK_PDL_WAIT();
+    using Ac = typename Acc<T>::type;
+    constexpr int ES = (int)sizeof(T);
+    constexpr int V = 16 / ES;
+    __shared__ Ac red[8][R];
+    __shared__ int am_last;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+    const int64_t set = blockIdx.x;
+    const int64_t row0 = (set / P) * ((int64_t)R * P) + set % P;
+    if (row0 >= m) return;                                  // block-uniform
+    const int64_t left = (m - row0 + P - 1) / P;            // rows from row0 on, P apart
+    const int nr = left < R ? (int)left : R;
+    const int split = blockIdx.y, nsplit = gridDim.y;
+
+    const T *a = A + row0 * lda;
+    const int64_t step = (int64_t)P * lda;                  // from row to row of the set
+    const int64_t mis = (int64_t)((uintptr_t)a % 16) / ES;
+    int64_t h = mis ? V - mis : 0;
+    if (h > n) h = n;
+    int64_t b0 = 0, b1 = (n - h) / V;                       // packs of the body
+    const uint32_t sb = (uint32_t)((uintptr_t)(x + h) % 16);
+    if (sb) {
+        // the window of pack c: 32 bytes from x + h + c V - sb/ES
+        if (h * ES < sb) b0 = 1;
+        if (h + b1 * V + V - (int64_t)sb / ES > n) --b1;
+        if (b1 < b0) b1 = b0 = 0;
+    }
+    const int64_t head = b1 > b0 ? h + b0 * V : n;          // elements done one by one
+    const int64_t tail = b1 > b0 ? h + b1 * V : n;
+
+    Ac acc[R];
+#pragma unroll
+    for (int j = 0; j < R; ++j) acc[j] = Ac(0);
+    if (split == 0)
+        for (int64_t k = tid; k < head; k += blockDim.x) {
+            const T xv = ld_cached(x + k);
+#pragma unroll
+            for (int j = 0; j < R; ++j)
+                if (j < nr) acc[j] = fma_wide(a[j * step + k], xv, acc[j]);
+        }
+    if (split == nsplit - 1)
+        for (int64_t k = tail + tid; k < n; k += blockDim.x) {
+            const T xv = ld_cached(x + k);
+#pragma unroll
+            for (int j = 0; j < R; ++j)
+                if (j < nr) acc[j] = fma_wide(a[j * step + k], xv, acc[j]);
+        }
+    const int64_t per = (b1 - b0 + nsplit - 1) / nsplit;
+    const int64_t s0 = b0 + split * per;
+    const int64_t s1 = s0 + per < b1 ? s0 + per : b1;
+    const T *ab = a + h;
+    const T *xb = x + h;
+    auto body = [&](auto shifted, auto full) {
+        // U packs a step: their loads are issued together, and FP32 sums them before
+        // the one add to the running sum
+        constexpr int U = R == 1 ? 4 : 2;
+        auto load_x = [&](Pack<T, V> &px, int64_t c) {
+            if constexpr (shifted.value)
+                load_window<T, CACHED>(px, xb + c * V, sb);
+            else
+                load_pack<T, V, CACHED>(px, xb + c * V);
+        };
+        int64_t c = s0 + tid;
+        for (; c + (U - 1) * (int64_t)blockDim.x < s1; c += U * (int64_t)blockDim.x) {
+            Pack<T, V> px[U], pa[U][R];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int64_t cu = c + u * (int64_t)blockDim.x;
+#pragma unroll
+                for (int j = 0; j < R; ++j)
+                    if (full.value || j < nr)
+                        load_pack<T, V, STREAM>(pa[u][j], ab + j * step + cu * V);
+                load_x(px[u], cu);
+            }
+#pragma unroll
+            for (int j = 0; j < R; ++j) {
+                if (!full.value && j >= nr) continue;
+                if constexpr (sizeof(Ac) == 8) {
+#pragma unroll
+                    for (int u = 0; u < U; ++u) acc[j] = pack_dot<T, V>(acc[j], pa[u][j], px[u]);
+                } else {
+                    Ac t = Ac(0);
+#pragma unroll
+                    for (int u = 0; u < U; ++u) t = pack_dot<T, V>(t, pa[u][j], px[u]);
+                    acc[j] += t;
+                }
+            }
+        }
+        for (; c < s1; c += blockDim.x) {
+            Pack<T, V> px;
+            load_x(px, c);
+#pragma unroll
+            for (int j = 0; j < R; ++j) {
+                if (!full.value && j >= nr) continue;
+                Pack<T, V> pa;
+                load_pack<T, V, STREAM>(pa, ab + j * step + c * V);
+                acc[j] += pack_dot<T, V>(Ac(0), pa, px);
+            }
+        }
+    };
+    using Yes = Flag<true>;
+    using No = Flag<false>;
+    if (nr == R) {
+        if (sb) body(Yes{}, Yes{}); else body(No{}, Yes{});
+    } else {
+        if (sb) body(Yes{}, No{}); else body(No{}, No{});
+    }
+
+    LAK_PDL_TRIGGER();
+    // block sums of the set's rows, held by thread j for row j
+#pragma unroll
+    for (int j = 0; j < R; ++j) acc[j] = group_sum(acc[j], 32);
+    Ac t = Ac(0);
+    if (nw == 1) {
+#pragma unroll
+        for (int j = 0; j < R; ++j)
+            if (lane == j) t = acc[j];
+    } else {
+        if (lane == 0) {
+#pragma unroll
+            for (int j = 0; j < R; ++j) red[warp][j] = acc[j];
+        }
+        __syncthreads();
+        if (tid < nr)
+            for (int w = 0; w < nw; ++w) t += red[w][tid];
+    }
+    if (nsplit == 1) {
+        if (tid < nr) {
+            const int64_t row = row0 + (int64_t)tid * P;
+            const Ac yold = beta != Ac(0) ? widen(y[row]) : Ac(0);
+            y[row] = epilogue<T>(t, alpha, beta, yold);
+        }
+        return;
+    }
+    if (tid < nr) partials[(int64_t)split * m + row0 + (int64_t)tid * P] = t;
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) am_last = ticket_acq_rel(tickets + set, nsplit - 1) == (unsigned)nsplit - 1;
+    __syncthreads();
+    if (!am_last) return;
+    for (int j = warp; j < nr; j += nw) {
+        const int64_t row = row0 + (int64_t)j * P;
+        double f = 0.0;                                     // split order per lane, then a tree
+#pragma unroll 8
+        for (int q = lane; q < nsplit; q += 32) f += (double)__ldcg(partials + (int64_t)q * m + row);
+        f = group_sum(f, 32);
+        if (lane == 0) {
+            const Ac yold = beta != Ac(0) ? widen(y[row]) : Ac(0);
+            y[row] = epilogue<T>((Ac)f, alpha, beta, yold);
+        }
+    }
+}
+
+// ---- column-major with very many rows ----------------------------------------------
+//
+// A thread owns V consecutive rows and walks all columns: every warp load is 32 V
+// consecutive entries of one column, and nothing is combined between threads (the
+// tile-per-block kernel splits its columns over the block's warps and adds their sums
+// in shared memory, which for 30 FP64 columns was a quarter of its FP64 work).
+// SHIFT: columns start at other offsets than a multiple of 16 bytes; each pack is
+// then read through two aligned loads and shifted by the column's offset (uniform
+// over the grid; the second load hits L1).  The first and the last column, whose
+// windows could leave the matrix, are read one element at a time.  Measured (us): FP64
+// 2097152 x 30 134 -> 121 (FP64 pipe: 107 with the epilogue), FP32 1000000 x 8 16.1 ->
+// 6.8, odd 999983 x 17 90 -> 15.5 (4.4 TB/s).
+template <typename T, int V, bool SHIFT>
+__global__ void __launch_bounds__(256)
+gemv_tall_kernel(T *__restrict__ y, const T *__restrict__ A, const T *__restrict__ x, int64_t m,
+                 int64_t n, int64_t lda, typename Acc<T>::type alpha,
+                 typename Acc<T>::type beta, bool y_ok) {
+    LAK_PDL_ENTRY();
+    using Ac = typename Acc<T>::type;
+    const int64_t r0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * V;
+    if (r0 >= m) return;
+    const T *a = A + r0;
+    if (r0 + V > m) {                                       // the last rows
+        for (int64_t r = r0; r < m; ++r) {
+            Ac t = Ac(0);
+            for (int64_t j = 0; j < n; ++j) t = fma_wide(A[j * lda + r], ld_cached(x + j), t);
+            const Ac yold = beta != Ac(0) ? widen(y[r]) : Ac(0);
+            y[r] = epilogue<T>(t, alpha, beta, yold);
+        }
+        return;
+    }
+    Ac acc[V];
+#pragma unroll
+    for (int v = 0; v < V; ++v) acc[v] = Ac(0);
+    auto scalar_column = [&](int64_t j) {
+        const T xj = ld_cached(x + j);
+#pragma unroll
+        for (int v = 0; v < V; ++v) acc[v] = fma_wide(a[j * lda + v], xj, acc[v]);
+    };
+    int64_t j = 0, j1 = n;
+    if constexpr (SHIFT) {
+        scalar_column(0);
+        j = 1;
+        j1 = n - 1;
+    }
+#pragma unroll(SHIFT ? 4 : 8)
+    for (; j < j1; ++j) {
+        Pack<T, V> pa;
+        const T *p = a + j * lda;
+        if constexpr (SHIFT)
+            load_window<T, CACHED>(pa, p, (uint32_t)((uintptr_t)p % 16));
+        else
+            load_pack<T, V, STREAM>(pa, p);
+        const T xj = ld_cached(x + j);
+#pragma unroll
+        for (int v = 0; v < V; ++v) acc[v] = fma_wide(pa.e[v], xj, acc[v]);
+    }
+    if constexpr (SHIFT)
+        if (n > 1) scalar_column(n - 1);
+    Pack<T, V> py;
+    if (beta != Ac(0)) {
+        if (y_ok) {
+            load_pack<T, V, COHERENT>(py, y + r0);
+        } else {
+#pragma unroll
+            for (int v = 0; v < V; ++v) py.e[v] = y[r0 + v];
+        }
+    }
+#pragma unroll
+    for (int v = 0; v < V; ++v)
+        py.e[v] = epilogue<T>(acc[v], alpha, beta, beta != Ac(0) ? widen(py.e[v]) : Ac(0));
+    if (y_ok) {
+        store_pack<T, V>(y + r0, py);
+    } else {
+#pragma unroll
+        for (int v = 0; v < V; ++v) y[r0 + v] = py.e[v];
+    }
+}
+
+template <typename T>
+lak_status rows_t(void *y, const void *A, const void *x, int64_t m, int64_t n, int64_t lda,
+                  const RowsLaunch &L, void *ws, double alpha, double beta, cudaStream_t s) {
+    using Ac = typename Acc<T>::type;
+    T *yp = static_cast<T *>(y);
+    const T *Ap = static_cast<const T *>(A);
+    const T *xp = static_cast<const T *>(x);
+    unsigned int *tickets = static_cast<unsigned int *>(ws);
+    Ac *partials = nullptr;
+    if (L.splits > 1)
+        partials = reinterpret_cast<Ac *>(static_cast<char *>(ws) + LAK_WS_COUNTER_BYTES);
+    const dim3 grid((unsigned)L.sets, (unsigned)L.splits);
+#define LAK_ROWS(RR)                                                                           \
+    launch_k(gemv_rows_kernel<T, RR>, grid, L.block, 0, s, yp, Ap, xp, m, n, lda, L.period,    \
+             (Ac)alpha, (Ac)beta, partials, tickets)
+    if (L.rows == 1)
+        LAK_ROWS(1);
+    else
+        LAK_ROWS(4);
+#undef LAK_ROWS
+    return check_launch("dense_gemv (row-major, row sets)");
+}
+
+template <typename T>
+lak_status tall_t(void *y, const void *A, const void *x, int64_t m, int64_t n, int64_t lda,
+                  double alpha, double beta, cudaStream_t s) {
+    using Ac = typename Acc<T>::type;
+    constexpr int V = 16 / (int)sizeof(T);
+    constexpr int block = kGemvTallBlock;
+    T *yp = static_cast<T *>(y);
+    const T *Ap = static_cast<const T *>(A);
+    const T *xp = static_cast<const T *>(x);
+    const bool aligned = (uintptr_t)A % 16 == 0 && (lda * (int64_t)sizeof(T)) % 16 == 0;
+    const bool y_ok = (uintptr_t)y % 16 == 0;
+    const unsigned grid = (unsigned)ceil_div(m, (int64_t)V * block);
+    if (aligned)
+        launch_k(gemv_tall_kernel<T, V, false>, grid, block, 0, s, yp, Ap, xp, m, n, lda,
+                 (Ac)alpha, (Ac)beta, y_ok);
+    else
+        launch_k(gemv_tall_kernel<T, V, true>, grid, block, 0, s, yp, Ap, xp, m, n, lda,
+                 (Ac)alpha, (Ac)beta, y_ok);
+    return check_launch("dense_gemv (column-major, many rows)");
+}
+
+}  // namespace
+
+lak_status launch_gemv_rows(lak_dtype dt, void *y, const void *A, const void *x, int64_t m,
+                            int64_t n, int64_t lda, const RowsLaunch &L, void *ws, double alpha,
+                            double beta, cudaStream_t s) {
+    switch (dt) {
+    case LAK_F32: return rows_t<float>(y, A, x, m, n, lda, L, ws, alpha, beta, s);
+    case LAK_F64: return rows_t<double>(y, A, x, m, n, lda, L, ws, alpha, beta, s);
+    case LAK_BF16: return rows_t<__nv_bfloat16>(y, A, x, m, n, lda, L, ws, alpha, beta, s);
+    case LAK_F16: return rows_t<__half>(y, A, x, m, n, lda, L, ws, alpha, beta, s);
+    }
+    return fail(LAK_EDTYPE, "dense_gemv: unknown dtype %d", (int)dt);
+}
+
+lak_status launch_gemv_tall(lak_dtype dt, void *y, const void *A, const void *x, int64_t m,
+                            int64_t n, int64_t lda, double alpha, double beta, cudaStream_t s) {
+    switch (dt) {
+    case LAK_F32: return tall_t<float>(y, A, x, m, n, lda, alpha, beta, s);
+    case LAK_F64: return tall_t<double>(y, A, x, m, n, lda, alpha, beta, s);
+    case LAK_BF16: return tall_t<__nv_bfloat16>(y, A, x, m, n, lda, alpha, beta, s);
+    case LAK_F16: return tall_t<__half>(y, A, x, m, n, lda, alpha, beta, s);
+    }
+    return fail(LAK_EDTYPE, "dense_gemv: unknown dtype %d", (int)dt);
+}
+
+}  // namespace lak

@@ -355,6 +355,102 @@ lak_status plan_gemv_row(lak_dtype dt, int64_t m, int64_t n, int64_t lda, const 
     return LAK_OK;
 }
 
+int64_t env_int(const char *name, int64_t dflt) {
+    const char *e = getenv(name);
+    if (e && *e) {
+        char *end = nullptr;
+        const long long x = strtoll(e, &end, 10);
+        if (end && *end == 0 && x >= 0) return (int64_t)x;
+    }
+    return dflt;
+}
+
+// Whether a call takes the op's built-in launch shape: no explicit cfg and no
+// override installed for its size bucket.
+bool builtin_shape(lak_op op, lak_dtype dt, int bucket, const lak_cfg *cfg) {
+    if (cfg && cfg->block != 0) return false;
+    std::lock_guard<std::mutex> lk(g_cfg_mu);
+    return !g_has_override[op][dt][bucket];
+}
+
+// Row-major products taken by sets of rows (gemv_rows_kernel, k_gemv_wide.cu);
+// rows = 0 where the one-row kernel keeps the call.  Every line is drawn where both
+// kernels were timed (back to back launches over buffers larger than L2, us, one-row
+// kernel -> row sets):
+//   FP64 from 768 columns (x or rows off 16 bytes: from 2048): one row per set, so
+//     that many small blocks balance the FP64 pipe: 4096^2 38.1 -> 34.5, 12007 x 11003
+//     265 -> 240, 16384^2 457 -> 449, 300 x 100000 598 -> 58; 4096 x 512 7.5 -> 8.3
+//   FP32 and 16 bits, rows of 96 packs of 16 bytes and more:
+//     rows that start at other offsets than x: BF16 12007 x 11003 78.7 -> 45, FP32
+//       4096 x 4095 26.7 -> 12.8; below 8 MiB (bucket 0) both take 2-5 us
+//     few rows of 32 KB and more: FP32 300 x 100000 158 -> 28, 300 x 4096 3.8 -> 4.8
+//     aligned rows from 8 MiB on: 4096^2 FP32 13.3 -> 12.5, BF16 9.7 -> 7.1, BF16
+//       16384^2 87.7 -> 80; FP32 16384^2 155 -> 156, so FP32 stops at 512 MiB;
+//       16384 x 256 FP32 5.1 -> 8.2
+RowsLaunch plan_gemv_rows(lak_dtype dt, int64_t m, int64_t n, int64_t lda, const lak_cfg *cfg,
+                          const void *A, const void *x) {
+    RowsLaunch R{};
+    const int bucket = bucket_of(op_bytes(LAK_OP_GEMV_ROW, dt, m, n, 0));
+    const int es = esize(dt);
+    const bool f64 = es == 8;
+    const int64_t nch = n / (16 / es);                   // 16-byte packs of a row
+    const bool off = (lda * es) % 16 || (uintptr_t)A % 16 || (uintptr_t)x % 16;
+    const bool few = m <= (bucket == 0 ? 128 : 600) && n * es >= 32768;
+    if (f64) {
+        if (nch < (off ? 1024 : 384)) return R;
+    } else {
+        if (nch < 96) return R;
+        if (!few && (bucket == 0 || (!off && es == 4 && bucket == 3))) return R;
+        if (!few && !off && m <= 600) return R;
+    }
+    if (m == 0 || !builtin_shape(LAK_OP_GEMV_ROW, dt, bucket, cfg)) return R;
+    const DeviceInfo *di = device_info();
+    if (!di) return R;
+    R.period = 1;
+    while ((lda * es * R.period) % 16) R.period *= 2;
+    // one row per set where sets of four would leave SMs unevenly filled: FP32
+    // 1000 x 4096 4.5 against 8.2, 1000 x 16384 12.2 against 16; 2000 x 8000 13.0
+    // with four against 14.1
+    R.rows = f64 || (m > 600 && m < 1536) || m < 4 * R.period ? 1 : 4;
+    R.sets = ceil_div(m, (int64_t)R.rows * R.period) * R.period;
+    // threads per set: a dozen packs or so per thread and row, more threads when the
+    // sets alone would leave the SMs with few warps
+    int64_t g = R.rows == 4 ? nch / 11 : f64 ? nch / 120 : 128;
+    const int lo = 32, hi = R.rows == 4 ? 256 : f64 ? 64 : 128;
+    R.block = pow2_floor(g < lo ? lo : g > hi ? hi : g);
+    const int64_t warps = R.rows == 4 ? 8LL * di->sms : 13LL * di->sms;
+    while (R.block < 256 && R.sets * (R.block / 32) < warps && nch >= 8LL * R.block) R.block *= 2;
+    // column splits where one wave of blocks leaves SMs idle; four waves of smaller
+    // blocks where the rows are long enough (30 x 2097152 FP64: 130 -> 118 us)
+    R.splits = 1;
+    const int64_t resident = (R.rows == 4 ? 2LL : 4LL) * di->sms;
+    if (R.block == 256 && R.sets <= LAK_WS_COUNTER_BYTES / 4) {
+        int64_t s = resident / R.sets;
+        if (nch >= 4 * s * 256 * 16) s *= 4;
+        if (s > nch / 2048) s = nch / 2048;
+        if (s > 1) R.splits = (int)s;
+    }
+    return R;
+}
+
+size_t rows_ws_bytes(const RowsLaunch &R, lak_dtype dt, int64_t m) {
+    if (R.rows == 0 || R.splits < 2) return 0;
+    return (size_t)LAK_WS_COUNTER_BYTES + (size_t)R.splits * (size_t)m * (dt == LAK_F64 ? 8 : 4);
+}
+
+// Column-major products with very many rows and few columns, a thread per 16 bytes
+// of rows (gemv_tall_kernel): from 768 threads per SM on.  Timed against the
+// tile-per-block kernel (us): 2097152 x 30 FP64 134 -> 122, FP32 56 -> 39; 999983 x 17
+// FP32 (odd) 90 -> 15.5; 500000 x 50 FP32 (820 threads per SM) 21.8 -> 17.9; 300000 x
+// 1000 FP32 (490) 173 -> 235.  With more columns the tiles' combine no longer shows.
+bool use_gemv_tall(lak_dtype dt, int64_t m, int64_t n, const lak_cfg *cfg) {
+    if (n < 1 || n > 64 || m < 65536) return false;
+    const DeviceInfo *di = device_info();
+    if (!di || m * esize(dt) / 16 < 768LL * di->sms) return false;
+    return builtin_shape(LAK_OP_GEMV_COL, dt, bucket_of(op_bytes(LAK_OP_GEMV_COL, dt, m, n, 0)),
+                         cfg);
+}
+
 struct ColPlan {
     Launch L;
     int splits;
@@ -403,16 +499,6 @@ struct SpmvPlan {
 
 // Mean row lengths between which the warp-segmented variant is used; below
 // the range one lane (or two) per row, above it a group of lanes per row.
-int64_t env_int(const char *name, int64_t dflt) {
-    const char *e = getenv(name);
-    if (e && *e) {
-        char *end = nullptr;
-        const long long x = strtoll(e, &end, 10);
-        if (end && *end == 0 && x >= 0) return (int64_t)x;
-    }
-    return dflt;
-}
-
 int64_t spmv_seg_min_mean() {
     static const int64_t v = env_int("LAK_SPMV_SEG_MIN_MEAN", 13);
     return v;
@@ -610,12 +696,23 @@ LAK_API lak_status lak_resolve_cfg(lak_op op, lak_dtype dtype, int64_t m, int64_
         break;
     }
     case LAK_OP_GEMV_ROW: {
+        const RowsLaunch R = plan_gemv_rows(dtype, m, n, n > 1 ? n : 1, cfg, nullptr, nullptr);
+        if (R.rows > 0) {
+            L = Launch{R.block, (int)(R.sets * R.splits), 16 / esize(dtype), LAK_INC_GLOBAL};
+            break;
+        }
         RowPlan p;
         st = plan_gemv_row(dtype, m, n, n, cfg, nullptr, nullptr, &p);
         L = p.L;
         break;
     }
     case LAK_OP_GEMV_COL: {
+        if (use_gemv_tall(dtype, m, n, cfg)) {
+            const int v = 16 / esize(dtype);
+            L = Launch{kGemvTallBlock, (int)ceil_div(m, (int64_t)v * kGemvTallBlock), v,
+                       LAK_INC_GLOBAL};
+            break;
+        }
         ColPlan p;
         st = plan_gemv_col(dtype, m, n, m, cfg, nullptr, &p);
         L = p.L;
@@ -805,7 +902,10 @@ LAK_API size_t dense_gemv_workspace(int64_t m, int64_t n, lak_layout layout, lak
                                     const lak_cfg *cfg) {
     if (!valid_dtype(dtype) || m < 0 || n < 0 || check_cfg(cfg, "dense_gemv_workspace") != LAK_OK)
         return 0;
-    if (layout != LAK_COL_MAJOR) return 0;
+    if (layout == LAK_COL_MAJOR && use_gemv_tall(dtype, m, n, cfg)) return 0;
+    if (layout != LAK_COL_MAJOR)
+        return rows_ws_bytes(plan_gemv_rows(dtype, m, n, n > 1 ? n : 1, cfg, nullptr, nullptr),
+                             dtype, m);
     // the widest vec the call could pick gives the fewest tiles; narrower vecs
     // (forced by alignment) only add tiles, so size for vec = 1 as well
     size_t best = 0;
@@ -845,11 +945,21 @@ lak_status gemv_impl(const char *who, void *y, const void *A, const void *x, int
         return fail(LAK_EINVAL, "%s: pointers not aligned to the element size", who);
     cudaStream_t s = (cudaStream_t)stream;
     if (layout == LAK_ROW_MAJOR) {
+        RowsLaunch R = plan_gemv_rows(dtype, m, n, lda, cfg, A, x);
+        if (R.rows > 0) {
+            // the workspace is optional here: without one the columns stay unsplit
+            const size_t need = rows_ws_bytes(R, dtype, m);
+            if (need > 0 && (!workspace || ws_bytes < need || (uintptr_t)workspace % 256))
+                R.splits = 1;
+            return launch_gemv_rows(dtype, y, A, x, m, n, lda, R, workspace, alpha, beta, s);
+        }
         RowPlan p;
         st = plan_gemv_row(dtype, m, n, lda, cfg, A, x, &p);
         if (st != LAK_OK) return st;
         return launch_gemv_row(dtype, y, A, x, m, n, lda, p.L, p.group, alpha, beta, s);
     }
+    if (use_gemv_tall(dtype, m, n, cfg))
+        return launch_gemv_tall(dtype, y, A, x, m, n, lda, alpha, beta, s);
     ColPlan p;
     st = plan_gemv_col(dtype, m, n, lda, cfg, A, &p);
     if (st != LAK_OK) return st;

@@ -71,10 +71,12 @@ inline int access_bytes(int vec, int es) {
 // No kernel touches global memory before the wait, so the stream's ordering is
 // unchanged; launch_k launches with the attribute unless LAK_PDL=0.  (The
 // batched GEMV only waits; it lets its dependents launch when it completes.)
-#define LAK_PDL_ENTRY()                                              \
-    do {                                                             \
-        asm volatile("griddepcontrol.wait;" ::: "memory");           \
-        asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); \
+#define LAK_PDL_WAIT() asm volatile("griddepcontrol.wait;" ::: "memory")
+#define LAK_PDL_TRIGGER() asm volatile("griddepcontrol.launch_dependents;" ::: "memory")
+#define LAK_PDL_ENTRY()    \
+    do {                   \
+        LAK_PDL_WAIT();    \
+        LAK_PDL_TRIGGER(); \
     } while (0)
 
 // Host: whether launches ask for programmatic serialization (LAK_PDL, read once).
@@ -144,6 +146,20 @@ lak_status launch_gemv_row(lak_dtype dt, void *y, const void *A, const void *x, 
 lak_status launch_gemv_col(lak_dtype dt, void *y, const void *A, const void *x, int64_t m,
                            int64_t n, int64_t lda, const Launch &L, int splits, void *ws,
                            double alpha, double beta, cudaStream_t s);
+// Row-major product by sets of `rows` rows that start at the same offset modulo
+// 16 bytes (rows r, r + period, ...), one set and one of `splits` column ranges per
+// block; splits > 1 needs the workspace (counter area, then splits * m sums).
+struct RowsLaunch {
+    int block, rows, period, splits;
+    int64_t sets;
+};
+lak_status launch_gemv_rows(lak_dtype dt, void *y, const void *A, const void *x, int64_t m,
+                            int64_t n, int64_t lda, const RowsLaunch &L, void *ws, double alpha,
+                            double beta, cudaStream_t s);
+// Column-major product with very many rows: a thread per 16 bytes of rows.
+constexpr int kGemvTallBlock = 256;
+lak_status launch_gemv_tall(lak_dtype dt, void *y, const void *A, const void *x, int64_t m,
+                            int64_t n, int64_t lda, double alpha, double beta, cudaStream_t s);
 lak_status launch_spmv(lak_dtype dt, void *y, const int32_t *rp, const int32_t *ci,
                        const void *vals, const void *x, int64_t m, const Launch &L, int group,
                        cudaStream_t s);
@@ -354,6 +370,44 @@ __device__ __forceinline__ void store_pack(T *p, const Pack<T, V> &pk) {
             st_raw<32>(reinterpret_cast<char *>(p) + 32 * c,
                        reinterpret_cast<const char *>(&pk) + 32 * c);
     }
+}
+
+template <bool B> struct Flag { static constexpr bool value = B; };
+
+// The 16 bytes that start `sb` bytes (a multiple of the element size) into w[0..7].
+template <int ES> __device__ __forceinline__ void shift_words(uint32_t (&w)[8], uint32_t sb) {
+    if (sb & 8) {
+#pragma unroll
+        for (int i = 0; i < 6; ++i) w[i] = w[i + 2];
+    }
+    if constexpr (ES <= 4) {
+        if (sb & 4) {
+#pragma unroll
+            for (int i = 0; i < 5; ++i) w[i] = w[i + 1];
+        }
+    }
+    if constexpr (ES <= 2) {
+        if (sb & 2) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) w[i] = __funnelshift_r(w[i], w[i + 1], 16);
+        }
+    }
+}
+
+// 16 bytes of consecutive elements from any element address p, sb = p % 16: two
+// aligned loads around them, shifted in registers (one load when sb is 0).  Reads the
+// aligned 32 bytes from p - sb (16 when sb is 0), which must be readable.
+template <typename T, int P>
+__device__ __forceinline__ void load_window(Pack<T, 16 / (int)sizeof(T)> &pk, const T *p,
+                                            uint32_t sb) {
+    const char *q = reinterpret_cast<const char *>(p) - sb;
+    uint32_t w[8];
+    ld_raw<16, P>(w, q);
+    if (sb) {
+        ld_raw<16, P>(w + 4, q + 16);
+        shift_words<(int)sizeof(T)>(w, sb);
+    }
+    memcpy(&pk, w, 16);
 }
 
 // Cached (L1-allocating) read-only scalar load, for operands that many
