@@ -28,7 +28,7 @@ __all__ = ["vec_copy", "vec_axpy", "vec_axpby", "vec_axpy_norm2", "vec_axpy_norm
            "vec_dot_sparse_workspace", "vec_dot_compensated",
            "vec_dot_noalloc", "dense_gemv",
            "dense_gemv_workspace", "csr_spmv", "dense_outer", "csr_sampled_outer",
-           "csr_transpose", "vec_gather", "vec_scale_dev", "resolve_cfg", "set_default_cfg",
+           "csr_transpose", "csr_transpose_vals", "vec_gather", "vec_scale_dev", "resolve_cfg", "set_default_cfg",
            "size_bucket", "SIZE_BUCKETS", "Cfg", "set_batch_default_cfg", "probe_fma_f64",
            "LakError", "storage_of", "library_path"]
 
@@ -557,21 +557,72 @@ def csr_sampled_outer(row_ptr: torch.Tensor, col_idx: torch.Tensor, dy: torch.Te
     return out
 
 
-def csr_transpose(row_ptr: torch.Tensor, col_idx: torch.Tensor, n_cols: int, stream=None):
-    """(col_ptr, row_idx, perm) of the CSC form (int32 device tensors)."""
-    m = row_ptr.numel() - 1
+def _stream_scratch(nbytes: int, device: torch.device, stream) -> torch.Tensor:
+    """Scratch for one call on `stream` (None: the current one), owned by that stream,
+    so that the allocator hands it on only behind the call's kernels."""
+    if stream is None:
+        return torch.empty(max(nbytes, 256), dtype=torch.uint8, device=device)
+    if not isinstance(stream, torch.cuda.Stream):
+        stream = torch.cuda.ExternalStream(int(stream), device=device)
+    with torch.cuda.stream(stream):
+        return torch.empty(max(nbytes, 256), dtype=torch.uint8, device=device)
+
+
+def _csc_arrays(row_ptr, col_idx, n_cols):
+    _vec_arg(row_ptr, "row_ptr")
     nnz = col_idx.numel()
+    if nnz:
+        _vec_arg(col_idx, "col_idx")
     dev = row_ptr.device
-    col_ptr = torch.empty(n_cols + 1, dtype=torch.int32, device=dev)
-    row_idx = torch.empty(max(nnz, 1), dtype=torch.int32, device=dev)
-    perm = torch.empty(max(nnz, 1), dtype=torch.int32, device=dev)
-    ws_bytes = int(_lib.csr_transpose_workspace(int(n_cols)))
-    ws = torch.empty(max(ws_bytes, 256), dtype=torch.uint8, device=dev)
+    return (torch.empty(n_cols + 1, dtype=torch.int32, device=dev),
+            torch.empty(max(nnz, 1), dtype=torch.int32, device=dev),
+            torch.empty(max(nnz, 1), dtype=torch.int32, device=dev))
+
+
+def csr_transpose(row_ptr: torch.Tensor, col_idx: torch.Tensor, n_cols: int, stream=None):
+    """(col_ptr, row_idx, perm) of the CSC form (int32 device tensors).  Takes 16 bytes
+    of scratch per entry for the call, or the least the library needs where the device
+    has no room for that."""
+    n_cols, nnz = int(n_cols), col_idx.numel()
+    col_ptr, row_idx, perm = _csc_arrays(row_ptr, col_idx, n_cols)
+    try:
+        ws = _stream_scratch(int(_lib.csr_transpose_vals_workspace(n_cols, nnz, DTYPES["f32"])),
+                             row_ptr.device, stream)
+    except torch.cuda.OutOfMemoryError:
+        ws = _stream_scratch(int(_lib.csr_transpose_workspace(n_cols)), row_ptr.device, stream)
     st = _lib.csr_transpose(col_ptr.data_ptr(), row_idx.data_ptr(), perm.data_ptr(),
-                            _vec_arg(row_ptr, "row_ptr"), _vec_arg(col_idx, "col_idx") if nnz else None,
-                            m, int(n_cols), nnz, ws.data_ptr(), ws.numel(), _stream(stream))
+                            row_ptr.data_ptr(), col_idx.data_ptr() if nnz else None,
+                            row_ptr.numel() - 1, n_cols, nnz, ws.data_ptr(), ws.numel(),
+                            _stream(stream))
     _native.check("csr_transpose", st)
     return col_ptr, row_idx[:nnz], perm[:nnz]
+
+
+def csr_transpose_vals(row_ptr: torch.Tensor, col_idx: torch.Tensor, vals: torch.Tensor,
+                       n_cols: int, stream=None):
+    """(col_ptr, row_idx, perm, vals_t) of the CSC form with the values carried along
+    (vals_t = vals[perm]), in one pass over the entries."""
+    s = storage_of(vals)
+    n_cols, nnz = int(n_cols), col_idx.numel()
+    if vals.numel() != nnz:
+        raise ValueError("col_idx and vals must have nnz entries each")
+    if nnz:
+        _vec_arg(vals, "vals")
+    col_ptr, row_idx, perm = _csc_arrays(row_ptr, col_idx, n_cols)
+    vals_t = torch.empty(max(nnz, 1), dtype=vals.dtype, device=vals.device)
+    try:
+        ws = _stream_scratch(int(_lib.csr_transpose_vals_workspace(n_cols, nnz, DTYPES[s])),
+                             row_ptr.device, stream)
+    except torch.cuda.OutOfMemoryError:
+        col_ptr, row_idx, perm = csr_transpose(row_ptr, col_idx, n_cols, stream=stream)
+        return col_ptr, row_idx, perm, vec_gather(vals, perm, out=vals_t[:nnz], stream=stream)
+    st = _lib.csr_transpose_vals(col_ptr.data_ptr(), row_idx.data_ptr(), perm.data_ptr(),
+                                 vals_t.data_ptr(), row_ptr.data_ptr(),
+                                 col_idx.data_ptr() if nnz else None,
+                                 vals.data_ptr() if nnz else None, row_ptr.numel() - 1, n_cols,
+                                 nnz, DTYPES[s], ws.data_ptr(), ws.numel(), _stream(stream))
+    _native.check("csr_transpose_vals", st)
+    return col_ptr, row_idx[:nnz], perm[:nnz], vals_t[:nnz]
 
 
 def vec_gather(src: torch.Tensor, idx: torch.Tensor, out: Optional[torch.Tensor] = None,

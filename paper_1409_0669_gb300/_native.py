@@ -30,7 +30,8 @@ EXPORTS = ("lak_last_error", "lak_abi_version", "lak_set_default_cfg", "lak_reso
            "vec_dot_noalloc",
            "dense_gemv_workspace", "dense_gemv", "dense_gemv_axpby", "dense_gemv_trans",
            "csr_spmv", "dense_outer", "csr_sampled_outer",
-           "csr_transpose_workspace", "csr_transpose", "vec_gather", "vec_scale_dev",
+           "csr_transpose_workspace", "csr_transpose", "csr_transpose_vals_workspace",
+           "csr_transpose_vals", "vec_gather", "vec_scale_dev",
            "csr_to_sell_count", "csr_to_sell_fill", "sell_pack_values", "sell_spmv",
            "lak_batch_plan", "lak_batch_run", "lak_set_batch_default_cfg", "lak_probe_fma_f64",
            "lak_probe_fma_f64_flops")
@@ -121,6 +122,8 @@ _SIGNATURES = {
     "csr_sampled_outer": (_I32, [_P, _P, _P, _P, _P, _I64, _I64, _I32, _P]),
     "csr_transpose_workspace": (_SZ, [_I64]),
     "csr_transpose": (_I32, [_P, _P, _P, _P, _P, _I64, _I64, _I64, _P, _SZ, _P]),
+    "csr_transpose_vals_workspace": (_SZ, [_I64, _I64, _I32]),
+    "csr_transpose_vals": (_I32, [_P, _P, _P, _P, _P, _P, _P, _I64, _I64, _I64, _I32, _P, _SZ, _P]),
     "vec_gather": (_I32, [_P, _P, _P, _I64, _I32, _P]),
     "vec_scale_dev": (_I32, [_P, _P, _P, _I64, _I32, _P]),
     "csr_to_sell_count": (_I32, [_P, _I64, _I32, _P, _P, _P, _P]),

@@ -7,6 +7,7 @@
 //   vec_scale_dev      out = alpha * v, alpha read from device memory
 //                      (gradient of <x, y>: dx = ds * y without a host sync)
 #include "lak_internal.cuh"
+#include "transpose.cuh"
 
 namespace lak {
 namespace {
@@ -256,6 +257,31 @@ bool valid_dt(lak_dtype dt) { return dt == LAK_F32 || dt == LAK_F64 || dt == LAK
 }  // namespace
 }  // namespace lak
 
+namespace lak {
+
+int64_t scan_scratch_ints(int64_t len) {
+    const int64_t tiles = (len + kScanTile - 1) / kScanTile;
+    const int64_t tiles2 = (tiles + kScanTile - 1) / kScanTile;
+    return (tiles + 63) / 64 * 64 + (tiles2 + 63) / 64 * 64 + 64;
+}
+
+void launch_scan_i32(int32_t *v, int64_t len, int32_t *sums, cudaStream_t s) {
+    const int64_t tiles = (len + kScanTile - 1) / kScanTile;
+    const int64_t tiles2 = (tiles + kScanTile - 1) / kScanTile;
+    int32_t *sums2 = sums + (tiles + 63) / 64 * 64;
+    launch_k(scan_tiles_kernel, (unsigned)tiles, kScanBlock, 0, s, v, len, sums);
+    if (tiles > 1) {
+        launch_k(scan_tiles_kernel, (unsigned)tiles2, kScanBlock, 0, s, sums, tiles, sums2);
+        if (tiles2 > 1) {
+            launch_k(scan_tiles_kernel, 1, kScanBlock, 0, s, sums2, tiles2, sums2 + tiles2);
+            launch_k(add_tile_offsets_kernel, (unsigned)tiles2, 256, 0, s, sums, tiles, sums2);
+        }
+        launch_k(add_tile_offsets_kernel, (unsigned)tiles, 256, 0, s, v, len, sums);
+    }
+}
+
+}  // namespace lak
+
 using namespace lak;
 
 extern "C" {
@@ -316,11 +342,17 @@ LAK_API lak_status csr_sampled_outer(void *dvals, const int32_t *row_ptr, const 
 
 LAK_API size_t csr_transpose_workspace(int64_t n) {
     if (n < 0) return 0;
-    const int64_t tiles = (n + kScanTile - 1) / kScanTile;
-    // cursor (n) + tile sums + sums of tile sums, all int32, 256-byte sections
+    // cursor (n) and the scan's sums, 256-byte sections
     auto up = [](size_t b) { return (b + 255) / 256 * 256; };
-    const int64_t tiles2 = (tiles + kScanTile - 1) / kScanTile;
-    return up((size_t)n * 4) + up((size_t)tiles * 4) + up((size_t)tiles2 * 4) + 256;
+    return up((size_t)n * 4) + up((size_t)scan_scratch_ints(n) * 4) + 256;
+}
+
+LAK_API size_t csr_transpose_vals_workspace(int64_t n, int64_t nnz, lak_dtype dtype) {
+    if (n < 0 || nnz < 0 || nnz > 0x7fffffffLL || n > 0x7fffffffLL || !valid_dt(dtype)) return 0;
+    const size_t least = csr_transpose_workspace(n);
+    if (n == 0 || nnz == 0) return least;
+    const size_t w = transpose_workspace(n, nnz, esize(dtype));
+    return w > least ? w : least;
 }
 
 LAK_API lak_status csr_transpose(int32_t *col_ptr, int32_t *row_idx, int32_t *perm,
@@ -331,9 +363,12 @@ LAK_API lak_status csr_transpose(int32_t *col_ptr, int32_t *row_idx, int32_t *pe
         return fail(LAK_EINVAL, "csr_transpose: bad sizes");
     if (!col_ptr) return fail(LAK_EINVAL, "csr_transpose: NULL col_ptr");
     cudaStream_t s = (cudaStream_t)stream;
-    cudaError_t e = cudaMemsetAsync(col_ptr, 0, (size_t)(n + 1) * 4, s);
-    if (e != cudaSuccess) return fail(LAK_ECUDA, "csr_transpose: memset: %s", cudaGetErrorString(e));
-    if (n == 0 || nnz == 0) return LAK_OK;
+    if (n == 0 || nnz == 0) {
+        const cudaError_t e = cudaMemsetAsync(col_ptr, 0, (size_t)(n + 1) * 4, s);
+        if (e != cudaSuccess)
+            return fail(LAK_ECUDA, "csr_transpose: memset: %s", cudaGetErrorString(e));
+        return LAK_OK;
+    }
     if (!row_ptr || !col_idx || !row_idx || !perm)
         return fail(LAK_EINVAL, "csr_transpose: NULL pointer");
     const size_t need = csr_transpose_workspace(n);
@@ -342,33 +377,64 @@ LAK_API lak_status csr_transpose(int32_t *col_ptr, int32_t *row_idx, int32_t *pe
                     workspace ? ws_bytes : (size_t)0);
     if ((uintptr_t)workspace % 256)
         return fail(LAK_EWORKSPACE, "csr_transpose: workspace not 256-byte aligned");
+    // with room for the entries' records: the stable partition (k_transpose.cu)
+    if (n <= kTransposeMaxCols && m > 0 && ws_bytes >= csr_transpose_vals_workspace(n, nnz, LAK_F32))
+        return launch_transpose(col_ptr, row_idx, perm, nullptr, row_ptr, col_idx, nullptr, m, n,
+                                nnz, 4, workspace, s);
+    cudaError_t e = cudaMemsetAsync(col_ptr, 0, (size_t)(n + 1) * 4, s);
+    if (e != cudaSuccess) return fail(LAK_ECUDA, "csr_transpose: memset: %s", cudaGetErrorString(e));
     auto up = [](size_t b) { return (b + 255) / 256 * 256; };
-    const int64_t tiles = (n + kScanTile - 1) / kScanTile;
-    const int64_t tiles2 = (tiles + kScanTile - 1) / kScanTile;
     char *w = static_cast<char *>(workspace);
     int32_t *cursor = reinterpret_cast<int32_t *>(w);
     int32_t *sums = reinterpret_cast<int32_t *>(w + up((size_t)n * 4));
-    int32_t *sums2 = reinterpret_cast<int32_t *>(w + up((size_t)n * 4) + up((size_t)tiles * 4));
-    if (tiles2 > kScanTile)
+    if (n > kScanTile * kScanTile * kScanTile)
         return fail(LAK_EINVAL, "csr_transpose: n = %lld is beyond the two-level scan",
                     (long long)n);
     const int block = 256;
     // counts land in col_ptr[1..n]
     launch_k(count_cols_kernel, grid_for(nnz, block), block, 0, s, col_ptr + 1, col_idx, nnz);
     // inclusive scan of col_ptr[1..n] -> col_ptr[j+1] = entries in columns <= j
-    launch_k(scan_tiles_kernel, (unsigned)tiles, kScanBlock, 0, s, col_ptr + 1, n, sums);
-    if (tiles > 1) {
-        launch_k(scan_tiles_kernel, (unsigned)tiles2, kScanBlock, 0, s, sums, tiles, sums2);
-        if (tiles2 > 1) {
-            launch_k(scan_tiles_kernel, 1, kScanBlock, 0, s, sums2, tiles2, sums2 + tiles2);
-            launch_k(add_tile_offsets_kernel, (unsigned)tiles2, 256, 0, s, sums, tiles, sums2);
-        }
-        launch_k(add_tile_offsets_kernel, (unsigned)tiles, 256, 0, s, col_ptr + 1, n, sums);
-    }
+    launch_scan_i32(col_ptr + 1, n, sums, s);
     launch_k(copy_i32_kernel, grid_for(n, block), block, 0, s, cursor, col_ptr, n);
     launch_k(scatter_kernel, grid_for(m, block), block, 0, s, row_idx, perm, cursor, row_ptr, col_idx, m);
     launch_k(sort_columns_kernel, grid_for(n, block), block, 0, s, row_idx, perm, col_ptr, n);
     return check_launch("csr_transpose");
+}
+
+LAK_API lak_status csr_transpose_vals(int32_t *col_ptr, int32_t *row_idx, int32_t *perm,
+                                      void *vals_t, const int32_t *row_ptr,
+                                      const int32_t *col_idx, const void *vals, int64_t m,
+                                      int64_t n, int64_t nnz, lak_dtype dtype, void *workspace,
+                                      size_t ws_bytes, void *stream) {
+    const char *who = "csr_transpose_vals";
+    if (!valid_dt(dtype)) return fail(LAK_EDTYPE, "%s: unknown dtype %d", who, (int)dtype);
+    if (m < 0 || n < 0 || nnz < 0 || nnz > 0x7fffffffLL || n > 0x7fffffffLL)
+        return fail(LAK_EINVAL, "%s: bad sizes", who);
+    if (!col_ptr) return fail(LAK_EINVAL, "%s: NULL col_ptr", who);
+    cudaStream_t s = (cudaStream_t)stream;
+    if (m == 0 || n == 0 || nnz == 0) {
+        const cudaError_t e = cudaMemsetAsync(col_ptr, 0, (size_t)(n + 1) * 4, s);
+        if (e != cudaSuccess) return fail(LAK_ECUDA, "%s: memset: %s", who, cudaGetErrorString(e));
+        return LAK_OK;
+    }
+    const int es = esize(dtype);
+    if (!row_ptr || !col_idx || !row_idx || !perm || !vals || !vals_t)
+        return fail(LAK_EINVAL, "%s: NULL pointer", who);
+    if ((uintptr_t)vals % es || (uintptr_t)vals_t % es)
+        return fail(LAK_EINVAL, "%s: pointers not aligned to the element size", who);
+    const size_t need = csr_transpose_vals_workspace(n, nnz, dtype);
+    if (!workspace || ws_bytes < need)
+        return fail(LAK_EWORKSPACE, "%s: workspace of %zu bytes needed, %zu given", who, need,
+                    workspace ? ws_bytes : (size_t)0);
+    if ((uintptr_t)workspace % 256)
+        return fail(LAK_EWORKSPACE, "%s: workspace not 256-byte aligned", who);
+    if (n > kTransposeMaxCols) {
+        const lak_status st = csr_transpose(col_ptr, row_idx, perm, row_ptr, col_idx, m, n, nnz,
+                                            workspace, ws_bytes, stream);
+        return st != LAK_OK ? st : vec_gather(vals_t, vals, perm, nnz, dtype, stream);
+    }
+    return launch_transpose(col_ptr, row_idx, perm, vals_t, row_ptr, col_idx, vals, m, n, nnz, es,
+                            workspace, s);
 }
 
 LAK_API lak_status vec_gather(void *dst, const void *src, const int32_t *idx, int64_t n,

@@ -1,0 +1,678 @@
+// CSC form of a CSR pattern by stable partitioning (csr_transpose and
+// csr_transpose_vals of include/lak.h).
+//
+// What bounds it: moving nnz entries into column order.  Serving each entry's place
+// from an atomic cursor scatters 4-byte stores over the whole output (one DRAM sector
+// each) and leaves every column to be sorted afterwards; 32 M entries of a power-law
+// matrix took 3.6 ms that way, and bringing the values into that order by a gather
+// another 0.57 ms.  Here the entries move twice, as 16-byte records (column, row, CSR
+// position, value):
+//
+//   1. partition by column block (2^s columns, about 4600 entries), a tile of
+//      consecutive entries per thread block: counts per tile and column block, a scan
+//      over the tiles of each column block, then every tile orders its records by
+//      column block in shared memory and stores them as runs behind those of the
+//      tiles before it.  Tiles run in order, so the stores of the tiles in flight lie
+//      side by side and L2 completes the sectors.
+//   2. one thread block per column block orders its records by column on chip the same
+//      way (the scan also gives col_ptr) and writes the outputs consecutively.
+//
+// Ranks are stable: a warp ranks its 32 entries against counters of its own, and the
+// warps' counters are scanned in warp order.  So every column keeps its entries in CSR
+// order: the result of a stable counting sort, independent of scheduling, with no
+// global atomics.  More than 1024 column blocks take the partition twice (low half of
+// the block number, then high half).  Blocks are half an SM, so that one's loads and
+// stores run under the other's ranking.
+//
+// Measured (32 M entries, 2 M columns, FP32 values carried along): 1.03 ms against
+// 4.1 ms for the atomic scatter, the columns' sort and the gather (FP64 values 1.52 ms);
+// three passes of 0.9-1.0 GB each, 0.45 ms at the copy rate.  Blocks of a whole SM
+// (1024 threads, tiles of 8192) took 1.42 ms, ten-bit digits in one pass with column
+// blocks of 32 K entries gathered through L2 1.30 ms, per-warp fronts without the
+// exchange 2.1 ms.
+#include "lak_internal.cuh"
+#include "transpose.cuh"
+
+namespace lak {
+namespace {
+
+constexpr int kDigitBits = 10;
+constexpr int kMaxBlocks = 1 << kDigitBits;     // digits of a partition pass, at most
+constexpr int kMaxColBits = 10;         // columns per block: at most 2^10
+constexpr int kTileWarps = 16;          // warps per block of the partition kernels
+constexpr int kTileThreads = 32 * kTileWarps;
+constexpr int kItems = 8;               // entries a lane takes of a tile
+constexpr int kTile = kTileThreads * kItems;
+constexpr int kSegTiles = 64;           // tiles per segment of the scan over tiles
+constexpr int kOrderWarps = 16;         // warps per block of the ordering kernel
+constexpr int kBigWarps = 8;            // warps that work on a column block beyond that
+
+struct __align__(16) Rec {
+    int32_t col, row, k;
+    uint32_t v;                         // 16- or 32-bit value (64-bit ones go beside)
+};
+
+// Stable rank of this lane's entry among the entries of digit d that the warp has seen:
+// the warp's counter plus the number of lower lanes with that digit; the counter
+// advances by the lanes'.  The lanes with equal digits are found with one ballot per
+// bit of the digit (match.any measured about 100 cycles of an SM per warp here).
+// All 32 lanes call it.
+template <typename C>
+__device__ __forceinline__ int32_t warp_rank(C *counter, int32_t d, int bits, bool valid,
+                                             int lane) {
+    unsigned same = __ballot_sync(0xffffffffu, valid);
+    auto split = [&](int from, int to) {
+#pragma unroll
+        for (int i = from; i < to; ++i) {
+            const bool one = d & (1 << i);
+            const unsigned ones = __ballot_sync(0xffffffffu, one);
+            same &= one ? ones : ~ones;
+        }
+    };
+    split(0, 4);
+    if (bits > 4) split(4, 6);          // warp-uniform
+    if (bits > 6) split(6, 9);
+    if (bits > 9) split(9, 11);
+    const int leader = __ffs((int)same) - 1;        // of an invalid lane: any
+    int32_t base = 0;
+    if (valid && lane == leader) {
+        base = counter[d];
+        counter[d] = (C)(base + __popc(same));
+    }
+    base = __shfl_sync(0xffffffffu, base, leader < 0 ? 0 : leader);
+    __syncwarp();                       // the next entry's leader may be another lane
+    return base + __popc(same & ((1u << lane) - 1u));
+}
+
+// first[c] = row of entry c * kChunk, by the rows (every non-empty row holds the chunk
+// starts that lie in it)
+constexpr int kChunk = 128;
+__global__ void __launch_bounds__(256)
+chunk_rows_kernel(int32_t *__restrict__ first, const int32_t *__restrict__ rp, int64_t m) {
+    LAK_PDL_ENTRY();
+    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < m;
+         r += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t a = __ldg(rp + r), b = __ldg(rp + r + 1);
+        for (int64_t c = (a + kChunk - 1) / kChunk; c * kChunk < b; ++c) first[c] = (int32_t)r;
+    }
+}
+
+// cells[tile * nb + b] = entries of the tile in column block b
+__global__ void __launch_bounds__(kTileThreads)
+part_count_kernel(int32_t *__restrict__ cells, const int32_t *__restrict__ keys, int key_stride,
+                  int64_t nnz, int shift, int mask, int nb) {
+    LAK_PDL_ENTRY();
+    extern __shared__ int32_t part_smem[];
+    for (int b = threadIdx.x; b < nb; b += blockDim.x) part_smem[b] = 0;
+    __syncthreads();
+    const int64_t k0 = (int64_t)blockIdx.x * kTile + threadIdx.x;
+    int32_t c[kItems];
+#pragma unroll
+    for (int i = 0; i < kItems; ++i) {
+        const int64_t k = k0 + i * kTileThreads;
+        if (k < nnz) c[i] = __ldg(keys + k * key_stride);
+    }
+#pragma unroll
+    for (int i = 0; i < kItems; ++i)
+        if (k0 + i * kTileThreads < nnz) atomicAdd(part_smem + ((c[i] >> shift) & mask), 1);
+    __syncthreads();
+    int32_t *out = cells + (int64_t)blockIdx.x * nb;
+    for (int b = threadIdx.x; b < nb; b += blockDim.x) out[b] = part_smem[b];
+}
+
+// Scan over the tiles of each column block, in three steps: sums per segment of tiles,
+// starts of every (column block, segment), then of every (column block, tile).
+__global__ void __launch_bounds__(256)
+seg_sum_kernel(int32_t *__restrict__ segs, const int32_t *__restrict__ cells, int64_t tiles,
+               int nb) {
+    LAK_PDL_ENTRY();
+    const int b = blockIdx.x * 256 + threadIdx.x;
+    if (b >= nb) return;
+    const int64_t t0 = (int64_t)blockIdx.y * kSegTiles;
+    const int64_t t1 = t0 + kSegTiles < tiles ? t0 + kSegTiles : tiles;
+    int32_t s = 0;
+#pragma unroll 8
+    for (int64_t t = t0; t < t1; ++t) s += __ldg(cells + t * nb + b);
+    segs[(int64_t)blockIdx.y * nb + b] = s;
+}
+
+// v[i * ld], i = i0 .. i1 - 1, replaced by start plus the sum of those before it; 16 at a
+// time, so that their loads are in flight together
+__device__ __forceinline__ void running(int32_t *v, int64_t ld, int64_t i0, int64_t i1,
+                                        int32_t start) {
+    for (int64_t i = i0; i < i1; i += 16) {
+        int32_t c[16];
+#pragma unroll
+        for (int u = 0; u < 16; ++u) c[u] = i + u < i1 ? v[(i + u) * ld] : 0;
+#pragma unroll
+        for (int u = 0; u < 16; ++u)
+            if (i + u < i1) {
+                v[(i + u) * ld] = start;
+                start += c[u];
+            }
+    }
+}
+
+// segs[seg * nb + b] -> start of that segment's entries; starts[b] of the column block
+__global__ void __launch_bounds__(1024)
+seg_scan_kernel(int32_t *__restrict__ segs, int32_t *__restrict__ starts, int64_t nseg, int nb) {
+    LAK_PDL_ENTRY();
+    __shared__ int32_t wtot[32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int PER = (kMaxBlocks + 1023) / 1024;     // column blocks of a thread
+    int32_t tot[PER], sum = 0;
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        const int b = tid * PER + i;
+        tot[i] = 0;
+        if (b < nb) {
+#pragma unroll 8
+            for (int64_t g = 0; g < nseg; ++g) tot[i] += segs[g * nb + b];
+        }
+        sum += tot[i];
+    }
+    int32_t incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int32_t up = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += up;
+    }
+    if (lane == 31) wtot[warp] = incl;
+    __syncthreads();
+    int32_t at = incl - sum;
+    for (int w = 0; w < warp; ++w) at += wtot[w];
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        const int b = tid * PER + i;
+        if (b < nb) {
+            starts[b] = at;
+            running(segs + b, nb, 0, nseg, at);
+        }
+        at += tot[i];
+    }
+}
+
+__global__ void __launch_bounds__(256)
+seg_apply_kernel(int32_t *__restrict__ cells, const int32_t *__restrict__ segs, int64_t tiles,
+                 int nb) {
+    LAK_PDL_ENTRY();
+    const int b = blockIdx.x * 256 + threadIdx.x;
+    if (b >= nb) return;
+    const int64_t t0 = (int64_t)blockIdx.y * kSegTiles;
+    const int64_t t1 = t0 + kSegTiles < tiles ? t0 + kSegTiles : tiles;
+    running(cells + b, nb, t0, t1, segs[(int64_t)blockIdx.y * nb + b]);
+}
+
+template <typename E> constexpr size_t move_smem(int nb) {
+    return (size_t)kTile * (16 + (sizeof(E) == 8 ? 8 : 0)) + (size_t)nb * 4 +
+           (size_t)kTileWarps * nb * 2;
+}
+
+// Orders a tile's records by column block in shared memory and stores them as runs.
+// From the CSR arrays, or (CSR false) from the records of an earlier pass.
+// E: the values' type (uint16_t, uint32_t, uint64_t; vals may be null).
+template <typename E, bool CSR>
+__global__ void __launch_bounds__(kTileThreads, 2)
+part_move_kernel(Rec *__restrict__ out, uint64_t *__restrict__ out64,
+                 const int32_t *__restrict__ rp, const int32_t *__restrict__ ci,
+                 const E *__restrict__ vals, const Rec *__restrict__ in,
+                 const uint64_t *__restrict__ in64, const int32_t *__restrict__ cells,
+                 const int32_t *__restrict__ first, int64_t m, int64_t nnz, int shift, int mask,
+                 int nb, int bits) {
+    LAK_PDL_ENTRY();
+    constexpr bool WIDE = sizeof(E) == 8;
+    constexpr int ITEMS = kItems, TILE = kTile;
+    extern __shared__ __align__(16) unsigned char move_raw[];
+    Rec *stage = reinterpret_cast<Rec *>(move_raw);
+    uint64_t *stage64 = reinterpret_cast<uint64_t *>(move_raw + (size_t)TILE * 16);
+    int32_t *delta = reinterpret_cast<int32_t *>(move_raw + (size_t)TILE * (WIDE ? 24 : 16));
+    uint16_t *count = reinterpret_cast<uint16_t *>(delta + nb);        // [warp][nb]
+    __shared__ int32_t wtot[kTileWarps];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t t0 = (int64_t)blockIdx.x * TILE;
+    const int64_t t1 = t0 + TILE < nnz ? t0 + TILE : nnz;
+    for (int i = tid; i < kTileWarps * nb / 2; i += kTileThreads)
+        reinterpret_cast<uint32_t *>(count)[i] = 0;
+    __syncthreads();
+
+    // 1. ranks within the warp; a lane keeps (digit, rank) and the row of its entries
+    const int64_t w0 = t0 + (int64_t)warp * 32 * ITEMS;
+    uint16_t *mine = count + warp * nb;
+    uint32_t where[ITEMS];
+    int32_t row[ITEMS];
+    Rec rec[ITEMS];
+    uint64_t wide[ITEMS];
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) {
+        const int64_t k = w0 + 32 * i + lane;
+        rec[i].col = 0;
+        rec[i].v = 0;
+        wide[i] = 0;
+        if (k < t1) {
+            if constexpr (CSR) {
+                rec[i].col = __ldg(ci + k);
+                if (vals) {
+                    if constexpr (WIDE) wide[i] = __ldg((const unsigned long long *)vals + k);
+                    else rec[i].v = __ldg(vals + k);
+                }
+            } else {
+                ld_raw<16, STREAM>(&rec[i], in + k);
+                if (WIDE && in64) wide[i] = in64[k];
+            }
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) {
+        const int64_t k = w0 + 32 * i + lane;
+        const int32_t d = (rec[i].col >> shift) & mask;
+        const int32_t r = warp_rank(mine, d, bits, k < t1, lane);
+        where[i] = (uint32_t)d << 16 | (uint32_t)r;
+    }
+    if constexpr (CSR) {
+        // every non-empty row that begins inside the warp's entries leaves its number at
+        // its first entry; an entry's row is the last such number up to it
+        int32_t *marks = reinterpret_cast<int32_t *>(stage) + warp * 32 * ITEMS;
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) marks[32 * i + lane] = 0;
+        __syncwarp();
+        int32_t run = 0;
+        if (w0 < t1) {
+            run = __ldg(first + w0 / kChunk);
+            const int64_t w1 = w0 + 32 * ITEMS < t1 ? w0 + 32 * ITEMS : t1;
+            for (int64_t rb = run + 1; rb < m; rb += 32) {
+                const int64_t r = rb + lane;
+                const int64_t a = r < m ? (int64_t)__ldg(rp + r) : w1;
+                const int64_t b = r < m ? (int64_t)__ldg(rp + r + 1) : w1;
+                if (a < w1 && b > a) marks[a - w0] = (int32_t)r;
+                if (__any_sync(0xffffffffu, a >= w1)) break;
+            }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) {
+            const int32_t v = marks[32 * i + lane];
+            const unsigned begun = __ballot_sync(0xffffffffu, v) & (0xffffffffu >> (31 - lane));
+            const int32_t r = __shfl_sync(0xffffffffu, v, begun ? 31 - __clz((int)begun) : 0);
+            row[i] = begun ? r : run;
+            run = __shfl_sync(0xffffffffu, row[i], 31);
+        }
+    }
+    __syncthreads();
+
+    // 2. counts -> places in the tile (by column block, then warp); delta: from a place
+    // in the tile to the place in the output
+    {
+        const int per = (nb + kTileThreads - 1) / kTileThreads;
+        int32_t sum = 0;
+        for (int b = tid * per; b < (tid + 1) * per && b < nb; ++b) {
+#pragma unroll
+            for (int w = 0; w < kTileWarps; ++w) sum += count[w * nb + b];
+        }
+        int32_t incl = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t up = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += up;
+        }
+        if (lane == 31) wtot[warp] = incl;
+        __syncthreads();
+        int32_t at = incl - sum;
+        for (int w = 0; w < warp; ++w) at += wtot[w];
+        const int32_t *cell = cells + (int64_t)blockIdx.x * nb;
+        for (int b = tid * per; b < (tid + 1) * per && b < nb; ++b) {
+            delta[b] = __ldg(cell + b) - at;
+#pragma unroll
+            for (int w = 0; w < kTileWarps; w += 4) {
+                int32_t c[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) c[u] = count[(w + u) * nb + b];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    count[(w + u) * nb + b] = (uint16_t)at;
+                    at += c[u];
+                }
+            }
+        }
+    }
+    __syncthreads();
+
+    // 3. records to their places in the tile
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) {
+        const int64_t k = w0 + 32 * i + lane;
+        if (k >= t1) break;
+        if constexpr (CSR) {
+            rec[i].row = row[i];
+            rec[i].k = (int32_t)k;
+        }
+        const int place = (int)mine[where[i] >> 16] + (int)(where[i] & 0xffffu);
+        stage[place] = rec[i];
+        if (WIDE) stage64[place] = wide[i];
+    }
+    __syncthreads();
+
+    // 4. runs to the output
+    const int len = (int)(t1 - t0);
+    for (int q = tid; q < len; q += kTileThreads) {
+        const Rec rec = stage[q];
+        const int32_t pos = delta[(rec.col >> shift) & mask] + q;
+        st_raw<16>(out + pos, &rec);
+        if (WIDE && out64) out64[pos] = stage64[q];
+    }
+}
+
+// bounds[b] = first record with a column of block b or later (records in block order)
+__global__ void __launch_bounds__(128)
+bounds_kernel(int32_t *__restrict__ bounds, const Rec *__restrict__ recs, int64_t nnz,
+              int64_t blocks, int s) {
+    LAK_PDL_ENTRY();
+    const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (b >= blocks) return;
+    const int64_t c = b << s;
+    int64_t lo = 0, hi = nnz;
+    while (lo < hi) {
+        const int64_t mid = (lo + hi) >> 1;
+        if (__ldg(&recs[mid].col) < c) lo = mid + 1; else hi = mid;
+    }
+    bounds[b] = (int32_t)lo;
+}
+
+// Records of a column block that are ordered on chip: 12 bytes each (16 with 64-bit
+// values) beside the counters.
+template <typename E> constexpr int kOrderItems = sizeof(E) == 8 ? 10 : 12;
+template <typename E> constexpr int kOrderCap = 32 * kOrderWarps * kOrderItems<E>;
+
+template <typename E> constexpr size_t order_smem(int s) {
+    return (size_t)kOrderWarps * (1 << s) * 2 + 16 + (size_t)kOrderCap<E> * (8 + (sizeof(E) == 8 ? 8 : 4));
+}
+
+// One block per column block: orders its records by column and writes the CSC arrays.
+// bounds: first record of every column block.
+// The usual column block fits on chip: its records are read, ranked, placed in shared
+// memory and written out consecutively.  A larger one (hub columns) is counted and
+// ranked in place, its entries stored one by one.
+template <typename E>
+__global__ void __launch_bounds__(32 * kOrderWarps, 2)
+order_kernel(int32_t *__restrict__ col_ptr, int32_t *__restrict__ row_idx,
+             int32_t *__restrict__ perm, E *__restrict__ vals_t, const Rec *__restrict__ recs,
+             const uint64_t *__restrict__ recs64, const int32_t *__restrict__ bounds, int64_t n,
+             int64_t nnz, int s) {
+    LAK_PDL_ENTRY();
+    constexpr bool WIDE = sizeof(E) == 8;
+    constexpr int ITEMS = kOrderItems<E>, CAP = kOrderCap<E>;
+    extern __shared__ __align__(16) unsigned char order_raw[];
+    __shared__ int32_t wtot[kOrderWarps];
+    __shared__ int64_t range[2];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int nc = 1 << s;
+    const int64_t c0 = (int64_t)blockIdx.x << s;
+    if (tid < 2) range[tid] = blockIdx.x + tid == gridDim.x ? nnz : bounds[blockIdx.x + tid];
+    // counters per warp and column: 16 bits for the records on chip, 32 bits and half
+    // the warps for more
+    uint16_t *half = reinterpret_cast<uint16_t *>(order_raw);
+    int32_t *full = reinterpret_cast<int32_t *>(order_raw);
+    for (int i = tid; i < kOrderWarps * nc / 2; i += 32 * kOrderWarps) full[i] = 0;
+    __syncthreads();
+    const int64_t b0 = range[0];
+    const int64_t len = range[1] - b0;
+    const bool small = len <= CAP;
+    const int nw = small ? kOrderWarps : kBigWarps;
+    const int64_t per = (len + nw * 32 - 1) / (nw * 32) * 32;
+    const int64_t e0 = warp < nw ? warp * per : len;
+    const int64_t e1 = e0 + per < len ? e0 + per : len;
+    uint16_t *mine16 = half + warp * nc;
+    int32_t *mine32 = full + warp * nc;
+    uint32_t where[ITEMS];
+    if (small) {
+        int32_t c[ITEMS];
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) {
+            const int64_t k = e0 + 32 * i + lane;
+            c[i] = k < e1 ? (int32_t)(__ldg(&recs[b0 + k].col) - c0) : 0;
+        }
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) {
+            if (e0 + 32 * i >= e1) break;                   // warp-uniform
+            const int32_t r = warp_rank(mine16, c[i], s, e0 + 32 * i + lane < e1, lane);
+            where[i] = (uint32_t)c[i] << 16 | (uint32_t)r;
+        }
+    } else {
+        for (int64_t k = e0 + lane; k < e1; k += 32)
+            atomicAdd(mine32 + (int)(__ldg(&recs[b0 + k].col) - c0), 1);
+    }
+    __syncthreads();
+    // exclusive scan over (column, warp); thread t takes columns [t cpt, t cpt + cpt)
+    const int cpt = (nc + 32 * kOrderWarps - 1) / (32 * kOrderWarps);
+    int32_t total = 0;
+    for (int j = tid * cpt; j < (tid + 1) * cpt && j < nc; ++j) {
+        if (small) {
+#pragma unroll 8
+            for (int w = 0; w < kOrderWarps; ++w) total += half[w * nc + j];
+        } else {
+            for (int w = 0; w < kBigWarps; ++w) total += full[w * nc + j];
+        }
+    }
+    int32_t incl = total;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int32_t up = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += up;
+    }
+    if (lane == 31) wtot[warp] = incl;
+    __syncthreads();
+    int32_t at = incl - total;
+    for (int w = 0; w < warp; ++w) at += wtot[w];
+    for (int j = tid * cpt; j < (tid + 1) * cpt && j < nc; ++j) {
+        if (c0 + j < n) col_ptr[c0 + j] = (int32_t)(b0 + at);
+        if (small) {
+#pragma unroll
+            for (int w = 0; w < kOrderWarps; w += 4) {
+                int32_t c[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) c[u] = half[(w + u) * nc + j];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    half[(w + u) * nc + j] = (uint16_t)at;
+                    at += c[u];
+                }
+            }
+        } else {
+            for (int w = 0; w < kBigWarps; ++w) {
+                const int32_t c = full[w * nc + j];
+                full[w * nc + j] = at;
+                at += c;
+            }
+        }
+    }
+    if (blockIdx.x == gridDim.x - 1 && tid == 0) col_ptr[n] = (int32_t)nnz;
+    __syncthreads();
+    if (small) {
+        // 64-bit values first (aligned), then rows, positions and narrow values
+        const size_t at0 = ((size_t)kOrderWarps * nc * 2 + 15) / 16 * 16;
+        uint64_t *s64 = reinterpret_cast<uint64_t *>(order_raw + at0);
+        int32_t *srow = reinterpret_cast<int32_t *>(order_raw + at0 + (WIDE ? 8 * CAP : 0));
+        int32_t *sk = srow + CAP;
+        uint32_t *sv = reinterpret_cast<uint32_t *>(sk + CAP);
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) {
+            const int64_t k = e0 + 32 * i + lane;
+            if (k >= e1) break;
+            Rec r;
+            ld_raw<16, CACHED>(&r, recs + b0 + k);
+            const int place = (int)mine16[where[i] >> 16] + (int)(where[i] & 0xffffu);
+            srow[place] = r.row;
+            sk[place] = r.k;
+            if (vals_t) {
+                if constexpr (WIDE) s64[place] = recs64[b0 + k];
+                else sv[place] = r.v;
+            }
+        }
+        __syncthreads();
+        for (int q = tid; q < (int)len; q += 32 * kOrderWarps) {
+            row_idx[b0 + q] = srow[q];
+            perm[b0 + q] = sk[q];
+            if (vals_t) {
+                if constexpr (WIDE) vals_t[b0 + q] = s64[q];
+                else vals_t[b0 + q] = (E)sv[q];
+            }
+        }
+        return;
+    }
+    for (int64_t kb = e0; kb < e1; kb += 32) {              // warp-uniform
+        const int64_t k = kb + lane;
+        const bool valid = k < e1;
+        Rec r{};
+        if (valid) ld_raw<16, CACHED>(&r, recs + b0 + k);
+        const int32_t pos = warp_rank(mine32, valid ? (int32_t)(r.col - c0) : 0, s, valid, lane);
+        if (valid) {
+            row_idx[b0 + pos] = r.row;
+            perm[b0 + pos] = r.k;
+            if (vals_t) {
+                if constexpr (WIDE) vals_t[b0 + pos] = recs64[b0 + k];
+                else vals_t[b0 + pos] = (E)r.v;
+            }
+        }
+    }
+}
+
+struct Plan {
+    int s;                  // log2 of the columns per block
+    int64_t blocks;         // column blocks
+    int passes;             // partition passes (1 or 2)
+    int bits[2], nb[2];     // of each pass: bits of its digit, number of digits
+    int64_t tiles, nseg;
+    size_t off_cells, off_segs, off_starts, off_first, off_rec[2], off_wide[2], bytes;
+};
+
+size_t up256(size_t b) { return (b + 255) / 256 * 256; }
+
+Plan make_plan(int64_t n, int64_t nnz, int vbytes) {
+    Plan p{};
+    // columns per block: as many as leave the mean column block three quarters of what
+    // the ordering kernel holds on chip, and two blocks per SM or more where they would
+    // still have 2048 entries
+    const int64_t mean = (vbytes == 8 ? kOrderCap<uint64_t> : kOrderCap<uint32_t>) / 4 * 3;
+    int s = kMaxColBits;
+    auto blocks = [&](int bits) { return ((n - 1) >> bits) + 1; };
+    while (s > 0 && blocks(s - 1) <= (int64_t)kMaxBlocks * kMaxBlocks &&
+           (blocks(s) * mean < nnz || (blocks(s) < 304 && blocks(s) * 2048 < nnz)))
+        --s;
+    p.s = s;
+    p.blocks = ((n - 1) >> s) + 1;
+    int bits = 0;
+    while ((1LL << bits) < p.blocks) ++bits;
+    p.passes = bits > kDigitBits ? 2 : 1;
+    p.bits[0] = p.passes == 1 ? bits : (bits + 1) / 2;
+    p.bits[1] = bits - p.bits[0];
+    p.nb[0] = p.passes == 1 ? (int)p.blocks : 1 << p.bits[0];
+    p.nb[1] = p.passes == 1 ? 0 : (int)((p.blocks - 1) >> p.bits[0]) + 1;
+    p.tiles = ceil_div(nnz, kTile);
+    p.nseg = ceil_div(p.tiles, kSegTiles);
+    const int64_t nb = p.nb[0] > p.nb[1] ? p.nb[0] : p.nb[1];
+    size_t at = 0;
+    p.off_cells = at;
+    at += up256((size_t)(p.tiles * nb) * 4);
+    p.off_segs = at;
+    at += up256((size_t)(p.nseg * nb) * 4);
+    p.off_starts = at;
+    at += up256((size_t)(p.blocks > nb ? p.blocks : nb) * 4);
+    p.off_first = at;
+    at += up256((size_t)ceil_div(nnz, kChunk) * 4);
+    for (int i = 0; i < p.passes; ++i) {
+        p.off_rec[i] = at;
+        at += up256((size_t)nnz * 16);
+        p.off_wide[i] = at;
+        if (vbytes == 8) at += up256((size_t)nnz * 8);
+    }
+    p.bytes = at;
+    return p;
+}
+
+template <typename E>
+lak_status run(const Plan &p, int32_t *col_ptr, int32_t *row_idx, int32_t *perm, E *vals_t,
+               const int32_t *rp, const int32_t *ci, const E *vals, int64_t m, int64_t n,
+               int64_t nnz, char *w, cudaStream_t st) {
+    int32_t *cells = reinterpret_cast<int32_t *>(w + p.off_cells);
+    int32_t *segs = reinterpret_cast<int32_t *>(w + p.off_segs);
+    int32_t *starts = reinterpret_cast<int32_t *>(w + p.off_starts);
+    int32_t *first = reinterpret_cast<int32_t *>(w + p.off_first);
+    const bool wide = sizeof(E) == 8 && vals != nullptr;
+    Rec *rec[2];
+    uint64_t *r64[2];
+    for (int i = 0; i < 2; ++i) {
+        const int j = i < p.passes ? i : 0;
+        rec[i] = reinterpret_cast<Rec *>(w + p.off_rec[j]);
+        r64[i] = wide ? reinterpret_cast<uint64_t *>(w + p.off_wide[j]) : nullptr;
+    }
+    const int move_most = (int)move_smem<E>(kMaxBlocks);
+    const int order_most = (int)order_smem<E>(kMaxColBits);
+    cudaError_t e = cudaFuncSetAttribute(part_move_kernel<E, true>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, move_most);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(part_move_kernel<E, false>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, move_most);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(order_kernel<E>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 order_most);
+    if (e != cudaSuccess)
+        return fail(LAK_ECUDA, "csr_transpose: shared memory: %s", cudaGetErrorString(e));
+    launch_k(chunk_rows_kernel, (unsigned)(ceil_div(m, 256) < 65535 ? ceil_div(m, 256) : 65535), 256,
+             0, st, first, rp, m);
+    for (int i = 0; i < p.passes; ++i) {
+        const int nb = p.nb[i];
+        const int shift = p.s + (i ? p.bits[0] : 0);
+        const int mask = p.passes == 2 && i == 0 ? nb - 1 : 0x7fffffff;
+        const dim3 sgrid((unsigned)ceil_div(nb, 256), (unsigned)p.nseg);
+        const int32_t *keys = i == 0 ? ci : &rec[0]->col;
+        const int bits = p.bits[i];
+        launch_k(part_count_kernel, (unsigned)p.tiles, kTileThreads, (size_t)nb * 4, st, cells,
+                 keys, i == 0 ? 1 : 4, nnz, shift, mask, nb);
+        launch_k(seg_sum_kernel, sgrid, 256, 0, st, segs, (const int32_t *)cells, p.tiles, nb);
+        launch_k(seg_scan_kernel, 1, 1024, 0, st, segs, starts, p.nseg, nb);
+        launch_k(seg_apply_kernel, sgrid, 256, 0, st, cells, (const int32_t *)segs, p.tiles, nb);
+        if (i == 0)
+            launch_k(part_move_kernel<E, true>, (unsigned)p.tiles, kTileThreads, move_smem<E>(nb),
+                     st, rec[0], r64[0], rp, ci, vals, (const Rec *)nullptr,
+                     (const uint64_t *)nullptr, (const int32_t *)cells,
+                     (const int32_t *)first, m, nnz, shift, mask, nb, bits);
+        else
+            launch_k(part_move_kernel<E, false>, (unsigned)p.tiles, kTileThreads, move_smem<E>(nb),
+                     st, rec[1], r64[1], rp, ci, (const E *)nullptr, (const Rec *)rec[0],
+                     (const uint64_t *)r64[0], (const int32_t *)cells,
+                     (const int32_t *)first, m, nnz, shift, mask, nb, bits);
+    }
+    if (p.passes == 2)
+        launch_k(bounds_kernel, (unsigned)ceil_div(p.blocks, 128), 128, 0, st, starts,
+                 (const Rec *)rec[1], nnz, p.blocks, p.s);
+    launch_k(order_kernel<E>, (unsigned)p.blocks, 32 * kOrderWarps, order_smem<E>(p.s), st,
+             col_ptr, row_idx, perm, vals ? vals_t : (E *)nullptr, (const Rec *)rec[p.passes - 1],
+             (const uint64_t *)r64[p.passes - 1],
+             (const int32_t *)starts, n, nnz, p.s);
+    return check_launch("csr_transpose");
+}
+
+}  // namespace
+
+size_t transpose_workspace(int64_t n, int64_t nnz, int vbytes) {
+    return n < 1 || nnz < 1 || n > kTransposeMaxCols ? 0 : make_plan(n, nnz, vbytes).bytes;
+}
+
+lak_status launch_transpose(int32_t *col_ptr, int32_t *row_idx, int32_t *perm, void *vals_t,
+                            const int32_t *rp, const int32_t *ci, const void *vals, int64_t m,
+                            int64_t n, int64_t nnz, int vbytes, void *ws, cudaStream_t s) {
+    const Plan p = make_plan(n, nnz, vbytes);
+    char *w = static_cast<char *>(ws);
+    switch (vbytes) {
+    case 2:
+        return run<uint16_t>(p, col_ptr, row_idx, perm, (uint16_t *)vals_t, rp, ci,
+                             (const uint16_t *)vals, m, n, nnz, w, s);
+    case 8:
+        return run<uint64_t>(p, col_ptr, row_idx, perm, (uint64_t *)vals_t, rp, ci,
+                             (const uint64_t *)vals, m, n, nnz, w, s);
+    default:
+        return run<uint32_t>(p, col_ptr, row_idx, perm, (uint32_t *)vals_t, rp, ci,
+                             (const uint32_t *)vals, m, n, nnz, w, s);
+    }
+}
+
+}  // namespace lak
