@@ -5,6 +5,9 @@
 // realised as V consecutive elements per thread read with the widest aligned
 // loads (up to 256-bit on sm_103a).  A scalar prologue/epilogue covers the
 // elements before the first aligned address and after the last full group.
+// Operands of unlike alignment (slices of one array, odd offsets) take the kernels'
+// SH forms: the first operand is accessed at its alignment, the others through two
+// aligned 16-byte loads shifted in registers, the second of which hits L1.
 #include "lak_internal.cuh"
 #include "vec_loop.cuh"
 
@@ -13,7 +16,7 @@ namespace {
 
 // ---- copy: a bit copy of elements of 2, 4 or 8 bytes ----------------------
 
-template <typename E, int V>
+template <typename E, int V, bool SH = false>
 __global__ void __launch_bounds__(512)
 copy_kernel(E *__restrict__ x, const E *__restrict__ y, int64_t n, int64_t head,
             int64_t nchunks, int inc) {
@@ -23,7 +26,7 @@ copy_kernel(E *__restrict__ x, const E *__restrict__ y, int64_t n, int64_t head,
     const Range r = chunk_range(nchunks, inc);
     for (int64_t c = r.begin; c < r.end; c += r.stride) {
         Pack<E, V> p;
-        load_pack<E, V, STREAM>(p, yb + c * V);
+        load_operand<E, V, STREAM, SH, CACHED>(p, yb + c * V);
         store_pack<E, V>(xb + c * V, p);
     }
     const int64_t body_end = head + nchunks * V;
@@ -37,7 +40,7 @@ copy_kernel(E *__restrict__ x, const E *__restrict__ y, int64_t n, int64_t head,
 
 // ---- axpy: x = y + alpha*z, one fused multiply-add per element -------------
 
-template <typename T, int V>
+template <typename T, int V, bool SH = false>
 __global__ void __launch_bounds__(512)
 axpy_kernel(T *x, const T *y, const T *z, typename Acc<T>::type alpha, int64_t n, int64_t head,
             int64_t nchunks, int inc) {
@@ -47,8 +50,8 @@ axpy_kernel(T *x, const T *y, const T *z, typename Acc<T>::type alpha, int64_t n
     for (int64_t c = r.begin; c < r.end; c += r.stride) {
         const int64_t o = head + c * V;
         Pack<T, V> py, pz, px;
-        load_pack<T, V, COHERENT>(py, y + o);
-        load_pack<T, V, COHERENT>(pz, z + o);
+        load_operand<T, V, COHERENT, SH>(py, y + o);
+        load_operand<T, V, COHERENT, SH>(pz, z + o);
 #pragma unroll
         for (int v = 0; v < V; ++v)
             px.e[v] = narrow<T>(fma_acc(alpha, widen(pz.e[v]), widen(py.e[v])));
@@ -75,7 +78,7 @@ axpy_kernel(T *x, const T *y, const T *z, typename Acc<T>::type alpha, int64_t n
 // call leaves the counter at zero for the next call; a one-block grid writes
 // its sum directly.
 
-template <typename T, int V>
+template <typename T, int V, bool SH = false>
 __global__ void __launch_bounds__(512)
 dot_kernel(void *out, const T *__restrict__ x, const T *__restrict__ y, int64_t n,
            int64_t head, int64_t nchunks, int inc, unsigned int *counter,
@@ -87,13 +90,20 @@ dot_kernel(void *out, const T *__restrict__ x, const T *__restrict__ y, int64_t 
     for (int v = 0; v < V; ++v) acc[v] = A(0);
 
     const Range r = chunk_range(nchunks, inc);
-    for (int64_t c = r.begin; c < r.end; c += r.stride) {
+    auto chunk = [&](int64_t c) {
         const int64_t o = head + c * V;
         Pack<T, V> px, py;
-        load_pack<T, V, STREAM>(px, x + o);
-        load_pack<T, V, STREAM>(py, y + o);
+        load_operand<T, V, STREAM, SH, CACHED>(px, x + o);
+        load_operand<T, V, STREAM, SH, CACHED>(py, y + o);
 #pragma unroll
         for (int v = 0; v < V; ++v) acc[v] = fma_acc(widen(px.e[v]), widen(py.e[v]), acc[v]);
+    };
+    if constexpr (SH) {
+        // the grids are sized for packs of 32 to 64 bytes: four 16-byte ones at a time
+#pragma unroll 4
+        for (int64_t c = r.begin; c < r.end; c += r.stride) chunk(c);
+    } else {
+        for (int64_t c = r.begin; c < r.end; c += r.stride) chunk(c);
     }
     {
         const int64_t body_end = head + nchunks * V;
@@ -126,7 +136,7 @@ dot_kernel(void *out, const T *__restrict__ x, const T *__restrict__ y, int64_t 
 // last-block combines run in FP64 as in dot_kernel.  The result is written as
 // a double.
 
-template <typename T, int V>
+template <typename T, int V, bool SH = false>
 __global__ void __launch_bounds__(512)
 dot_comp_kernel(double *out, const T *__restrict__ x, const T *__restrict__ y, int64_t n,
                 int64_t head, int64_t nchunks, int inc, unsigned int *counter,
@@ -154,8 +164,8 @@ dot_comp_kernel(double *out, const T *__restrict__ x, const T *__restrict__ y, i
     for (int64_t ch = r.begin; ch < r.end; ch += r.stride) {
         const int64_t o = head + ch * V;
         Pack<T, V> px, py;
-        load_pack<T, V, STREAM>(px, x + o);
-        load_pack<T, V, STREAM>(py, y + o);
+        load_operand<T, V, STREAM, SH, CACHED>(px, x + o);
+        load_operand<T, V, STREAM, SH, CACHED>(py, y + o);
 #pragma unroll
         for (int v = 0; v < V; ++v) add(sv[v], cv[v], widen(px.e[v]), widen(py.e[v]));
     }
@@ -179,7 +189,12 @@ dot_comp_kernel(double *out, const T *__restrict__ x, const T *__restrict__ y, i
 template <typename E>
 lak_status copy_vec(int vec, E *x, const E *y, int64_t n, int64_t head, const Launch &L,
                     cudaStream_t s) {
-    const int64_t nchunks = (n - head) / vec;
+    const int64_t nchunks = body_packs(n, head, L);
+    if (L.shifted) {
+        launch_k(copy_kernel<E, 16 / (int)sizeof(E), true>, L.grid, L.block, 0, s, x, y, n, head,
+                 nchunks, L.inc);
+        return check_launch("vec_copy");
+    }
     switch (vec) {
     case 1: launch_k(copy_kernel<E, 1>, L.grid, L.block, 0, s, x, y, n, head, nchunks, L.inc); break;
     case 2: launch_k(copy_kernel<E, 2>, L.grid, L.block, 0, s, x, y, n, head, nchunks, L.inc); break;
@@ -199,7 +214,12 @@ lak_status axpy_t(int vec, void *x, const void *y, const void *z, double alpha, 
     const T *yp = static_cast<const T *>(y);
     const T *zp = static_cast<const T *>(z);
     const A a = static_cast<A>(alpha);
-    const int64_t nchunks = (n - head) / vec;
+    const int64_t nchunks = body_packs(n, head, L);
+    if (L.shifted) {
+        launch_k(axpy_kernel<T, 16 / (int)sizeof(T), true>, L.grid, L.block, 0, s, xp, yp, zp, a, n,
+                 head, nchunks, L.inc);
+        return check_launch("vec_axpy");
+    }
     switch (vec) {
     case 1: launch_k(axpy_kernel<T, 1>, L.grid, L.block, 0, s, xp, yp, zp, a, n, head, nchunks, L.inc); break;
     case 2: launch_k(axpy_kernel<T, 2>, L.grid, L.block, 0, s, xp, yp, zp, a, n, head, nchunks, L.inc); break;
@@ -218,7 +238,12 @@ lak_status dot_t(int vec, void *out, const void *x, const void *y, int64_t n, in
     const T *yp = static_cast<const T *>(y);
     unsigned int *counter = static_cast<unsigned int *>(ws);
     double *partials = reinterpret_cast<double *>(static_cast<char *>(ws) + LAK_WS_COUNTER_BYTES);
-    const int64_t nchunks = (n - head) / vec;
+    const int64_t nchunks = body_packs(n, head, L);
+    if (L.shifted) {
+        launch_k(dot_kernel<T, 16 / (int)sizeof(T), true>, L.grid, L.block, 0, s, out, xp, yp, n,
+                 head, nchunks, L.inc, counter, partials);
+        return check_launch("vec_dot");
+    }
 #define LAK_DOT(VV)                                                                     \
     launch_k(dot_kernel<T, VV>, L.grid, L.block, 0, s, out, xp, yp, n, head, nchunks, L.inc, \
                                                  counter, partials)
@@ -242,7 +267,12 @@ lak_status dot_comp_t(int vec, void *out, const void *x, const void *y, int64_t 
     double *o = static_cast<double *>(out);
     unsigned int *counter = static_cast<unsigned int *>(ws);
     double *partials = reinterpret_cast<double *>(static_cast<char *>(ws) + LAK_WS_COUNTER_BYTES);
-    const int64_t nchunks = (n - head) / vec;
+    const int64_t nchunks = body_packs(n, head, L);
+    if (L.shifted) {
+        launch_k(dot_comp_kernel<T, 16 / (int)sizeof(T), true>, L.grid, L.block, 0, s, o, xp, yp, n,
+                 head, nchunks, L.inc, counter, partials);
+        return check_launch("vec_dot_compensated");
+    }
 #define LAK_DOTC(VV)                                                                    \
     launch_k(dot_comp_kernel<T, VV>, L.grid, L.block, 0, s, o, xp, yp, n, head, nchunks, L.inc, \
                                                       counter, partials)

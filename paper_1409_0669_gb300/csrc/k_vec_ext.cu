@@ -14,7 +14,7 @@
 namespace lak {
 namespace {
 
-template <typename T, int V>
+template <typename T, int V, bool SH = false>
 __global__ void __launch_bounds__(512)
 axpby_kernel(T *x, typename Acc<T>::type alpha, const T *y, typename Acc<T>::type beta,
              const T *z, int64_t n, int64_t head, int64_t nchunks, int inc) {
@@ -23,8 +23,8 @@ axpby_kernel(T *x, typename Acc<T>::type alpha, const T *y, typename Acc<T>::typ
     for (int64_t c = r.begin; c < r.end; c += r.stride) {
         const int64_t o = head + c * V;
         Pack<T, V> py, pz, px;
-        load_pack<T, V, COHERENT>(py, y + o);
-        load_pack<T, V, COHERENT>(pz, z + o);
+        load_operand<T, V, COHERENT, SH>(py, y + o);
+        load_operand<T, V, COHERENT, SH>(pz, z + o);
 #pragma unroll
         for (int v = 0; v < V; ++v)
             px.e[v] = narrow<T>(fma_acc(alpha, widen(py.e[v]), beta * widen(pz.e[v])));
@@ -52,7 +52,7 @@ axpby_strided_kernel(T *x, int64_t incx, typename Acc<T>::type alpha, const T *y
 // x = y + alpha*z; s = sum x_i^2 of the STORED x (after rounding to the storage
 // type), reduced like dot_kernel: per-thread accumulators, warp shuffles, FP64
 // block partials, last block combines in block order.
-template <typename T, int V>
+template <typename T, int V, bool SH = false>
 __global__ void __launch_bounds__(512, 2)     // two 512-thread blocks per SM
 axpy_norm2_kernel(T *x, const T *y, const T *z, typename Acc<T>::type alpha, void *out,
                   int64_t n, int64_t head, int64_t nchunks, int inc, unsigned int *counter,
@@ -66,8 +66,8 @@ axpy_norm2_kernel(T *x, const T *y, const T *z, typename Acc<T>::type alpha, voi
     for (int64_t c = r.begin; c < r.end; c += r.stride) {
         const int64_t o = head + c * V;
         Pack<T, V> py, pz, px;
-        load_pack<T, V, COHERENT>(py, y + o);
-        load_pack<T, V, COHERENT>(pz, z + o);
+        load_operand<T, V, COHERENT, SH>(py, y + o);
+        load_operand<T, V, COHERENT, SH>(pz, z + o);
 #pragma unroll
         for (int v = 0; v < V; ++v) {
             px.e[v] = narrow<T>(fma_acc(alpha, widen(pz.e[v]), widen(py.e[v])));
@@ -171,7 +171,12 @@ lak_status axpby_t(void *x, double alpha, const void *y, double beta, const void
     T *xp = static_cast<T *>(x);
     const T *yp = static_cast<const T *>(y);
     const T *zp = static_cast<const T *>(z);
-    const int64_t nchunks = (n - head) / L.vec;
+    const int64_t nchunks = body_packs(n, head, L);
+    if (L.shifted) {
+        launch_k(axpby_kernel<T, 16 / (int)sizeof(T), true>, L.grid, L.block, 0, s, xp, (A)alpha, yp,
+                 (A)beta, zp, n, head, nchunks, L.inc);
+        return check_launch("vec_axpby");
+    }
 #define LAK_AB(VV)                                                                        \
     launch_k(axpby_kernel<T, VV>, L.grid, L.block, 0, s, xp, (A)alpha, yp, (A)beta, zp, n, head, \
                                                    nchunks, L.inc)
@@ -207,7 +212,12 @@ lak_status axpy_norm2_t(void *x, const void *y, const void *z, double alpha, voi
     const T *zp = static_cast<const T *>(z);
     unsigned int *counter = static_cast<unsigned int *>(ws);
     double *partials = reinterpret_cast<double *>(static_cast<char *>(ws) + LAK_WS_COUNTER_BYTES);
-    const int64_t nchunks = (n - head) / L.vec;
+    const int64_t nchunks = body_packs(n, head, L);
+    if (L.shifted) {
+        launch_k(axpy_norm2_kernel<T, 16 / (int)sizeof(T), true>, L.grid, L.block, 0, s, xp, yp, zp,
+                 (A)alpha, out, n, head, nchunks, L.inc, counter, partials);
+        return check_launch("vec_axpy_norm2");
+    }
 #define LAK_AN(VV)                                                                          \
     launch_k(axpy_norm2_kernel<T, VV>, L.grid, L.block, 0, s, xp, yp, zp, (A)alpha, out, n, head,   \
                                                         nchunks, L.inc, counter, partials)

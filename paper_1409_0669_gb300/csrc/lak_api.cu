@@ -288,6 +288,22 @@ int waves_grid(const DeviceInfo *di, int block) {
     return di->sms * per_sm;
 }
 
+// Operands that share no 16-byte alignment: the scalar prologue that aligns the first
+// one and leaves every other's first 16-byte window inside its array.  False where
+// fewer than four packs would be left (all elements are then done one by one).
+bool shifted_head(int es, const void *const *ptrs, int nptrs, int64_t n, int64_t *head) {
+    const int v = 16 / es;
+    int64_t h = (int64_t)((16 - (uintptr_t)ptrs[0] % 16) % 16) / es;
+    for (int i = 1; i < nptrs; ++i)
+        if ((int64_t)(((uintptr_t)ptrs[i] + h * es) % 16) > h * es) {
+            h += v;
+            break;
+        }
+    if (n - h < 4 * v) return false;
+    *head = h;
+    return true;
+}
+
 struct VecPlan {
     Launch L;
     int64_t head;
@@ -303,12 +319,28 @@ lak_status plan_vector(lak_op op, lak_dtype dt, int64_t n, const lak_cfg *cfg,
     int want = c.vec ? c.vec : builtin_default(op, dt, bucket).vec;
     int64_t head = 0;
     int vec = ptrs ? pick_vec(want, es, ptrs, nptrs, n, &head) : want;
+    // Operands of unlike alignment, one-element accesses against windows (us; 21.5 M
+    // entries, L2 cold): BF16 update 44.8 -> 22.3, copy 22.3 -> 15.1, inner product 28.2 ->
+    // 19.4; FP32 update 56.0 -> 41.9, copy 31.4 -> 27.8.  The FP32 inner product keeps its
+    // one-element accesses (1e8 entries: 121 against 146 us), and FP64, whose warps read
+    // whole lines that way, too (update 86.0 against 88.5 us).
+    const bool unlike = ptrs && vec * es < 16 && want * es >= 16;
+    const bool shifted = unlike && es <= (op == LAK_OP_DOT ? 2 : 4) &&
+                         shifted_head(es, ptrs, nptrs, n, &head);
+    if (shifted) vec = 16 / es;
     const int64_t nchunks = vec > 0 ? (n - head) / vec : n;
     int64_t grid = c.grid;
     if (grid == 0) {
         const int64_t need = ceil_div(nchunks > 0 ? nchunks : 1, c.block);
         const int per_sm = default_grid_per_sm(op, dt, bucket);
-        const int64_t cap = per_sm > 0 ? (int64_t)per_sm * di->sms : waves_grid(di, c.block);
+        int64_t cap = per_sm > 0 ? (int64_t)per_sm * di->sms : waves_grid(di, c.block);
+        // the table's caps go with its pack widths: narrower accesses take as many more
+        // blocks, up to a full SM (FP32 dot of 21.5 M entries 49.9 -> 29.7 us)
+        if (unlike && es <= 4) {
+            const int64_t more = cap * (want * es / 16);
+            const int64_t most = waves_grid(di, c.block);
+            cap = more < most ? more : cap > most ? cap : most;
+        }
         grid = need < cap ? need : cap;
         // an inner product one block covers in two passes skips the grid-wide
         // combine (a ticket and a second block pass, ~2 us; a pass is less)
@@ -316,7 +348,7 @@ lak_status plan_vector(lak_op op, lak_dtype dt, int64_t n, const lak_cfg *cfg,
     }
     if (grid < 1) grid = 1;
     if (grid > 0x7fffffff) grid = 0x7fffffff;
-    out->L = Launch{c.block, (int)grid, vec, c.increment};
+    out->L = Launch{c.block, (int)grid, vec, c.increment, shifted};
     out->head = head;
     return LAK_OK;
 }
@@ -615,6 +647,16 @@ namespace {
 
 bool aligned_elem(const void *p, int es) { return (uintptr_t)p % (uintptr_t)es == 0; }
 
+// Blocks a call whose plans at the wanted and at the narrowest width are a and b can
+// launch: operands of unlike alignment may take a full wave (plan_vector).
+int widest_grid(const Launch &a, const Launch &b, const lak_cfg *cfg) {
+    int g = a.grid > b.grid ? a.grid : b.grid;
+    const DeviceInfo *di = device_info();
+    const bool automatic = !cfg || cfg->block == 0 || cfg->grid == 0;
+    if (automatic && di && b.grid > 1 && waves_grid(di, a.block) > g) g = waves_grid(di, a.block);
+    return g;
+}
+
 lak_status common_checks(const char *who, lak_dtype dt, const lak_cfg *cfg) {
     if (!valid_dtype(dt)) return fail(LAK_EDTYPE, "%s: unknown dtype %d", who, (int)dt);
     return check_cfg(cfg, who);
@@ -776,8 +818,7 @@ LAK_API size_t vec_dot_workspace(int64_t n, lak_dtype dtype, const lak_cfg *cfg)
     lak_cfg c = base_cfg(LAK_OP_DOT, dtype, bucket_of(op_bytes(LAK_OP_DOT, dtype, n, n, 0)), cfg);
     c.vec = 1;
     if (plan_vector(LAK_OP_DOT, dtype, n, &c, nullptr, 0, &p1) != LAK_OK) return 0;
-    const int grid = p1.L.grid > p.L.grid ? p1.L.grid : p.L.grid;
-    return (size_t)LAK_WS_COUNTER_BYTES + 8 * (size_t)grid;
+    return (size_t)LAK_WS_COUNTER_BYTES + 8 * (size_t)widest_grid(p.L, p1.L, cfg);
 }
 
 LAK_API lak_status vec_dot(void *out, const void *x, const void *y, int64_t n, lak_dtype dtype,
@@ -1012,8 +1053,7 @@ LAK_API size_t vec_axpy_norm2_workspace(int64_t n, lak_dtype dtype, const lak_cf
     lak_cfg c = base_cfg(LAK_OP_AXPY, dtype, bucket_of(op_bytes(LAK_OP_AXPY, dtype, n, n, 0)), cfg);
     c.vec = 1;
     if (plan_vector(LAK_OP_AXPY, dtype, n, &c, nullptr, 0, &p1) != LAK_OK) return 0;
-    const int grid = p1.L.grid > p.L.grid ? p1.L.grid : p.L.grid;
-    return (size_t)LAK_WS_COUNTER_BYTES + 8 * (size_t)grid;
+    return (size_t)LAK_WS_COUNTER_BYTES + 8 * (size_t)widest_grid(p.L, p1.L, cfg);
 }
 
 LAK_API lak_status vec_axpy_norm2(void *x, const void *y, const void *z, double alpha, void *out,

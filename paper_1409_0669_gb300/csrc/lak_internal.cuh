@@ -41,7 +41,15 @@ struct Launch {
     int grid;    // blocks (for column-major GEMV: total over both grid axes)
     int vec;     // elements per access group (see lak_cfg)
     int inc;     // LAK_INC_GLOBAL / LAK_INC_LOCAL
+    // vector ops: operands of unlike alignment, read through shifted 16-byte windows
+    // (vec is 16 bytes, the first operand is aligned, the body ends a pack early)
+    bool shifted = false;
 };
+
+// Packs of a vector op's body: n elements after `head` scalar ones.
+inline int64_t body_packs(int64_t n, int64_t head, const Launch &L) {
+    return (n - head) / L.vec - (L.shifted ? 1 : 0);
+}
 
 inline int esize(lak_dtype dt) {
     switch (dt) {
@@ -221,7 +229,9 @@ template <typename T, int V> struct Pack { T e[V]; };
 // not written by the kernel).  COHERENT: ordinary coherent load, no L1
 // allocation (an output may alias this input).  CACHED: read-only path with
 // L1 allocation (operands many threads re-read, e.g. the GEMV right-hand side).
-enum { STREAM = 0, COHERENT = 1, CACHED = 2 };
+// WINDOW: coherent, with L1 allocation (16-byte windows, every second load of which
+// hits the line the first one brought).
+enum { STREAM = 0, COHERENT = 1, CACHED = 2, WINDOW = 3 };
 
 template <int B, int P> __device__ __forceinline__ void ld_raw(void *dst, const void *p);
 
@@ -313,6 +323,13 @@ template <> __device__ __forceinline__ void ld_raw<32, CACHED>(void *dst, const 
           "=r"(w[7])
         : "l"(p));
     memcpy(dst, w, 32);
+}
+
+template <> __device__ __forceinline__ void ld_raw<16, WINDOW>(void *dst, const void *p) {
+    uint32_t w[4];
+    asm("ld.global.v4.b32 {%0,%1,%2,%3}, [%4];"
+        : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "l"(p));
+    memcpy(dst, w, 16);
 }
 
 template <int B> __device__ __forceinline__ void st_raw(void *p, const void *src);
@@ -408,6 +425,16 @@ __device__ __forceinline__ void load_window(Pack<T, 16 / (int)sizeof(T)> &pk, co
         shift_words<(int)sizeof(T)>(w, sb);
     }
     memcpy(&pk, w, 16);
+}
+
+// One pack of an operand of a vector op: at its own alignment, or (SH) through a window
+// at any element address; P is the policy of the former, WP of the latter.
+template <typename T, int V, int P, bool SH, int WP = WINDOW>
+__device__ __forceinline__ void load_operand(Pack<T, V> &pk, const T *p) {
+    if constexpr (SH)
+        load_window<T, WP>(pk, p, (uint32_t)((uintptr_t)p % 16));
+    else
+        load_pack<T, V, P>(pk, p);
 }
 
 // Cached (L1-allocating) read-only scalar load, for operands that many
