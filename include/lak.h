@@ -392,8 +392,9 @@ LAK_API lak_status dense_gemv_trans(void *y, const void *A, const void *x, int64
  *     them with one fused multiply-add each and splits at row ends; rows
  *     crossing lanes are joined by a segmented warp scan, deterministically and
  *     without atomics;
- *   mean > 64: a power-of-two group of lanes per row (up to a warp) strides
- *     through the row and reduces with shuffles.
+ *   mean > 64: a power-of-two group of lanes per row (4 for FP64 rows of about 80
+ *     entries, up to a warp) strides through the row and reduces with shuffles;
+ *     warps with rows far longer than their mean take those with all lanes.
  * The environment variables LAK_SPMV_SEG_MIN_MEAN / LAK_SPMV_SEG_MAX_MEAN
  * (read once) move the bounds of the middle range.
  * Requirements the library does not check

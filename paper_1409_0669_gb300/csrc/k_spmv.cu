@@ -10,8 +10,9 @@
 // <= 12) take one or two lanes per row with U covering the row, so a warp
 // keeps 16-32 rows' loads in flight; their col_idx / vals loads are strided
 // across the warp and go through L1 (one miss brings the lines the next lanes
-// need).  Long rows (mean > 64) take more lanes per row and stream col_idx /
-// vals past L1.  In FP64 each lane keeps one accumulator chain.
+// need).  In FP64 each lane keeps one accumulator chain.  Long rows (mean > 64) take
+// spmv_long_kernel below; with an explicit configuration they take this kernel with
+// more lanes per row, col_idx / vals streamed past L1.
 //
 // Warp-segmented (spmv_seg_kernel, 13 <= mean <= 64): a warp owns 32
 // consecutive rows, whose entries are contiguous, and walks them in chunks of
@@ -88,6 +89,87 @@ spmv_kernel(T *__restrict__ y, const int32_t *__restrict__ rp, const int32_t *__
         }
         const Ac s = group_sum(acc[0], G);
         if (lg == 0 && row < row_end) y[row] = narrow<T>(s);
+    }
+}
+
+// One lane group's row: the G lanes of a group stride through its entries U at a time,
+// `longest` (uniform over the warp) bounding the steps so that slots no row of the warp
+// fills are not issued -- in FP64 a predicated-off FMA costs as much as a full one.
+// FP32 keeps two partial sums, FP64 one chain.  All 32 lanes call it; every lane of a
+// group returns the row's sum.
+template <typename T, int G, int U, int P>
+__device__ __forceinline__ typename Acc<T>::type group_row(const int32_t *__restrict__ c,
+                                                           const T *__restrict__ v,
+                                                           const T *__restrict__ x, int32_t len,
+                                                           int32_t longest, int lg) {
+    using Ac = typename Acc<T>::type;
+    constexpr int S = sizeof(Ac) == 8 ? 1 : 2;              // partial sums
+    Ac acc[S];
+#pragma unroll
+    for (int i = 0; i < S; ++i) acc[i] = Ac(0);
+    for (int32_t base = 0; base < longest; base += G * U) {
+        int32_t col[U];
+        T val[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int32_t k = base + u * G + lg;
+            if (k < len) {
+                ld_raw<4, P>(&col[u], c + k);
+                ld_raw<(int)sizeof(T), P>(&val[u], v + k);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int32_t k = base + u * G + lg;
+            if (base + u * G < longest && k < len) {        // the first part is uniform
+                Ac &a = acc[u % S];
+                a = fma_acc(widen(val[u]), widen(ld_cached(x + col[u])), a);
+            }
+        }
+    }
+    if constexpr (S == 2) acc[0] += acc[1];
+    return group_sum(acc[0], G);
+}
+
+// Long rows (mean > 64): G lanes per row, 32 / G rows per warp (group_row).  A warp
+// whose longest row is far from the mean of its rows takes them one by one with all
+// its lanes instead.  FP64 is bound by the pipe's warp instructions, so fewer lanes per
+// row than the one-row form's serve it: 81 entries in 16 lanes took 8 FMAs (2 of them
+// for slots no row fills) and 4 adds for two rows, in 4 lanes 21 and 2 for eight.
+// Measured (us, one-row groups -> this; 41 M entries of a 3D elasticity matrix, L2 cold):
+// FP64 196 -> 108 (4.7 TB/s; FP64 pipe 78), FP32 90 -> 66, BF16 111 -> 59; rows with a
+// heavy tail (up to 50000 entries, mean 76) as before (FP64 899 -> 865, FP32 441 -> 411).
+template <typename T, int G>
+__global__ void __launch_bounds__(kSpmvLongBlock)
+spmv_long_kernel(T *__restrict__ y, const int32_t *__restrict__ rp,
+                 const int32_t *__restrict__ ci, const T *__restrict__ vals,
+                 const T *__restrict__ x, int64_t m) {
+    LAK_PDL_ENTRY();
+    using Ac = typename Acc<T>::type;
+    constexpr int U = 4, rows = 32 / G;
+    const int lane = threadIdx.x & 31, lg = lane % G;
+    const int64_t row0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * rows;
+    if (row0 >= m) return;                                   // warp-uniform
+    const int64_t row = row0 + lane / G;
+    const int64_t last = row0 + rows < m ? row0 + rows : m;
+    int32_t k0 = 0, len = 0;
+    if (row < m) {
+        k0 = __ldg(rp + row);
+        len = __ldg(rp + row + 1) - k0;
+    }
+    const int32_t longest = __reduce_max_sync(0xffffffffu, len);
+    const int64_t total = (int64_t)__ldg(rp + last) - __ldg(rp + row0);
+    constexpr int F = rows == 2 ? 3 : 4;                    // twice the factor on the mean
+    if (2 * (int64_t)longest * rows <= F * total + 64 * rows) {
+        const Ac t = group_row<T, G, U, CACHED>(ci + k0, vals + k0, x, len, longest, lg);
+        if (lg == 0 && row < m) y[row] = narrow<T>(t);
+    } else {
+        for (int r = 0; r < rows && row0 + r < m; ++r) {
+            const int32_t a = __shfl_sync(0xffffffffu, k0, r * G);
+            const int32_t n = __shfl_sync(0xffffffffu, len, r * G);
+            const Ac t = group_row<T, 32, U, STREAM>(ci + a, vals + a, x, n, n, lane);
+            if (lane == 0) y[row0 + r] = narrow<T>(t);
+        }
     }
 }
 
@@ -195,6 +277,41 @@ lak_status spmv_t(void *y, const int32_t *rp, const int32_t *ci, const void *val
 }
 
 }  // namespace
+
+namespace {
+
+template <typename T>
+lak_status spmv_long_t(void *y, const int32_t *rp, const int32_t *ci, const void *vals,
+                       const void *x, int64_t m, int G, cudaStream_t s) {
+    T *yp = static_cast<T *>(y);
+    const T *vp = static_cast<const T *>(vals);
+    const T *xp = static_cast<const T *>(x);
+    const unsigned grid = (unsigned)ceil_div(m * G, kSpmvLongBlock);
+#define LAK_LONG(GG)                                                                        \
+    launch_k(spmv_long_kernel<T, GG>, grid, kSpmvLongBlock, 0, s, yp, rp, ci, vp, xp, m)
+    switch (G) {
+    case 4: LAK_LONG(4); break;
+    case 8: LAK_LONG(8); break;
+    case 16: LAK_LONG(16); break;
+    default: LAK_LONG(32); break;
+    }
+#undef LAK_LONG
+    return check_launch("csr_spmv (long rows)");
+}
+
+}  // namespace
+
+lak_status launch_spmv_long(lak_dtype dt, void *y, const int32_t *rp, const int32_t *ci,
+                            const void *vals, const void *x, int64_t m, int group,
+                            cudaStream_t s) {
+    switch (dt) {
+    case LAK_F32: return spmv_long_t<float>(y, rp, ci, vals, x, m, group, s);
+    case LAK_F64: return spmv_long_t<double>(y, rp, ci, vals, x, m, group, s);
+    case LAK_BF16: return spmv_long_t<__nv_bfloat16>(y, rp, ci, vals, x, m, group, s);
+    case LAK_F16: return spmv_long_t<__half>(y, rp, ci, vals, x, m, group, s);
+    }
+    return fail(LAK_EDTYPE, "csr_spmv: unknown dtype %d", (int)dt);
+}
 
 lak_status launch_spmv(lak_dtype dt, void *y, const int32_t *rp, const int32_t *ci,
                        const void *vals, const void *x, int64_t m, const Launch &L, int group,

@@ -526,7 +526,8 @@ lak_status plan_gemv_col(lak_dtype dt, int64_t m, int64_t n, int64_t lda, const 
 
 struct SpmvPlan {
     Launch L;
-    int group;     // lanes per row (long-row variant); 0 = warp-stream variant
+    int group;     // lanes per row; 0 = warp-segmented variant
+    bool long_rows = false;    // spmv_long_kernel
 };
 
 // Mean row lengths between which the warp-segmented variant is used; below
@@ -560,6 +561,20 @@ lak_status plan_spmv(lak_dtype dt, int64_t m, int64_t n, int64_t nnz, const lak_
     const int bucket = bucket_of(op_bytes(LAK_OP_SPMV, dt, m, n, nnz));
     const int64_t mean = m > 0 ? ceil_div(nnz, m) : 1;
     const bool seg = mean >= spmv_seg_min_mean() && mean <= spmv_seg_max_mean();
+    if (mean > 64 && !seg && builtin_shape(LAK_OP_SPMV, dt, bucket, cfg)) {
+        // lanes per row by the mean row length, where they were timed (us): mean 81
+        // (elasticity) FP64 4 lanes 107, 8 lanes 119; FP32 4 and 8 lanes 65, 16 lanes 79;
+        // mean 130 (65..200) FP64 8 lanes 129, 4 lanes 141, 16 lanes 139; FP32 74, 88, 78;
+        // mean 600 FP64 32 lanes 131, 16 lanes 144; FP32 99 and 111
+        const int G = mean > 320 ? 32 : mean > 160 ? 16 : mean > 100 || dt != LAK_F64 ? 8 : 4;
+        int64_t blocks = ceil_div(m * G, kSpmvLongBlock);
+        if (blocks <= 0x7fffffff) {
+            out->L = Launch{kSpmvLongBlock, (int)blocks, 4, LAK_INC_GLOBAL};
+            out->group = G;
+            out->long_rows = true;
+            return LAK_OK;
+        }
+    }
     lak_cfg c = base_cfg(LAK_OP_SPMV, dt, bucket, cfg);
     bool overridden = cfg && cfg->block != 0;
     if (!overridden) {
@@ -1145,6 +1160,9 @@ LAK_API lak_status csr_spmv(void *y, const int32_t *row_ptr, const int32_t *col_
     SpmvPlan p;
     st = plan_spmv(dtype, m, n, nnz, cfg, &p);
     if (st != LAK_OK) return st;
+    if (p.long_rows)
+        return launch_spmv_long(dtype, y, row_ptr, col_idx, vals, x, m, p.group,
+                                (cudaStream_t)stream);
     return launch_spmv(dtype, y, row_ptr, col_idx, vals, x, m, p.L, p.group, (cudaStream_t)stream);
 }
 
