@@ -31,7 +31,7 @@ template <typename T, int U, int P>
 __global__ void __launch_bounds__(512)
 spmv_kernel(T *__restrict__ y, const int32_t *__restrict__ rp, const int32_t *__restrict__ ci,
             const T *__restrict__ vals, const T *__restrict__ x, int64_t m, int G, int inc) {
-    LAK_PDL_ENTRY();
+    LAK_PDL_WAIT();
     using Ac = typename Acc<T>::type;
     const int R = blockDim.x / G;
     const int grp = threadIdx.x / G;
@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(kSpmvLongBlock)
 spmv_long_kernel(T *__restrict__ y, const int32_t *__restrict__ rp,
                  const int32_t *__restrict__ ci, const T *__restrict__ vals,
                  const T *__restrict__ x, int64_t m) {
-    LAK_PDL_ENTRY();
+    LAK_PDL_WAIT();
     using Ac = typename Acc<T>::type;
     constexpr int U = 4, rows = 32 / G;
     const int lane = threadIdx.x & 31, lg = lane % G;
@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(512)
 spmv_seg_kernel(T *__restrict__ y, const int32_t *__restrict__ rp,
                 const int32_t *__restrict__ ci, const T *__restrict__ vals,
                 const T *__restrict__ x, int64_t m, int inc) {
-    LAK_PDL_ENTRY();
+    LAK_PDL_WAIT();
     using Ac = typename Acc<T>::type;
     const int warp = threadIdx.x >> 5;
     const int wpb = blockDim.x >> 5;

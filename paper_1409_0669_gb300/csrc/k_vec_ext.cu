@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(512, 2)     // two 512-thread blocks per SM
 axpy_norm2_kernel(T *x, const T *y, const T *z, typename Acc<T>::type alpha, void *out,
                   int64_t n, int64_t head, int64_t nchunks, int inc, unsigned int *counter,
                   double *partials) {
-    LAK_PDL_ENTRY();
+    LAK_PDL_WAIT();
     using A = typename Acc<T>::type;
     A acc[V];
 #pragma unroll
@@ -87,6 +87,7 @@ axpy_norm2_kernel(T *x, const T *y, const T *z, typename Acc<T>::type alpha, voi
             acc[0] = fma_acc(widen(xi), widen(xi), acc[0]);
         }
     }
+    LAK_PDL_TRIGGER();          // not at entry (lak_internal.cuh)
 #pragma unroll
     for (int w = 1; w < V; w <<= 1) {
 #pragma unroll

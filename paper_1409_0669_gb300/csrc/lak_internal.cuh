@@ -77,8 +77,12 @@ inline int access_bytes(int vec, int es) {
 // next grid is scheduled once every block of this one has started, so its
 // launch and block set-up overlap this grid's tail instead of following it).
 // No kernel touches global memory before the wait, so the stream's ordering is
-// unchanged; launch_k launches with the attribute unless LAK_PDL=0.  (The
-// batched GEMV only waits; it lets its dependents launch when it completes.)
+// unchanged; launch_k launches with the attribute unless LAK_PDL=0.  Kernels that only
+// wait (LAK_PDL_WAIT) let their dependents launch at their end, or where they say
+// LAK_PDL_TRIGGER: a dependent of few, equal blocks that starts while SMs of a large
+// grid are still busy gets several of its blocks on the SMs that are free first, and
+// its slowest SM sets its time.  So do the CSR products, the fused update and norm,
+// the GEMV by row sets, the FP64 column-major GEMV and the batched GEMV.
 #define LAK_PDL_WAIT() asm volatile("griddepcontrol.wait;" ::: "memory")
 #define LAK_PDL_TRIGGER() asm volatile("griddepcontrol.launch_dependents;" ::: "memory")
 #define LAK_PDL_ENTRY()    \
