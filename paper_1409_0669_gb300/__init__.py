@@ -23,6 +23,15 @@ import torch
 from . import _native
 from ._native import DTYPES, INCREMENTS, LAYOUTS, OPS, LakCfg, LakError
 
+_lib = _native.load()
+
+try:
+    # direct calls for the common forms (csrc/py_fast.cpp); each returns None where the
+    # Python path has to take the call
+    from . import _fast
+except ImportError:             # built against another torch: the Python paths serve all
+    _fast = None
+
 __all__ = ["vec_copy", "vec_axpy", "vec_axpby", "vec_axpy_norm2", "vec_axpy_norm2_workspace",
            "dense_gemv_trans", "vec_dot", "vec_dot_workspace", "vec_dot_sparse",
            "vec_dot_sparse_workspace", "vec_dot_compensated",
@@ -31,8 +40,6 @@ __all__ = ["vec_copy", "vec_axpy", "vec_axpby", "vec_axpy_norm2", "vec_axpy_norm
            "csr_transpose", "csr_transpose_vals", "vec_gather", "vec_scale_dev", "resolve_cfg", "set_default_cfg",
            "size_bucket", "SIZE_BUCKETS", "Cfg", "set_batch_default_cfg", "probe_fma_f64",
            "LakError", "storage_of", "library_path"]
-
-_lib = _native.load()
 
 _TORCH_TO_STORAGE = {torch.float32: "f32", torch.float64: "f64", torch.bfloat16: "bf16",
                      torch.float16: "f16"}
@@ -141,6 +148,8 @@ def _workspace(nbytes: int, stream_handle: int, device: torch.device) -> torch.T
     if ws is None or ws.numel() < nbytes:
         ws = torch.zeros(max(nbytes, 256), dtype=torch.uint8, device=device)
         _workspaces[key] = ws
+        if _fast is not None:
+            _fast.keep_workspace(device.index, stream_handle, ws)
     return ws
 
 
@@ -229,6 +238,10 @@ def _dot_ws_need(n: int, storage: str, cfg: CfgLike) -> int:
 
 def vec_copy(x: torch.Tensor, y: torch.Tensor, cfg: CfgLike = None, stream=None) -> torch.Tensor:
     """x[:] = y (bit copy)."""
+    if _fast is not None and cfg is None and stream is None:
+        r = _fast.vec_copy(x, y)
+        if r is not None:
+            return r
     s = _same_storage(x, y)
     if x.numel() != y.numel():
         raise ValueError("x and y must have the same length")
@@ -241,6 +254,10 @@ def vec_copy(x: torch.Tensor, y: torch.Tensor, cfg: CfgLike = None, stream=None)
 def vec_axpy(x: torch.Tensor, y: torch.Tensor, z: torch.Tensor, alpha: float,
              cfg: CfgLike = None, stream=None) -> torch.Tensor:
     """x[:] = y + alpha * z."""
+    if _fast is not None and cfg is None and stream is None:
+        r = _fast.vec_axpy(x, y, z, alpha)
+        if r is not None:
+            return r
     s = _same_storage(x, y, z)
     n = x.numel()
     if y.numel() != n or z.numel() != n:
@@ -255,6 +272,10 @@ def vec_axpby(x: torch.Tensor, alpha: float, y: torch.Tensor, beta: float, z: to
               cfg: CfgLike = None, stream=None) -> torch.Tensor:
     """x[:] = alpha*y + beta*z; 1-D views with any (nonzero for x) strides take
     the strided kernel, contiguous ones the vectorised kernel."""
+    if _fast is not None and cfg is None and stream is None:
+        r = _fast.vec_axpby(x, alpha, y, beta, z)
+        if r is not None:
+            return r
     s = _same_storage(x, y, z)
     n = x.numel()
     if y.numel() != n or z.numel() != n:
@@ -279,6 +300,10 @@ def vec_axpy_norm2(x: torch.Tensor, y: torch.Tensor, z: torch.Tensor, alpha: flo
                    out: Optional[torch.Tensor] = None, workspace: Optional[torch.Tensor] = None,
                    cfg: CfgLike = None, stream=None) -> torch.Tensor:
     """x[:] = y + alpha*z and returns <x, x> (one-element device tensor), in one pass."""
+    if _fast is not None and cfg is None and stream is None and workspace is None:
+        r = _fast.vec_axpy_norm2(x, y, z, alpha, out)
+        if r is not None:
+            return r
     s = _same_storage(x, y, z)
     n = x.numel()
     if y.numel() != n or z.numel() != n:
@@ -310,6 +335,10 @@ def vec_dot(x: torch.Tensor, y: torch.Tensor, out: Optional[torch.Tensor] = None
             stream=None) -> torch.Tensor:
     """<x, y> into a one-element device tensor (float32 for FP32/BF16/FP16
     storage, float64 for FP64)."""
+    if _fast is not None and cfg is None and stream is None and workspace is None:
+        r = _fast.vec_dot(x, y, out, False)
+        if r is not None:
+            return r
     s = _same_storage(x, y)
     n = x.numel()
     if y.numel() != n:
@@ -369,6 +398,10 @@ def vec_dot_compensated(x: torch.Tensor, y: torch.Tensor, out: Optional[torch.Te
     """<x, y> for FP32/BF16/FP16 storage with compensated (Dot2) FP32
     accumulation and an FP64 combine; the result is a one-element float64
     device tensor."""
+    if _fast is not None and cfg is None and stream is None and workspace is None:
+        r = _fast.vec_dot_compensated(x, y, out)
+        if r is not None:
+            return r
     s = _same_storage(x, y)
     n = x.numel()
     if y.numel() != n:
@@ -433,6 +466,11 @@ def dense_gemv(A: torch.Tensor, x: torch.Tensor, y: Optional[torch.Tensor] = Non
     """y = alpha * A x + beta * y (y is not read when beta == 0).  A is a 2-D
     tensor (its strides give the layout and lda), or a 1-D buffer with
     explicit m, n, lda and layout ('row' or 'col')."""
+    if _fast is not None and cfg is None and stream is None and workspace is None and m is None and n is None \
+            and lda is None and layout is None:
+        r = _fast.dense_gemv(A, x, y, alpha, beta, False)
+        if r is not None:
+            return r
     s = _same_storage(A, x)
     if A.dim() == 2 and m is None:
         m, n, lda, lay = _matrix_layout(A)
@@ -476,6 +514,10 @@ def dense_gemv_trans(A: torch.Tensor, x: torch.Tensor, y: Optional[torch.Tensor]
                      stream=None) -> torch.Tensor:
     """y = A^T x for a 2-D tensor A (row- or column-major), through the
     dense_gemv_trans entry point."""
+    if _fast is not None and cfg is None and stream is None and workspace is None:
+        r = _fast.dense_gemv(A, x, y, 1.0, 0.0, True)
+        if r is not None:
+            return r
     s = _same_storage(A, x)
     m, n, lda, layout = _matrix_layout(A)
     if x.numel() != m:
@@ -500,6 +542,10 @@ def csr_spmv(row_ptr: torch.Tensor, col_idx: torch.Tensor, vals: torch.Tensor, x
              y: Optional[torch.Tensor] = None, n_cols: Optional[int] = None,
              cfg: CfgLike = None, stream=None) -> torch.Tensor:
     """y = A x for A in CSR form (int32 row_ptr of m+1 entries, int32 col_idx)."""
+    if _fast is not None and cfg is None and stream is None:
+        r = _fast.csr_spmv(row_ptr, col_idx, vals, x, y, n_cols)
+        if r is not None:
+            return r
     s = _same_storage(vals, x)
     if row_ptr.dtype != torch.int32 or col_idx.dtype != torch.int32:
         raise TypeError("row_ptr and col_idx must be int32")
@@ -527,6 +573,10 @@ def csr_spmv(row_ptr: torch.Tensor, col_idx: torch.Tensor, vals: torch.Tensor, x
 def dense_outer(dy: torch.Tensor, x: torch.Tensor, out: Optional[torch.Tensor] = None,
                 stream=None) -> torch.Tensor:
     """dA = dy x^T as an (m, n) row-major tensor."""
+    if _fast is not None and out is None and stream is None:
+        r = _fast.dense_outer(dy, x)
+        if r is not None:
+            return r
     s = _same_storage(dy, x)
     m, n = dy.numel(), x.numel()
     if out is None:
@@ -544,6 +594,10 @@ def csr_sampled_outer(row_ptr: torch.Tensor, col_idx: torch.Tensor, dy: torch.Te
                       x: torch.Tensor, out: Optional[torch.Tensor] = None,
                       stream=None) -> torch.Tensor:
     """dvals[k] = dy[row(k)] * x[col(k)] on the CSR pattern."""
+    if _fast is not None and out is None and stream is None:
+        r = _fast.csr_sampled_outer(row_ptr, col_idx, dy, x)
+        if r is not None:
+            return r
     s = _same_storage(dy, x)
     m = row_ptr.numel() - 1
     nnz = col_idx.numel()
@@ -642,6 +696,10 @@ def vec_scale_dev(v: torch.Tensor, alpha: torch.Tensor, out: Optional[torch.Tens
                   stream=None) -> torch.Tensor:
     """out = alpha * v with alpha a one-element device tensor (float32; float64
     for FP64 storage)."""
+    if _fast is not None and out is None and stream is None:
+        r = _fast.vec_scale_dev(v, alpha)
+        if r is not None:
+            return r
     s = storage_of(v)
     adt = torch.float64 if s == "f64" else torch.float32
     if alpha.dtype != adt or not alpha.is_cuda:

@@ -1,16 +1,21 @@
-"""In-tree build of the CUDA library ``liblak_gb300.so`` for sm_103a.
+"""In-tree build of the CUDA library ``liblak_gb300.so`` for sm_103a and of the
+Python extension ``_fast`` that calls it.
 
 Each translation unit under ``csrc/`` is compiled by nvcc in parallel into
 ``_build/`` and linked (static CUDA runtime) into a shared library beside this
-file.  A rebuild happens only when a source or header is newer than the
-library, unless ``force`` is set.
+file; the extension (``csrc/py_fast.cpp``) is compiled by g++ against the
+installed torch's headers and linked against that library.  A rebuild happens
+only when a source or header is newer than the results, unless ``force`` is
+set.
 """
 from __future__ import annotations
 
 import concurrent.futures
+import importlib.util
 import os
 import shutil
 import subprocess
+import sysconfig
 import tempfile
 
 PKG = os.path.dirname(os.path.abspath(__file__))
@@ -19,6 +24,7 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 OBJDIR = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "liblak_gb300.so")
+FAST = os.path.join(PKG, "_fast" + sysconfig.get_config_var("EXT_SUFFIX"))
 ARCH = "-gencode=arch=compute_103a,code=sm_103a"
 SOURCES = ["lak_api.cu", "k_vec.cu", "k_gemv.cu", "k_gemv_wide.cu", "k_spmv.cu", "k_dot_noalloc.cu", "k_batch.cu", "k_grad.cu", "k_transpose.cu", "k_vec_ext.cu", "k_sell.cu", "k_csr_bin.cu", "k_probe.cu"]
 
@@ -41,15 +47,49 @@ def _deps():
 
 
 def up_to_date() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(FAST):
         return False
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(FAST))
     return all(os.path.getmtime(f) <= t for f in _deps())
 
 
 def compile_flags():
     return [ARCH, "-lineinfo", "-O3", "-std=c++17", "-Xcompiler", "-fPIC",
             "-Xcompiler", "-fvisibility=hidden", "-I", INCLUDE, "-I", CSRC]
+
+
+def torch_dir() -> str:
+    spec = importlib.util.find_spec("torch")
+    if spec is None or not spec.submodule_search_locations:
+        raise RuntimeError("torch not found")
+    return list(spec.submodule_search_locations)[0]
+
+
+def compile_fast() -> str:
+    """Object file of the Python extension."""
+    inc = os.path.join(torch_dir(), "include")
+    cuda = os.path.join(os.path.dirname(os.path.dirname(nvcc_path())), "include")
+    obj = os.path.join(OBJDIR, "py_fast.o")
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-fvisibility=hidden", "-I", INCLUDE, "-I", inc,
+           "-I", os.path.join(inc, "torch", "csrc", "api", "include"), "-I", cuda, "-I",
+           sysconfig.get_paths()["include"], "-c", os.path.join(CSRC, "py_fast.cpp"), "-o", obj]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"g++ failed on py_fast.cpp:\n{r.stderr}")
+    return obj
+
+
+def link_fast(obj: str):
+    lib = os.path.join(torch_dir(), "lib")
+    fd, tmp = tempfile.mkstemp(suffix=".so", dir=PKG)
+    os.close(fd)
+    cmd = ["g++", "-shared", "-o", tmp, obj, "-L", lib, "-lc10", "-lc10_cuda", "-ltorch_cpu",
+           "-ltorch_python", "-L", PKG, "-l:" + os.path.basename(LIB), "-Wl,-rpath,$ORIGIN"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        os.unlink(tmp)
+        raise RuntimeError(f"link of the Python extension failed:\n{r.stderr}")
+    os.replace(tmp, FAST)
 
 
 def build(force: bool = False, verbose: bool = False, ptxas_verbose: bool = False) -> str:
@@ -67,8 +107,10 @@ def build(force: bool = False, verbose: bool = False, ptxas_verbose: bool = Fals
             raise RuntimeError(f"nvcc failed on {src}:\n{r.stderr}")
         return obj, r.stderr
 
-    with concurrent.futures.ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
+    with concurrent.futures.ThreadPoolExecutor(max_workers=len(SOURCES) + 1) as ex:
+        fast = ex.submit(compile_fast)
         results = list(ex.map(one, SOURCES))
+        fast_obj = fast.result()
     if verbose or ptxas_verbose:
         for _, log in results:
             if log:
@@ -81,6 +123,7 @@ def build(force: bool = False, verbose: bool = False, ptxas_verbose: bool = Fals
         os.unlink(tmp)
         raise RuntimeError(f"link failed:\n{r.stderr}")
     os.replace(tmp, LIB)
+    link_fast(fast_obj)
     return LIB
 
 

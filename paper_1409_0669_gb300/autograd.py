@@ -14,8 +14,8 @@ from __future__ import annotations
 
 import torch
 
-from . import (csr_sampled_outer, csr_spmv, csr_transpose, csr_transpose_vals, dense_gemv,
-               dense_outer, vec_dot, vec_gather, vec_scale_dev)
+from . import (_fast, csr_sampled_outer, csr_spmv, csr_transpose, csr_transpose_vals, dense_gemv,
+               dense_gemv_trans, dense_outer, vec_dot, vec_gather, vec_scale_dev)
 
 
 class CsrPattern:
@@ -59,7 +59,7 @@ class _Gemv(torch.autograd.Function):
         if ctx.needs_input_grad[0]:
             dA = dense_outer(dy, x)
         if ctx.needs_input_grad[1]:
-            dx = dense_gemv(A.t(), dy)          # A^T dy: same storage, other layout
+            dx = dense_gemv_trans(A, dy)        # A^T dy: same storage, other layout
         return dA, dx
 
 
@@ -88,12 +88,12 @@ class _Dot(torch.autograd.Function):
     @staticmethod
     def forward(ctx, x, y):
         ctx.save_for_backward(x, y)
-        return vec_dot(x, y).reshape(())
+        s = _fast.vec_dot(x, y, None, True) if _fast is not None else None
+        return vec_dot(x, y).reshape(()) if s is None else s
 
     @staticmethod
     def backward(ctx, ds):
         x, y = ctx.saved_tensors
-        ds = ds.reshape(1).contiguous()
         if ds.dtype != (torch.float64 if x.dtype == torch.float64 else torch.float32):
             ds = ds.to(torch.float64 if x.dtype == torch.float64 else torch.float32)
         dx = vec_scale_dev(y, ds) if ctx.needs_input_grad[0] else None
