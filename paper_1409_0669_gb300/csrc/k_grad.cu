@@ -351,7 +351,7 @@ LAK_API size_t csr_transpose_vals_workspace(int64_t n, int64_t nnz, lak_dtype dt
     if (n < 0 || nnz < 0 || nnz > 0x7fffffffLL || n > 0x7fffffffLL || !valid_dt(dtype)) return 0;
     const size_t least = csr_transpose_workspace(n);
     if (n == 0 || nnz == 0) return least;
-    const size_t w = transpose_workspace(n, nnz, esize(dtype));
+    const size_t w = transpose_workspace(n, nnz);
     return w > least ? w : least;
 }
 
@@ -428,7 +428,7 @@ LAK_API lak_status csr_transpose_vals(int32_t *col_ptr, int32_t *row_idx, int32_
                     workspace ? ws_bytes : (size_t)0);
     if ((uintptr_t)workspace % 256)
         return fail(LAK_EWORKSPACE, "%s: workspace not 256-byte aligned", who);
-    if (n > kTransposeMaxCols) {
+    if (n > kTransposeMaxCols || es == 8) {             // 64-bit values: k_transpose.cu
         const lak_status st = csr_transpose(col_ptr, row_idx, perm, row_ptr, col_idx, m, n, nnz,
                                             workspace, ws_bytes, stream);
         return st != LAK_OK ? st : vec_gather(vals_t, vals, perm, nnz, dtype, stream);

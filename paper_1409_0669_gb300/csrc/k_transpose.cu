@@ -24,9 +24,13 @@
 // the block number, then high half).  Blocks are half an SM, so that one's loads and
 // stores run under the other's ranking.
 //
-// Measured (32 M entries, 2 M columns, FP32 values carried along): 1.03 ms against
-// 4.1 ms for the atomic scatter, the columns' sort and the gather (FP64 values 1.52 ms);
-// three passes of 0.9-1.0 GB each, 0.45 ms at the copy rate.  Blocks of a whole SM
+// Values of 16 and 32 bits travel in the records; 64-bit ones are gathered afterwards
+// (beside the records they cost more than the gather: 3D Laplacian 128^3 666 against
+// 548 us, power law about equal).
+//
+// Measured (32 M entries of a power-law matrix, 2 M columns, FP32 values carried along):
+// 1.03 ms against 3.3 ms for the atomic scatter, the columns' sort and the gather; three
+// passes of 0.9-1.0 GB each, 0.45 ms at the copy rate.  Blocks of a whole SM
 // (1024 threads, tiles of 8192) took 1.42 ms, ten-bit digits in one pass with column
 // blocks of 32 K entries gathered through L2 1.30 ms, per-warp fronts without the
 // exchange 2.1 ms.
@@ -49,7 +53,7 @@ constexpr int kBigWarps = 8;            // warps that work on a column block bey
 
 struct __align__(16) Rec {
     int32_t col, row, k;
-    uint32_t v;                         // 16- or 32-bit value (64-bit ones go beside)
+    uint32_t v;                         // 16- or 32-bit value
 };
 
 // Stable rank of this lane's entry among the entries of digit d that the warp has seen:
@@ -203,29 +207,25 @@ seg_apply_kernel(int32_t *__restrict__ cells, const int32_t *__restrict__ segs, 
     running(cells + b, nb, t0, t1, segs[(int64_t)blockIdx.y * nb + b]);
 }
 
-template <typename E> constexpr size_t move_smem(int nb) {
-    return (size_t)kTile * (16 + (sizeof(E) == 8 ? 8 : 0)) + (size_t)nb * 4 +
-           (size_t)kTileWarps * nb * 2;
+constexpr size_t move_smem(int nb) {
+    return (size_t)kTile * 16 + (size_t)nb * 4 + (size_t)kTileWarps * nb * 2;
 }
 
 // Orders a tile's records by column block in shared memory and stores them as runs.
 // From the CSR arrays, or (CSR false) from the records of an earlier pass.
-// E: the values' type (uint16_t, uint32_t, uint64_t; vals may be null).
+// E: the values' type (uint16_t, uint32_t; vals may be null).
 template <typename E, bool CSR>
 __global__ void __launch_bounds__(kTileThreads, 2)
-part_move_kernel(Rec *__restrict__ out, uint64_t *__restrict__ out64,
-                 const int32_t *__restrict__ rp, const int32_t *__restrict__ ci,
-                 const E *__restrict__ vals, const Rec *__restrict__ in,
-                 const uint64_t *__restrict__ in64, const int32_t *__restrict__ cells,
+part_move_kernel(Rec *__restrict__ out, const int32_t *__restrict__ rp,
+                 const int32_t *__restrict__ ci, const E *__restrict__ vals,
+                 const Rec *__restrict__ in, const int32_t *__restrict__ cells,
                  const int32_t *__restrict__ first, int64_t m, int64_t nnz, int shift, int mask,
                  int nb, int bits) {
     LAK_PDL_ENTRY();
-    constexpr bool WIDE = sizeof(E) == 8;
     constexpr int ITEMS = kItems, TILE = kTile;
     extern __shared__ __align__(16) unsigned char move_raw[];
     Rec *stage = reinterpret_cast<Rec *>(move_raw);
-    uint64_t *stage64 = reinterpret_cast<uint64_t *>(move_raw + (size_t)TILE * 16);
-    int32_t *delta = reinterpret_cast<int32_t *>(move_raw + (size_t)TILE * (WIDE ? 24 : 16));
+    int32_t *delta = reinterpret_cast<int32_t *>(move_raw + (size_t)TILE * 16);
     uint16_t *count = reinterpret_cast<uint16_t *>(delta + nb);        // [warp][nb]
     __shared__ int32_t wtot[kTileWarps];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -241,23 +241,17 @@ part_move_kernel(Rec *__restrict__ out, uint64_t *__restrict__ out64,
     uint32_t where[ITEMS];
     int32_t row[ITEMS];
     Rec rec[ITEMS];
-    uint64_t wide[ITEMS];
 #pragma unroll
     for (int i = 0; i < ITEMS; ++i) {
         const int64_t k = w0 + 32 * i + lane;
         rec[i].col = 0;
         rec[i].v = 0;
-        wide[i] = 0;
         if (k < t1) {
             if constexpr (CSR) {
                 rec[i].col = __ldg(ci + k);
-                if (vals) {
-                    if constexpr (WIDE) wide[i] = __ldg((const unsigned long long *)vals + k);
-                    else rec[i].v = __ldg(vals + k);
-                }
+                if (vals) rec[i].v = __ldg(vals + k);
             } else {
                 ld_raw<16, STREAM>(&rec[i], in + k);
-                if (WIDE && in64) wide[i] = in64[k];
             }
         }
     }
@@ -347,7 +341,6 @@ part_move_kernel(Rec *__restrict__ out, uint64_t *__restrict__ out64,
         }
         const int place = (int)mine[where[i] >> 16] + (int)(where[i] & 0xffffu);
         stage[place] = rec[i];
-        if (WIDE) stage64[place] = wide[i];
     }
     __syncthreads();
 
@@ -357,7 +350,6 @@ part_move_kernel(Rec *__restrict__ out, uint64_t *__restrict__ out64,
         const Rec rec = stage[q];
         const int32_t pos = delta[(rec.col >> shift) & mask] + q;
         st_raw<16>(out + pos, &rec);
-        if (WIDE && out64) out64[pos] = stage64[q];
     }
 }
 
@@ -377,13 +369,12 @@ bounds_kernel(int32_t *__restrict__ bounds, const Rec *__restrict__ recs, int64_
     bounds[b] = (int32_t)lo;
 }
 
-// Records of a column block that are ordered on chip: 12 bytes each (16 with 64-bit
-// values) beside the counters.
-template <typename E> constexpr int kOrderItems = sizeof(E) == 8 ? 10 : 12;
-template <typename E> constexpr int kOrderCap = 32 * kOrderWarps * kOrderItems<E>;
+// Records of a column block that are ordered on chip, 12 bytes each beside the counters
+constexpr int kOrderItems = 12;
+constexpr int kOrderCap = 32 * kOrderWarps * kOrderItems;
 
-template <typename E> constexpr size_t order_smem(int s) {
-    return (size_t)kOrderWarps * (1 << s) * 2 + 16 + (size_t)kOrderCap<E> * (8 + (sizeof(E) == 8 ? 8 : 4));
+constexpr size_t order_smem(int s) {
+    return (size_t)kOrderWarps * (1 << s) * 2 + 16 + (size_t)kOrderCap * 12;
 }
 
 // One block per column block: orders its records by column and writes the CSC arrays.
@@ -395,11 +386,9 @@ template <typename E>
 __global__ void __launch_bounds__(32 * kOrderWarps, 2)
 order_kernel(int32_t *__restrict__ col_ptr, int32_t *__restrict__ row_idx,
              int32_t *__restrict__ perm, E *__restrict__ vals_t, const Rec *__restrict__ recs,
-             const uint64_t *__restrict__ recs64, const int32_t *__restrict__ bounds, int64_t n,
-             int64_t nnz, int s) {
+             const int32_t *__restrict__ bounds, int64_t n, int64_t nnz, int s) {
     LAK_PDL_ENTRY();
-    constexpr bool WIDE = sizeof(E) == 8;
-    constexpr int ITEMS = kOrderItems<E>, CAP = kOrderCap<E>;
+    constexpr int ITEMS = kOrderItems, CAP = kOrderCap;
     extern __shared__ __align__(16) unsigned char order_raw[];
     __shared__ int32_t wtot[kOrderWarps];
     __shared__ int64_t range[2];
@@ -487,10 +476,7 @@ order_kernel(int32_t *__restrict__ col_ptr, int32_t *__restrict__ row_idx,
     if (blockIdx.x == gridDim.x - 1 && tid == 0) col_ptr[n] = (int32_t)nnz;
     __syncthreads();
     if (small) {
-        // 64-bit values first (aligned), then rows, positions and narrow values
-        const size_t at0 = ((size_t)kOrderWarps * nc * 2 + 15) / 16 * 16;
-        uint64_t *s64 = reinterpret_cast<uint64_t *>(order_raw + at0);
-        int32_t *srow = reinterpret_cast<int32_t *>(order_raw + at0 + (WIDE ? 8 * CAP : 0));
+        int32_t *srow = reinterpret_cast<int32_t *>(order_raw + ((size_t)kOrderWarps * nc * 2 + 15) / 16 * 16);
         int32_t *sk = srow + CAP;
         uint32_t *sv = reinterpret_cast<uint32_t *>(sk + CAP);
 #pragma unroll
@@ -502,19 +488,13 @@ order_kernel(int32_t *__restrict__ col_ptr, int32_t *__restrict__ row_idx,
             const int place = (int)mine16[where[i] >> 16] + (int)(where[i] & 0xffffu);
             srow[place] = r.row;
             sk[place] = r.k;
-            if (vals_t) {
-                if constexpr (WIDE) s64[place] = recs64[b0 + k];
-                else sv[place] = r.v;
-            }
+            sv[place] = r.v;
         }
         __syncthreads();
         for (int q = tid; q < (int)len; q += 32 * kOrderWarps) {
             row_idx[b0 + q] = srow[q];
             perm[b0 + q] = sk[q];
-            if (vals_t) {
-                if constexpr (WIDE) vals_t[b0 + q] = s64[q];
-                else vals_t[b0 + q] = (E)sv[q];
-            }
+            if (vals_t) vals_t[b0 + q] = (E)sv[q];
         }
         return;
     }
@@ -527,10 +507,7 @@ order_kernel(int32_t *__restrict__ col_ptr, int32_t *__restrict__ row_idx,
         if (valid) {
             row_idx[b0 + pos] = r.row;
             perm[b0 + pos] = r.k;
-            if (vals_t) {
-                if constexpr (WIDE) vals_t[b0 + pos] = recs64[b0 + k];
-                else vals_t[b0 + pos] = (E)r.v;
-            }
+            if (vals_t) vals_t[b0 + pos] = (E)r.v;
         }
     }
 }
@@ -541,17 +518,17 @@ struct Plan {
     int passes;             // partition passes (1 or 2)
     int bits[2], nb[2];     // of each pass: bits of its digit, number of digits
     int64_t tiles, nseg;
-    size_t off_cells, off_segs, off_starts, off_first, off_rec[2], off_wide[2], bytes;
+    size_t off_cells, off_segs, off_starts, off_first, off_rec[2], bytes;
 };
 
 size_t up256(size_t b) { return (b + 255) / 256 * 256; }
 
-Plan make_plan(int64_t n, int64_t nnz, int vbytes) {
+Plan make_plan(int64_t n, int64_t nnz) {
     Plan p{};
     // columns per block: as many as leave the mean column block three quarters of what
     // the ordering kernel holds on chip, and two blocks per SM or more where they would
     // still have 2048 entries
-    const int64_t mean = (vbytes == 8 ? kOrderCap<uint64_t> : kOrderCap<uint32_t>) / 4 * 3;
+    const int64_t mean = kOrderCap / 4 * 3;
     int s = kMaxColBits;
     auto blocks = [&](int bits) { return ((n - 1) >> bits) + 1; };
     while (s > 0 && blocks(s - 1) <= (int64_t)kMaxBlocks * kMaxBlocks &&
@@ -581,8 +558,6 @@ Plan make_plan(int64_t n, int64_t nnz, int vbytes) {
     for (int i = 0; i < p.passes; ++i) {
         p.off_rec[i] = at;
         at += up256((size_t)nnz * 16);
-        p.off_wide[i] = at;
-        if (vbytes == 8) at += up256((size_t)nnz * 8);
     }
     p.bytes = at;
     return p;
@@ -596,16 +571,11 @@ lak_status run(const Plan &p, int32_t *col_ptr, int32_t *row_idx, int32_t *perm,
     int32_t *segs = reinterpret_cast<int32_t *>(w + p.off_segs);
     int32_t *starts = reinterpret_cast<int32_t *>(w + p.off_starts);
     int32_t *first = reinterpret_cast<int32_t *>(w + p.off_first);
-    const bool wide = sizeof(E) == 8 && vals != nullptr;
     Rec *rec[2];
-    uint64_t *r64[2];
-    for (int i = 0; i < 2; ++i) {
-        const int j = i < p.passes ? i : 0;
-        rec[i] = reinterpret_cast<Rec *>(w + p.off_rec[j]);
-        r64[i] = wide ? reinterpret_cast<uint64_t *>(w + p.off_wide[j]) : nullptr;
-    }
-    const int move_most = (int)move_smem<E>(kMaxBlocks);
-    const int order_most = (int)order_smem<E>(kMaxColBits);
+    for (int i = 0; i < 2; ++i)
+        rec[i] = reinterpret_cast<Rec *>(w + p.off_rec[i < p.passes ? i : 0]);
+    const int move_most = (int)move_smem(kMaxBlocks);
+    const int order_most = (int)order_smem(kMaxColBits);
     cudaError_t e = cudaFuncSetAttribute(part_move_kernel<E, true>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, move_most);
     if (e == cudaSuccess)
@@ -631,48 +601,40 @@ lak_status run(const Plan &p, int32_t *col_ptr, int32_t *row_idx, int32_t *perm,
         launch_k(seg_scan_kernel, 1, 1024, 0, st, segs, starts, p.nseg, nb);
         launch_k(seg_apply_kernel, sgrid, 256, 0, st, cells, (const int32_t *)segs, p.tiles, nb);
         if (i == 0)
-            launch_k(part_move_kernel<E, true>, (unsigned)p.tiles, kTileThreads, move_smem<E>(nb),
-                     st, rec[0], r64[0], rp, ci, vals, (const Rec *)nullptr,
-                     (const uint64_t *)nullptr, (const int32_t *)cells,
+            launch_k(part_move_kernel<E, true>, (unsigned)p.tiles, kTileThreads, move_smem(nb),
+                     st, rec[0], rp, ci, vals, (const Rec *)nullptr, (const int32_t *)cells,
                      (const int32_t *)first, m, nnz, shift, mask, nb, bits);
         else
-            launch_k(part_move_kernel<E, false>, (unsigned)p.tiles, kTileThreads, move_smem<E>(nb),
-                     st, rec[1], r64[1], rp, ci, (const E *)nullptr, (const Rec *)rec[0],
-                     (const uint64_t *)r64[0], (const int32_t *)cells,
+            launch_k(part_move_kernel<E, false>, (unsigned)p.tiles, kTileThreads, move_smem(nb),
+                     st, rec[1], rp, ci, (const E *)nullptr, (const Rec *)rec[0],
+                     (const int32_t *)cells,
                      (const int32_t *)first, m, nnz, shift, mask, nb, bits);
     }
     if (p.passes == 2)
         launch_k(bounds_kernel, (unsigned)ceil_div(p.blocks, 128), 128, 0, st, starts,
                  (const Rec *)rec[1], nnz, p.blocks, p.s);
-    launch_k(order_kernel<E>, (unsigned)p.blocks, 32 * kOrderWarps, order_smem<E>(p.s), st,
+    launch_k(order_kernel<E>, (unsigned)p.blocks, 32 * kOrderWarps, order_smem(p.s), st,
              col_ptr, row_idx, perm, vals ? vals_t : (E *)nullptr, (const Rec *)rec[p.passes - 1],
-             (const uint64_t *)r64[p.passes - 1],
              (const int32_t *)starts, n, nnz, p.s);
     return check_launch("csr_transpose");
 }
 
 }  // namespace
 
-size_t transpose_workspace(int64_t n, int64_t nnz, int vbytes) {
-    return n < 1 || nnz < 1 || n > kTransposeMaxCols ? 0 : make_plan(n, nnz, vbytes).bytes;
+size_t transpose_workspace(int64_t n, int64_t nnz) {
+    return n < 1 || nnz < 1 || n > kTransposeMaxCols ? 0 : make_plan(n, nnz).bytes;
 }
 
 lak_status launch_transpose(int32_t *col_ptr, int32_t *row_idx, int32_t *perm, void *vals_t,
                             const int32_t *rp, const int32_t *ci, const void *vals, int64_t m,
                             int64_t n, int64_t nnz, int vbytes, void *ws, cudaStream_t s) {
-    const Plan p = make_plan(n, nnz, vbytes);
+    const Plan p = make_plan(n, nnz);
     char *w = static_cast<char *>(ws);
-    switch (vbytes) {
-    case 2:
+    if (vbytes == 2)
         return run<uint16_t>(p, col_ptr, row_idx, perm, (uint16_t *)vals_t, rp, ci,
                              (const uint16_t *)vals, m, n, nnz, w, s);
-    case 8:
-        return run<uint64_t>(p, col_ptr, row_idx, perm, (uint64_t *)vals_t, rp, ci,
-                             (const uint64_t *)vals, m, n, nnz, w, s);
-    default:
-        return run<uint32_t>(p, col_ptr, row_idx, perm, (uint32_t *)vals_t, rp, ci,
-                             (const uint32_t *)vals, m, n, nnz, w, s);
-    }
+    return run<uint32_t>(p, col_ptr, row_idx, perm, (uint32_t *)vals_t, rp, ci,
+                         (const uint32_t *)vals, m, n, nnz, w, s);
 }
 
 }  // namespace lak
