@@ -483,6 +483,41 @@ bool use_gemv_tall(lak_dtype dt, int64_t m, int64_t n, const lak_cfg *cfg) {
                          cfg);
 }
 
+// Column-major products with columns off 16 bytes (gemv_col_off_kernel): the column
+// splits, 0 where the tile-per-block kernel keeps the call.  The lines lie where both
+// were timed (us, L2 cold, tile-per-block -> this):
+//   FP32 from 1 MiB on, six blocks per SM: 1001^2 9.5 -> 7.5, 3001 x 5000 39 -> 16,
+//     7999 x 8000 117 -> 49, 16383 x 16384 541 -> 195; 301 x 300 3.8 -> 4.5
+//   16 bits from 2000 rows on: BF16 3001 x 5000 26 -> 15, 7999 x 8000 74 -> 33; 1001^2
+//     6.6 -> 7.8
+//   FP64 from 2000 rows and 700 columns up to 512 MiB, eight blocks per SM: 3001 x 5000
+//     55 -> 40, 7999 x 8000 211 -> 139; 16383 x 500 20 -> 23, 16383 x 16384 554 -> 568;
+//     and where the tiles alone fill the GPU (1216): 100003 x 200 55 -> 44
+// Eight columns per warp and split at least: the last block adds the splits one by one.
+int plan_gemv_col_off(lak_dtype dt, int64_t m, int64_t n, const lak_cfg *cfg) {
+    const int es = esize(dt), v = 16 / es;
+    const int64_t bytes = op_bytes(LAK_OP_GEMV_COL, dt, m, n, 0);
+    const int bucket = bucket_of(bytes);
+    if (bytes < (1 << 20) || m < (es == 4 ? 8 * v : 2000) || n < 8) return 0;
+    const int64_t tiles = ceil_div(m, 31LL * v);
+    if (es == 8 && tiles < 1216 && (n < 700 || bucket > 2)) return 0;
+    if (!builtin_shape(LAK_OP_GEMV_COL, dt, bucket, cfg)) return 0;
+    const DeviceInfo *di = device_info();
+    if (!di) return 0;
+    const int64_t per_sm = es == 8 || (es == 2 && bucket == 3) ? 8 : es == 4 ? 6 : 4;
+    int64_t splits = per_sm * di->sms / tiles;
+    const int64_t most = n / (8 * (kGemvOffBlock / 32));
+    if (splits > most) splits = most;
+    if (splits > 65535) splits = 65535;
+    if (tiles > LAK_WS_COUNTER_BYTES / 4) splits = 1;
+    return splits < 1 ? 1 : (int)splits;
+}
+
+size_t col_off_ws_bytes(lak_dtype dt, int64_t m, int splits) {
+    if (splits < 2) return 0;
+    return (size_t)LAK_WS_COUNTER_BYTES + (size_t)splits * (size_t)m * (dt == LAK_F64 ? 8 : 4);
+}
+
 struct ColPlan {
     Launch L;
     int splits;
@@ -770,6 +805,14 @@ LAK_API lak_status lak_resolve_cfg(lak_op op, lak_dtype dtype, int64_t m, int64_
                        LAK_INC_GLOBAL};
             break;
         }
+        if ((m * esize(dtype)) % 16) {
+            const int splits = plan_gemv_col_off(dtype, m, n, cfg);
+            if (splits > 0) {
+                const int v = 16 / esize(dtype);
+                L = Launch{kGemvOffBlock, (int)(ceil_div(m, 31LL * v) * splits), v, LAK_INC_GLOBAL};
+                break;
+            }
+        }
         ColPlan p;
         st = plan_gemv_col(dtype, m, n, m, cfg, nullptr, &p);
         L = p.L;
@@ -964,7 +1007,7 @@ LAK_API size_t dense_gemv_workspace(int64_t m, int64_t n, lak_layout layout, lak
                              dtype, m);
     // the widest vec the call could pick gives the fewest tiles; narrower vecs
     // (forced by alignment) only add tiles, so size for vec = 1 as well
-    size_t best = 0;
+    size_t best = col_off_ws_bytes(dtype, m, plan_gemv_col_off(dtype, m, n, cfg));
     const int bucket = bucket_of(op_bytes(LAK_OP_GEMV_COL, dtype, m, n, 0));
     lak_cfg c = base_cfg(LAK_OP_GEMV_COL, dtype, bucket, cfg);
     const int want = c.vec ? c.vec : builtin_default(LAK_OP_GEMV_COL, dtype, bucket).vec;
@@ -1016,6 +1059,13 @@ lak_status gemv_impl(const char *who, void *y, const void *A, const void *x, int
     }
     if (use_gemv_tall(dtype, m, n, cfg))
         return launch_gemv_tall(dtype, y, A, x, m, n, lda, alpha, beta, s);
+    if ((lda * es) % 16 || (uintptr_t)A % 16) {
+        const int splits = plan_gemv_col_off(dtype, m, n, cfg);
+        const size_t need = col_off_ws_bytes(dtype, m, splits);
+        if (splits > 0 &&
+            (need == 0 || (workspace && ws_bytes >= need && (uintptr_t)workspace % 256 == 0)))
+            return launch_gemv_col_off(dtype, y, A, x, m, n, lda, splits, workspace, alpha, beta, s);
+    }
     ColPlan p;
     st = plan_gemv_col(dtype, m, n, lda, cfg, A, &p);
     if (st != LAK_OK) return st;

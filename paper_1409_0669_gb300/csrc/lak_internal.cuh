@@ -172,6 +172,11 @@ lak_status launch_gemv_rows(lak_dtype dt, void *y, const void *A, const void *x,
 constexpr int kGemvTallBlock = 256;
 lak_status launch_gemv_tall(lak_dtype dt, void *y, const void *A, const void *x, int64_t m,
                             int64_t n, int64_t lda, double alpha, double beta, cudaStream_t s);
+// Column-major product whose columns start off 16 bytes; splits > 1 as above.
+constexpr int kGemvOffBlock = 256;
+lak_status launch_gemv_col_off(lak_dtype dt, void *y, const void *A, const void *x, int64_t m,
+                               int64_t n, int64_t lda, int splits, void *ws, double alpha,
+                               double beta, cudaStream_t s);
 // Long rows: `group` lanes per row (4, 8, 16 or 32).
 constexpr int kSpmvLongBlock = 128;
 lak_status launch_spmv_long(lak_dtype dt, void *y, const int32_t *rp, const int32_t *ci,

@@ -1,7 +1,8 @@
 """GPU parity of the dense products taken by sets of rows (few long rows, rows that
-start at other offsets than x) and by a thread per rows (column-major, very many
-rows), against the FP64 oracle: remainders of the 16-byte packs, every offset of A
-and x, the last incomplete set, column splits, alpha / beta."""
+start at other offsets than x), by a thread per rows (column-major, very many rows)
+and by windows shifted per column (column-major, columns off 16 bytes), against the
+FP64 oracle: remainders of the 16-byte packs, every offset of A and x, the last
+incomplete set, column splits, alpha / beta."""
 import ctypes
 
 import numpy as np
@@ -106,6 +107,39 @@ def test_row_sets_carry_nan_and_inf():
     A[1, 17], A[2, n - 1] = float("inf"), float("nan")
     y = lak().dense_gemv(A, x)
     assert y[0] == n and y[1] == float("inf") and torch.isnan(y[2]) and y[3] == n
+
+
+COL_SHAPES = {"f32": [(33, 9001), (1001, 1003), (2047, 300)], "f64": [(2001, 703), (3000, 901)],
+              "bf16": [(2001, 301), (2303, 777)], "f16": [(2001, 301), (2303, 777)]}
+
+
+@pytest.mark.parametrize("storage", STORAGES)
+@pytest.mark.parametrize("shape", [0, 1, 2])
+@pytest.mark.parametrize("ka,pad", [(0, 0), (0, 1), (1, 0), (1, 3), (3, 2), (5, 7), (1, 8)])
+def test_columns_off_alignment(storage, shape, ka, pad):
+    """Every offset of the first column and every period of the following ones; the
+    last rows' window past the matrix; columns split over blocks."""
+    shapes = COL_SHAPES[storage]
+    m, n = shapes[shape % len(shapes)]
+    if shape == 1:
+        run_case(storage, "col", m, n, pad, ka, 2, alpha=-0.5, beta=2.0)
+    else:
+        run_case(storage, "col", m, n, pad, ka, 0)
+
+
+def test_columns_off_alignment_repeat_and_small_workspace():
+    """Split columns: bit-equal over calls; a workspace too small for the splits falls
+    back to the other kernel's needs, and is refused below those as before."""
+    lk = lak()
+    m, n = 3001, 5000
+    A = synth.normal(m * n, 1, "f32").cuda()
+    x = synth.uniform(n, 2, "f32").cuda()
+    y = lk.dense_gemv(A, x, m=m, n=n, lda=m, layout="col")
+    for _ in range(5):
+        assert torch.equal(lk.dense_gemv(A, x, m=m, n=n, lda=m, layout="col"), y)
+    with pytest.raises(lk.LakError, match="LAK_EWORKSPACE"):
+        lk.dense_gemv(A, x, m=m, n=n, lda=m, layout="col",
+                      workspace=torch.zeros(256, dtype=torch.uint8, device="cuda"))
 
 
 @pytest.mark.parametrize("storage", STORAGES)
