@@ -532,7 +532,9 @@ LAK_API lak_status vec_scale_dev(void *out, const void *v, const void *alpha, in
  * for F32/BF16/F16, double for F64), LAK_OP_GEMV_ROW (lak_gemv_desc, row-major
  * instances), LAK_OP_SPMV (lak_csr_desc, warp-segmented rows; its warps take
  * 32-row blocks in order from a ticket counter in the workspace, so cfg.increment
- * does not apply to it).  The dot and CSR batches keep counters in the
+ * does not apply to it; plans without a cfg give FP32 and 16-bit instances whose x
+ * fits in shared memory to a second kernel of the same run, which reads all n
+ * values of x).  The dot and CSR batches keep counters in the
  * workspace: one run of a batch at a time per workspace.  Per instance
  * the results equal those of the single-instance calls up to the order of
  * floating-point summation (axpy: identical).  The dot keeps at most

@@ -145,6 +145,8 @@ def gemv_batch(As, xs, ys, cfg=None) -> Batch:
 def spmv_batch(csrs, xs, ys, cfg=None) -> Batch:
     """y_i = A_i x_i for CSR matrices given as (row_ptr, col_idx, vals, n_cols)."""
     s = _storage([c[2] for c in csrs] + list(xs) + list(ys))
-    descs = [CsrDesc(_ptr(y), _ptr(rp), _ptr(ci), _ptr(v), _ptr(x), rp.numel() - 1, int(ncols),
-                     v.numel()) for (rp, ci, v, ncols), x, y in zip(csrs, xs, ys)]
+    # n is the length of x, which may be read whole
+    descs = [CsrDesc(_ptr(y), _ptr(rp), _ptr(ci), _ptr(v), _ptr(x), rp.numel() - 1,
+                     x.numel() if int(ncols) >= 0 else int(ncols), v.numel())
+             for (rp, ci, v, ncols), x, y in zip(csrs, xs, ys)]
     return Batch("spmv", s, descs, cfg, keep=(csrs, xs, ys))

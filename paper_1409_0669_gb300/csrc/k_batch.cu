@@ -35,6 +35,8 @@ struct BatchHead {
     int32_t block;
     int32_t inc;
     int32_t pad;
+    int64_t main_units;      // CSR: units of the instances whose x is not staged,
+    int64_t staged_units;    // units of those whose x is
 };
 
 struct AxpyItem {
@@ -69,8 +71,38 @@ struct CsrItem {
     lak_csr_desc d;
     int64_t rows_per_unit;   // a multiple of the block's rows (32 per warp)
     int32_t vec_ok;
-    int32_t pad;
+    int32_t stage_rows;      // rows of a unit of the staged kernel; 0: not staged
 };
+
+// CSR instances (FP32 and 16-bit storage) whose x fits in one SM's shared memory are taken
+// by spmv_staged_kernel, in plans with the default shape.  spmv_batch_kernel is bound by
+// its gathers through L1 (one lane per clock and SM: 262 G entries/s) and, on short rows,
+// by the walk over their ends; shared memory serves about nine random lanes per clock.
+// Measured in G entries/s, spmv_batch_kernel against the staged one:
+//   1000 x 20000 rows of 5..64, random columns   FP32 267 -> 438   BF16 303 -> 471
+//   the same, columns within 64 of the diagonal  FP32 369 -> 447   BF16 427 -> 497
+//   300 x 30000 rows of 150..250                 FP32 301 -> 513   BF16 394 -> 563
+//   4096 x 4000 rows of 8..10                    FP32 142 -> 280   BF16 163 -> 297
+//   2000 x 20000 rows of 2                       FP32  53 ->  81   BF16  57 ->  82
+// 1024 instances of 1000..200000 rows of 5..64: FP32 5076 -> 4640 us (26 % of the rows
+// staged), BF16 4533 -> 3741 us (51 %).  FP32 rows of fewer than 16 entries stay with
+// spmv_batch_kernel all the same: the staged kernel rounds a product before it adds it,
+// which costs 1 % of accuracy at 9 entries and 17 % at 2 (from 16 on its shorter chains
+// more than make up for it; products of 16-bit values are exact in FP32).  FP64 stays
+// there too: one multiplication and one addition per entry in place of an FMA, the latter
+// with few lanes at work, made it 1.3 to 3.1 times slower.  Instances of fewer than
+// kStageMinEntries do not pay for looking up their unit (16000 of 5000 entries: 499 ->
+// 535 us), and fewer than kStageMinUnits units leave SMs idle at the end.
+constexpr int kStageThreads = 768;
+constexpr int kStageBlock = 16;                       // rows that a warp takes at a time
+constexpr int kStageQuads = 2;                        // 4 entries each, per lane and step
+constexpr int kStageStep = 128 * kStageQuads;         // entries of a warp's step
+constexpr int kStageLong = 96;                        // a row's part that the whole warp sums
+constexpr int64_t kStageEntries = 131072;             // of a unit, about
+constexpr int64_t kStageMinEntries = 32768;           // of an instance
+constexpr int64_t kStageMinUnits = 152 * 4;
+constexpr int64_t kStageBytes = 200 * 1024;           // for x
+constexpr int kStageSmem = (int)kStageBytes + kStageThreads / 32 * kStageStep * 4;
 
 constexpr size_t kHeadBytes = 64;
 static_assert(sizeof(BatchHead) <= kHeadBytes, "batch header");
@@ -86,6 +118,11 @@ size_t item_size(lak_op op) {
     case LAK_OP_SPMV: return sizeof(CsrItem);
     default: return 0;
     }
+}
+
+// The table without the CSR batch's two further prefixes (16-byte multiple)
+size_t base_bytes(lak_op op, int64_t count) {
+    return (items_offset(count) + item_size(op) * (size_t)count + 15) / 16 * 16;
 }
 
 int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
@@ -494,7 +531,7 @@ spmv_batch_kernel(const BatchHead *__restrict__ head, const int64_t *__restrict_
     using Ac = typename Acc<T>::type;
     __shared__ uint32_t rs_all[16][33];
     __shared__ Ac racc_all[16][32];
-    const int64_t count = head->count, total = head->total_units;
+    const int64_t count = head->count, total = head->main_units;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
     unsigned int *left = reinterpret_cast<unsigned int *>(sched + 1);
     unsigned long long next = 0;
@@ -533,7 +570,236 @@ spmv_batch_kernel(const BatchHead *__restrict__ head, const int64_t *__restrict_
     }
 }
 
+// What a block of the staged kernel needs to know of its unit
+struct StagedUnit {
+    const int32_t *rp, *ci;
+    const void *vals, *x;
+    void *y;
+    int64_t m, n;
+    uint32_t nnz;
+    int32_t nb, inst;                  // past the last row block; -1: no more units
+    unsigned int block;                // next row block to take
+};
+
+template <typename T>
+struct StagedStep {
+    int32_t col[kStageQuads][4];
+    T val[kStageQuads][4];
+};
+
+// Columns and values of a step that starts at c (a multiple of 4) in a block that ends at E
+template <typename T>
+__device__ __forceinline__ void staged_load(StagedStep<T> &st, const StagedUnit &un, uint32_t c,
+                                            uint32_t E) {
+    const int32_t *ci = un.ci;
+    const T *vals = static_cast<const T *>(un.vals);
+    const uint32_t nnz = un.nnz;
+#pragma unroll
+    for (int q = 0; q < kStageQuads; ++q) {
+        const uint32_t kq = c + q * 128 + (threadIdx.x & 31) * 4;
+        if (kq < E && kq + 4 <= nnz) {                     // past E: the next rows' entries
+            ld_raw<16, CACHED>(&st.col[q], ci + kq);
+            ld_raw<4 * (int)sizeof(T), CACHED>(&st.val[q], vals + kq);
+        } else {
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const bool in = kq + t < E;
+                st.col[q][t] = in ? __ldg(ci + kq + t) : 0;
+                st.val[q][t] = in ? vals[kq + t] : T(0);
+            }
+        }
+    }
+}
+
+// A warp's share of a unit, blocks of kStageBlock rows taken one by one: the products of
+// kStageStep entries at a time go to `buf`; two lanes then sum the part of a row that lies
+// there, in four chains each (the whole warp, where that part is longer than kStageLong).
+// The next step's columns and values, of the next block after the last, are in flight
+// while a step's x is gathered and while rows are summed.  All 32 lanes call it.
+template <typename T>
+__device__ __forceinline__ void staged_unit(StagedUnit &un, const T *xs, float *buf) {
+    const int lane = threadIdx.x & 31;
+    const int64_t m = un.m;
+    const uint32_t xlast = (uint32_t)un.n - 1;
+    auto take = [&]() {
+        unsigned int b = 0;
+        if (lane == 0) b = atomicAdd(&un.block, 1u);
+        return __shfl_sync(0xffffffffu, b, 0);
+    };
+    auto bounds = [&](unsigned int b, uint32_t &k0, uint32_t &k1) {
+        const int64_t row = (int64_t)b * kStageBlock + (lane >> 1);
+        k0 = (uint32_t)__ldg(un.rp + (row < m ? row : m));
+        k1 = (uint32_t)__ldg(un.rp + (row < m ? row + 1 : m));
+    };
+    unsigned int b = take();
+    if (b >= (unsigned int)un.nb) return;
+    uint32_t k0, k1;
+    bounds(b, k0, k1);
+    uint32_t E = __shfl_sync(0xffffffffu, k1, 31), c = __shfl_sync(0xffffffffu, k0, 0) & ~3u;
+    StagedStep<T> st;
+    staged_load(st, un, c, E);
+    for (;;) {
+        const unsigned int b2 = take();
+        const bool more = b2 < (unsigned int)un.nb;
+        uint32_t n0 = 0, n1 = 0;
+        if (more) bounds(b2, n0, n1);
+        float acc = 0.0f;
+        bool last;
+        do {                                               // warp-uniform
+            const uint32_t c0 = c;
+            StagedStep<T> nx;
+            const uint32_t c2 = c + kStageStep;
+            last = c2 >= E;
+            if (!last) staged_load(nx, un, c2, E);
+            else if (more)
+                staged_load(nx, un, __shfl_sync(0xffffffffu, n0, 0) & ~3u,
+                            __shfl_sync(0xffffffffu, n1, 31));
+            T xv[kStageQuads][4];
+#pragma unroll
+            for (int q = 0; q < kStageQuads; ++q)
+#pragma unroll
+                for (int t = 0; t < 4; ++t) {
+                    // entries before the block's first may lie before row_ptr[0]: in bounds
+                    // of x all the same
+                    const uint32_t col = (uint32_t)st.col[q][t];
+                    xv[q][t] = xs[col < xlast ? col : xlast];
+                }
+#pragma unroll
+            for (int q = 0; q < kStageQuads; ++q) {
+                float4 p;
+                p.x = widen(st.val[q][0]) * widen(xv[q][0]);
+                p.y = widen(st.val[q][1]) * widen(xv[q][1]);
+                p.z = widen(st.val[q][2]) * widen(xv[q][2]);
+                p.w = widen(st.val[q][3]) * widen(xv[q][3]);
+                *reinterpret_cast<float4 *>(buf + q * 128 + lane * 4) = p;
+            }
+            st = nx;
+            c = c2;
+            __syncwarp();
+            const uint32_t lo = k0 > c0 ? k0 - c0 : 0;
+            const uint32_t hi = k1 <= c0 ? 0 : k1 - c0 < kStageStep ? k1 - c0 : kStageStep;
+            int n = hi > lo ? (int)(hi - lo) : 0;
+            unsigned lng = __ballot_sync(0xffffffffu, n > kStageLong) & 0x55555555u;
+            if (n > kStageLong) n = 0;
+            for (; lng; lng &= lng - 1) {
+                const int src = __ffs((int)lng) - 1;
+                const uint32_t l = __shfl_sync(0xffffffffu, lo, src);
+                const uint32_t h = __shfl_sync(0xffffffffu, hi, src);
+                float part = 0.0f;
+#pragma unroll 4
+                for (uint32_t k = l + lane; k < h; k += 32) part += buf[k];
+                part = group_sum(part, 32);
+                if (lane == src) acc += part;
+            }
+            const int half = (n + 1) / 2;
+            const float *p = buf + lo + (lane & 1 ? half : 0);
+            n = lane & 1 ? n - half : half;
+            float a0 = 0.0f, a1 = 0.0f, a2 = 0.0f, a3 = 0.0f;
+            for (; n >= 4; n -= 4, p += 4) {
+                a0 += p[0];
+                a1 += p[1];
+                a2 += p[2];
+                a3 += p[3];
+            }
+            if (n > 0) a0 += p[0];
+            if (n > 1) a1 += p[1];
+            if (n > 2) a2 += p[2];
+            acc += (a0 + a1) + (a2 + a3);
+            __syncwarp();
+        } while (!last);
+        acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+        const int64_t row = (int64_t)b * kStageBlock + (lane >> 1);
+        if ((lane & 1) == 0 && row < m) static_cast<T *>(un.y)[row] = narrow<T>(acc);
+        if (!more) return;
+        b = b2;
+        k0 = n0;
+        k1 = n1;
+        E = __shfl_sync(0xffffffffu, k1, 31);
+        c = __shfl_sync(0xffffffffu, k0, 0) & ~3u;
+    }
+}
+
+// The staged instances (32- and 16-bit storage): one block per SM takes units from a
+// ticket counter, brings the unit's x into shared memory, and its warps take the unit's
+// row blocks one by one.  Thread 0 looks the next unit up meanwhile.  The last block to
+// leave resets the counters.  24 warps of 80 registers and a step of 256 entries: longer
+// steps (512, 768) ran the same rows up to 10 % faster but left less room for x.
+template <typename T>
+__global__ void __launch_bounds__(kStageThreads, 1)
+spmv_staged_kernel(const BatchHead *__restrict__ head, const int64_t *__restrict__ offs,
+                   const CsrItem *__restrict__ items, unsigned long long *sched) {
+    LAK_PDL_WAIT();            // dependents follow at the end: this grid's SMs have little L1
+    extern __shared__ __align__(16) unsigned char stage_raw[];
+    T *xs = reinterpret_cast<T *>(stage_raw);
+    float *buf = reinterpret_cast<float *>(stage_raw + kStageBytes) + (threadIdx.x / 32) * kStageStep;
+    __shared__ StagedUnit units[2];
+    const int64_t count = head->count, total = head->staged_units;
+    const int tid = threadIdx.x;
+    auto look_up = [&](StagedUnit &un) {                   // thread 0
+        const int64_t u = (int64_t)atomicAdd(sched, 1ull);
+        un.inst = -1;
+        if (u >= total) return;
+        const int64_t i = find_instance(offs, count, u);
+        const CsrItem &it = items[i];
+        const int64_t rows = it.stage_rows, r0 = (u - __ldg(offs + i)) * rows;
+        const int64_t r1 = r0 + rows < it.d.m ? r0 + rows : it.d.m;
+        un.rp = it.d.row_ptr;
+        un.ci = it.d.col_idx;
+        un.vals = it.d.vals;
+        un.x = it.d.x;
+        un.y = it.d.y;
+        un.m = it.d.m;
+        un.n = it.d.n;
+        un.block = (unsigned int)(r0 / kStageBlock);
+        un.nb = (int32_t)((r1 + kStageBlock - 1) / kStageBlock);
+        un.nnz = (uint32_t)__ldg(it.d.row_ptr + it.d.m);
+        un.inst = (int32_t)i;
+    };
+    if (tid == 0) look_up(units[0]);
+    for (int slot = 0;; slot ^= 1) {
+        __syncthreads();                                   // the unit is known, the last one done
+        StagedUnit &un = units[slot];
+        if (un.inst < 0) break;                            // block-uniform
+        {
+            const T *x = static_cast<const T *>(un.x);
+            const int size = (int)un.n;
+            constexpr int V = 16 / (int)sizeof(T);
+            const int packs = (uintptr_t)x % 16 == 0 ? size / V : 0;
+#pragma unroll 4
+            for (int k = tid; k < packs; k += kStageThreads) {
+                Pack<T, V> p;
+                load_pack<T, V, CACHED>(p, x + k * V);
+                memcpy(xs + k * V, &p, 16);
+            }
+            for (int k = packs * V + tid; k < size; k += kStageThreads) xs[k] = x[k];
+        }
+        __syncthreads();
+        if (tid == 0) look_up(units[slot ^ 1]);
+        staged_unit<T>(un, xs, buf);
+    }
+    if (tid == 0) {
+        __threadfence();
+        unsigned int *left = reinterpret_cast<unsigned int *>(sched + 1);
+        if (atomicAdd(left, 1u) == gridDim.x - 1u) {
+            atomicExch(sched, 0ull);
+            atomicExch(left, 0u);
+        }
+    }
+}
+
 // ---- host side ---------------------------------------------------------------
+
+template <typename T>
+lak_status run_staged(const BatchHead *head, const int64_t *offs, const CsrItem *items, void *ws,
+                      int sms, cudaStream_t s) {
+    const cudaError_t e = cudaFuncSetAttribute(
+        spmv_staged_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kStageSmem);
+    if (e != cudaSuccess)
+        return fail(LAK_ECUDA, "lak_batch_run: shared memory: %s", cudaGetErrorString(e));
+    launch_k(spmv_staged_kernel<T>, sms, kStageThreads, (size_t)kStageSmem, s, head, offs, items,
+             reinterpret_cast<unsigned long long *>(static_cast<char *>(ws) + 64));
+    return check_launch("lak_batch_run (staged)");
+}
 
 template <typename T>
 lak_status run_typed(const lak_batch_info &info, const char *table, void *ws, dim3 grid,
@@ -575,10 +841,22 @@ lak_status run_typed(const lak_batch_info &info, const char *table, void *ws, di
         }
         break;
     }
-    case LAK_OP_SPMV:
-        LAK_VECSW(spmv_batch_kernel, head, offs, reinterpret_cast<const CsrItem *>(items),
-                  static_cast<unsigned long long *>(ws));
+    case LAK_OP_SPMV: {
+        const CsrItem *csr = reinterpret_cast<const CsrItem *>(items);
+        const int64_t *main_offs = offs;
+        if (info.table_bytes > base_bytes(LAK_OP_SPMV, info.count)) {
+            main_offs = reinterpret_cast<const int64_t *>(table + base_bytes(LAK_OP_SPMV, info.count));
+            const DeviceInfo *di = device_info();
+            if (!di) return LAK_ECUDA;
+            const int64_t *staged = main_offs + info.count + 1;
+            if constexpr (sizeof(T) < 8) {                 // FP64 plans stage nothing
+                const lak_status st = run_staged<T>(head, staged, csr, ws, di->sms, s);
+                if (st != LAK_OK) return st;
+            }
+        }
+        LAK_VECSW(spmv_batch_kernel, head, main_offs, csr, static_cast<unsigned long long *>(ws));
         break;
+    }
     default: return fail(LAK_EINVAL, "lak_batch_run: unsupported op %d", info.op);
     }
 #undef LAK_VECSW
@@ -652,7 +930,16 @@ LAK_API lak_status lak_batch_plan(lak_op op, lak_dtype dtype, const void *host_d
         return it;
     };
     const size_t isz = item_size(op);
-    const size_t need = items_offset(count) + isz * (size_t)count;
+    // rows of a unit where spmv_staged_kernel takes the instance, else 0; only in plans
+    // with the default shape
+    auto stage_rows = [&](const lak_csr_desc &d) -> int64_t {
+        if (es == 8 || d.m <= 0 || d.n <= 0 || d.n * es > kStageBytes ||
+            d.nnz < kStageMinEntries || d.nnz < (es == 4 ? 16 : 2) * d.m || d.nnz < 2 * d.n ||
+            !aligned_to(d.col_idx, 16) || !aligned_to(d.vals, 16))
+            return 0;
+        return cdiv(kStageEntries, d.nnz / d.m * 32) * 32;
+    };
+    int64_t main_units = 0, staged_units = 0;
 
     // units per instance
     int64_t total = 0;
@@ -683,12 +970,17 @@ LAK_API lak_status lak_batch_plan(lak_op op, lak_dtype dtype, const void *host_d
             if (d.m < 0 || d.n < 0 || d.nnz < 0 || d.nnz > 0x7fffffffLL)
                 return fail(LAK_EINVAL, "lak_batch_plan: instance %lld: bad sizes", (long long)i);
             units = cdiv(d.m, csr_rows_per_unit(d));
+            if (stage_rows(d) > 0) staged_units += cdiv(d.m, stage_rows(d));
+            else main_units += units;
             break;
         }
         default: break;
         }
         total += units;
     }
+    const bool stage = op == LAK_OP_SPMV && !(cfg && cfg->block != 0) && staged_units >= kStageMinUnits;
+    const size_t base = base_bytes(op, count);
+    const size_t need = stage ? base + 2 * offsets_bytes(count) : items_offset(count) + isz * (size_t)count;
     info->count = count;
     info->total_units = total;
     info->unit_elems = ue;
@@ -715,6 +1007,8 @@ LAK_API lak_status lak_batch_plan(lak_op op, lak_dtype dtype, const void *host_d
     h->vec = vec;
     h->block = c.block;
     h->inc = c.increment;
+    h->main_units = stage ? main_units : total;
+    h->staged_units = stage ? staged_units : 0;
     int64_t *offs = reinterpret_cast<int64_t *>(t + kHeadBytes);
     char *items = t + items_offset(count);
     int64_t acc = 0;
@@ -753,6 +1047,7 @@ LAK_API lak_status lak_batch_plan(lak_op op, lak_dtype dtype, const void *host_d
             CsrItem it{};
             it.d = d;
             it.rows_per_unit = csr_rows_per_unit(d);
+            it.stage_rows = (int32_t)stage_rows(d);
             it.vec_ok = aligned_to(d.col_idx, 16) && aligned_to(d.vals, 16);
             memcpy(items + isz * i, &it, sizeof it);
             acc += cdiv(d.m, it.rows_per_unit);
@@ -762,6 +1057,19 @@ LAK_API lak_status lak_batch_plan(lak_op op, lak_dtype dtype, const void *host_d
         }
     }
     offs[count] = acc;
+    if (stage) {
+        int64_t *mo = reinterpret_cast<int64_t *>(t + base), *so = mo + count + 1;
+        int64_t a = 0, b = 0;
+        for (int64_t i = 0; i < count; ++i) {
+            mo[i] = a;
+            so[i] = b;
+            const lak_csr_desc &d = static_cast<const lak_csr_desc *>(host_descs)[i];
+            if (stage_rows(d) > 0) b += cdiv(d.m, stage_rows(d));
+            else a += cdiv(d.m, csr_rows_per_unit(d));
+        }
+        mo[count] = a;
+        so[count] = b;
+    }
     return LAK_OK;
 }
 
