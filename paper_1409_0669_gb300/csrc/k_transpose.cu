@@ -47,7 +47,6 @@ constexpr int kTileWarps = 16;          // warps per block of the partition kern
 constexpr int kTileThreads = 32 * kTileWarps;
 constexpr int kItems = 8;               // entries a lane takes of a tile
 constexpr int kTile = kTileThreads * kItems;
-constexpr int kSegTiles = 64;           // tiles per segment of the scan over tiles
 constexpr int kOrderWarps = 16;         // warps per block of the ordering kernel
 constexpr int kBigWarps = 8;            // warps that work on a column block beyond that
 
@@ -89,122 +88,125 @@ __device__ __forceinline__ int32_t warp_rank(C *counter, int32_t d, int bits, bo
 }
 
 // first[c] = row of entry c * kChunk, by the rows (every non-empty row holds the chunk
-// starts that lie in it)
+// starts that lie in it).  The whole warp fills in the chunks of a hub row (one thread's
+// stores took 31 us for a power-law matrix of 2 M rows, all of it waiting for the longest).
 constexpr int kChunk = 128;
 __global__ void __launch_bounds__(256)
 chunk_rows_kernel(int32_t *__restrict__ first, const int32_t *__restrict__ rp, int64_t m) {
     LAK_PDL_ENTRY();
-    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < m;
-         r += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t a = __ldg(rp + r), b = __ldg(rp + r + 1);
-        for (int64_t c = (a + kChunk - 1) / kChunk; c * kChunk < b; ++c) first[c] = (int32_t)r;
+    const int lane = threadIdx.x & 31;
+    for (int64_t r0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x - lane; r0 < m;
+         r0 += (int64_t)gridDim.x * blockDim.x) {           // warp-uniform
+        const int64_t r = r0 + lane;
+        const int64_t a = r < m ? __ldg(rp + r) : 0, b = r < m ? __ldg(rp + r + 1) : 0;
+        int32_t c = (int32_t)((a + kChunk - 1) / kChunk);
+        const int32_t e = (int32_t)((b + kChunk - 1) / kChunk);
+        for (unsigned hubs = __ballot_sync(0xffffffffu, e - c > 8); hubs; hubs &= hubs - 1) {
+            const int src = __ffs((int)hubs) - 1;
+            const int32_t c0 = __shfl_sync(0xffffffffu, c, src);
+            const int32_t e0 = __shfl_sync(0xffffffffu, e, src);
+            for (int32_t i = c0 + lane; i < e0; i += 32) first[i] = (int32_t)(r0 + src);
+            if (lane == src) c = e;
+        }
+        for (; c < e; ++c) first[c] = (int32_t)r;
     }
 }
 
-// cells[tile * nb + b] = entries of the tile in column block b
+// cells[b * tiles + tile] = entries of the tile with digit b.  Keys: columns, of which
+// the digit is (column >> shift) & mask, or the digits that an earlier pass left.
+template <typename K>
 __global__ void __launch_bounds__(kTileThreads)
-part_count_kernel(int32_t *__restrict__ cells, const int32_t *__restrict__ keys, int key_stride,
-                  int64_t nnz, int shift, int mask, int nb) {
+part_count_kernel(int32_t *__restrict__ cells, const K *__restrict__ keys, int64_t nnz, int shift,
+                  int mask, int nb) {
     LAK_PDL_ENTRY();
     extern __shared__ int32_t part_smem[];
     for (int b = threadIdx.x; b < nb; b += blockDim.x) part_smem[b] = 0;
     __syncthreads();
-    const int64_t k0 = (int64_t)blockIdx.x * kTile + threadIdx.x;
+    const int64_t t0 = (int64_t)blockIdx.x * kTile;
     int32_t c[kItems];
+    if constexpr (sizeof(K) == 2) {
+        // 16-byte aligned, and readable to the end of its 16 bytes
+        Pack<uint16_t, 8> p;
+        static_assert(kItems == 8, "digits of a thread");
+        const int64_t k = t0 + threadIdx.x * kItems;
+        if (k < nnz) load_pack<uint16_t, 8, STREAM>(p, keys + k);
 #pragma unroll
-    for (int i = 0; i < kItems; ++i) {
-        const int64_t k = k0 + i * kTileThreads;
-        if (k < nnz) c[i] = __ldg(keys + k * key_stride);
-    }
+        for (int i = 0; i < kItems; ++i)
+            if (k + i < nnz) atomicAdd(part_smem + p.e[i], 1);
+    } else {
+        const int64_t k0 = t0 + threadIdx.x;
 #pragma unroll
-    for (int i = 0; i < kItems; ++i)
-        if (k0 + i * kTileThreads < nnz) atomicAdd(part_smem + ((c[i] >> shift) & mask), 1);
-    __syncthreads();
-    int32_t *out = cells + (int64_t)blockIdx.x * nb;
-    for (int b = threadIdx.x; b < nb; b += blockDim.x) out[b] = part_smem[b];
-}
-
-// Scan over the tiles of each column block, in three steps: sums per segment of tiles,
-// starts of every (column block, segment), then of every (column block, tile).
-__global__ void __launch_bounds__(256)
-seg_sum_kernel(int32_t *__restrict__ segs, const int32_t *__restrict__ cells, int64_t tiles,
-               int nb) {
-    LAK_PDL_ENTRY();
-    const int b = blockIdx.x * 256 + threadIdx.x;
-    if (b >= nb) return;
-    const int64_t t0 = (int64_t)blockIdx.y * kSegTiles;
-    const int64_t t1 = t0 + kSegTiles < tiles ? t0 + kSegTiles : tiles;
-    int32_t s = 0;
-#pragma unroll 8
-    for (int64_t t = t0; t < t1; ++t) s += __ldg(cells + t * nb + b);
-    segs[(int64_t)blockIdx.y * nb + b] = s;
-}
-
-// v[i * ld], i = i0 .. i1 - 1, replaced by start plus the sum of those before it; 16 at a
-// time, so that their loads are in flight together
-__device__ __forceinline__ void running(int32_t *v, int64_t ld, int64_t i0, int64_t i1,
-                                        int32_t start) {
-    for (int64_t i = i0; i < i1; i += 16) {
-        int32_t c[16];
-#pragma unroll
-        for (int u = 0; u < 16; ++u) c[u] = i + u < i1 ? v[(i + u) * ld] : 0;
-#pragma unroll
-        for (int u = 0; u < 16; ++u)
-            if (i + u < i1) {
-                v[(i + u) * ld] = start;
-                start += c[u];
-            }
-    }
-}
-
-// segs[seg * nb + b] -> start of that segment's entries; starts[b] of the column block
-__global__ void __launch_bounds__(1024)
-seg_scan_kernel(int32_t *__restrict__ segs, int32_t *__restrict__ starts, int64_t nseg, int nb) {
-    LAK_PDL_ENTRY();
-    __shared__ int32_t wtot[32];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    constexpr int PER = (kMaxBlocks + 1023) / 1024;     // column blocks of a thread
-    int32_t tot[PER], sum = 0;
-#pragma unroll
-    for (int i = 0; i < PER; ++i) {
-        const int b = tid * PER + i;
-        tot[i] = 0;
-        if (b < nb) {
-#pragma unroll 8
-            for (int64_t g = 0; g < nseg; ++g) tot[i] += segs[g * nb + b];
+        for (int i = 0; i < kItems; ++i) {
+            const int64_t k = k0 + i * kTileThreads;
+            if (k < nnz) c[i] = __ldg(keys + k);
         }
-        sum += tot[i];
+#pragma unroll
+        for (int i = 0; i < kItems; ++i)
+            if (k0 + i * kTileThreads < nnz) atomicAdd(part_smem + ((c[i] >> shift) & mask), 1);
     }
-    int32_t incl = sum;
+    __syncthreads();
+    for (int b = threadIdx.x; b < nb; b += blockDim.x)
+        cells[(int64_t)b * gridDim.x + blockIdx.x] = part_smem[b];
+}
+
+// Sum over a block of 1024 threads up to this one (inclusive); wtot: 32 ints, free again
+// after the next barrier
+__device__ __forceinline__ int32_t block_scan(int32_t v, int32_t *wtot) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        const int32_t up = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += up;
+        const int32_t up = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += up;
     }
-    if (lane == 31) wtot[warp] = incl;
+    if (lane == 31) wtot[warp] = v;
     __syncthreads();
-    int32_t at = incl - sum;
-    for (int w = 0; w < warp; ++w) at += wtot[w];
-#pragma unroll
-    for (int i = 0; i < PER; ++i) {
-        const int b = tid * PER + i;
-        if (b < nb) {
-            starts[b] = at;
-            running(segs + b, nb, 0, nseg, at);
-        }
-        at += tot[i];
-    }
+    int32_t before = lane < warp ? wtot[lane] : 0;
+    before = __reduce_add_sync(0xffffffffu, before);
+    return v + before;
 }
 
-__global__ void __launch_bounds__(256)
-seg_apply_kernel(int32_t *__restrict__ cells, const int32_t *__restrict__ segs, int64_t tiles,
-                 int nb) {
+// Scan over the tiles of each digit, a block per digit: cells[b][tile] -> entries of the
+// digit in the tiles before; totals[b].  (Three kernels over segments of tiles, one
+// thread per digit, took 35 us a pass for 8000 tiles; this one and the next 9.)
+__global__ void __launch_bounds__(1024)
+cell_scan_kernel(int32_t *__restrict__ cells, int32_t *__restrict__ totals, int64_t tiles) {
     LAK_PDL_ENTRY();
-    const int b = blockIdx.x * 256 + threadIdx.x;
-    if (b >= nb) return;
-    const int64_t t0 = (int64_t)blockIdx.y * kSegTiles;
-    const int64_t t1 = t0 + kSegTiles < tiles ? t0 + kSegTiles : tiles;
-    running(cells + b, nb, t0, t1, segs[(int64_t)blockIdx.y * nb + b]);
+    __shared__ int32_t wtot[32];
+    __shared__ int32_t chunk;
+    int32_t *v = cells + (int64_t)blockIdx.x * tiles;
+    int32_t carry = 0;
+    for (int64_t base = 0; base < tiles; base += 1024 * 8) {
+        const int64_t i0 = base + threadIdx.x * 8;
+        int32_t c[8], sum = 0;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            c[u] = i0 + u < tiles ? v[i0 + u] : 0;
+            sum += c[u];
+        }
+        const int32_t incl = block_scan(sum, wtot);
+        int32_t at = carry + incl - sum;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            if (i0 + u < tiles) v[i0 + u] = at;
+            at += c[u];
+        }
+        if (threadIdx.x == 1023) chunk = incl;
+        __syncthreads();
+        carry += chunk;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) totals[blockIdx.x] = carry;
+}
+
+// starts[b] = entries with digits below b (nb <= 1024)
+__global__ void __launch_bounds__(1024)
+starts_kernel(int32_t *__restrict__ starts, const int32_t *__restrict__ totals, int nb) {
+    LAK_PDL_ENTRY();
+    __shared__ int32_t wtot[32];
+    const int b = threadIdx.x;
+    const int32_t v = b < nb ? totals[b] : 0;
+    const int32_t incl = block_scan(v, wtot);
+    if (b < nb) starts[b] = incl - v;
 }
 
 constexpr size_t move_smem(int nb) {
@@ -214,12 +216,14 @@ constexpr size_t move_smem(int nb) {
 // Orders a tile's records by column block in shared memory and stores them as runs.
 // From the CSR arrays, or (CSR false) from the records of an earlier pass.
 // E: the values' type (uint16_t, uint32_t; vals may be null).
+// digits (may be null): the digit from bit `above` of the column on, for a later pass.
 template <typename E, bool CSR>
 __global__ void __launch_bounds__(kTileThreads, 2)
-part_move_kernel(Rec *__restrict__ out, const int32_t *__restrict__ rp,
+part_move_kernel(Rec *__restrict__ out, uint16_t *__restrict__ digits, int above,
+                 const int32_t *__restrict__ rp,
                  const int32_t *__restrict__ ci, const E *__restrict__ vals,
                  const Rec *__restrict__ in, const int32_t *__restrict__ cells,
-                 const int32_t *__restrict__ first, int64_t m, int64_t nnz, int shift, int mask,
+                 const int32_t *__restrict__ starts, const int32_t *__restrict__ first, int64_t m, int64_t nnz, int shift, int mask,
                  int nb, int bits) {
     LAK_PDL_ENTRY();
     constexpr int ITEMS = kItems, TILE = kTile;
@@ -312,9 +316,9 @@ part_move_kernel(Rec *__restrict__ out, const int32_t *__restrict__ rp,
         __syncthreads();
         int32_t at = incl - sum;
         for (int w = 0; w < warp; ++w) at += wtot[w];
-        const int32_t *cell = cells + (int64_t)blockIdx.x * nb;
+        const int32_t *cell = cells + blockIdx.x;
         for (int b = tid * per; b < (tid + 1) * per && b < nb; ++b) {
-            delta[b] = __ldg(cell + b) - at;
+            delta[b] = __ldg(starts + b) + __ldg(cell + (int64_t)b * gridDim.x) - at;
 #pragma unroll
             for (int w = 0; w < kTileWarps; w += 4) {
                 int32_t c[4];
@@ -350,23 +354,32 @@ part_move_kernel(Rec *__restrict__ out, const int32_t *__restrict__ rp,
         const Rec rec = stage[q];
         const int32_t pos = delta[(rec.col >> shift) & mask] + q;
         st_raw<16>(out + pos, &rec);
+        if (CSR && digits) digits[pos] = (uint16_t)(rec.col >> above);
     }
 }
 
-// bounds[b] = first record with a column of block b or later (records in block order)
+// bounds[b] = first record with a column of block b or later (records in block order); a
+// warp per block, 33 ways at a time (25 dependent loads of a binary search took 25 us)
 __global__ void __launch_bounds__(128)
 bounds_kernel(int32_t *__restrict__ bounds, const Rec *__restrict__ recs, int64_t nnz,
               int64_t blocks, int s) {
     LAK_PDL_ENTRY();
-    const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= blocks) return;
+    const int lane = threadIdx.x & 31;
+    const int64_t b = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (b >= blocks) return;                                // warp-uniform
     const int64_t c = b << s;
     int64_t lo = 0, hi = nnz;
-    while (lo < hi) {
-        const int64_t mid = (lo + hi) >> 1;
-        if (__ldg(&recs[mid].col) < c) lo = mid + 1; else hi = mid;
+    while (hi - lo > 32) {
+        const int64_t at = lo + (hi - lo) * (lane + 1) / 33;
+        const int below = __popc(__ballot_sync(0xffffffffu, __ldg(&recs[at].col) < c));
+        const int64_t l = __shfl_sync(0xffffffffu, at, below > 0 ? below - 1 : 0);
+        const int64_t h = __shfl_sync(0xffffffffu, at, below < 32 ? below : 0);
+        if (below > 0) lo = l + 1;
+        if (below < 32) hi = h;
     }
-    bounds[b] = (int32_t)lo;
+    const bool is = lo + lane < hi && __ldg(&recs[lo + lane].col) < c;
+    lo += __popc(__ballot_sync(0xffffffffu, is));
+    if (lane == 0) bounds[b] = (int32_t)lo;
 }
 
 // Records of a column block that are ordered on chip, 12 bytes each beside the counters
@@ -517,8 +530,8 @@ struct Plan {
     int64_t blocks;         // column blocks
     int passes;             // partition passes (1 or 2)
     int bits[2], nb[2];     // of each pass: bits of its digit, number of digits
-    int64_t tiles, nseg;
-    size_t off_cells, off_segs, off_starts, off_first, off_rec[2], bytes;
+    int64_t tiles;
+    size_t off_cells, off_totals, off_starts, off_first, off_rec[2], bytes;
 };
 
 size_t up256(size_t b) { return (b + 255) / 256 * 256; }
@@ -544,13 +557,12 @@ Plan make_plan(int64_t n, int64_t nnz) {
     p.nb[0] = p.passes == 1 ? (int)p.blocks : 1 << p.bits[0];
     p.nb[1] = p.passes == 1 ? 0 : (int)((p.blocks - 1) >> p.bits[0]) + 1;
     p.tiles = ceil_div(nnz, kTile);
-    p.nseg = ceil_div(p.tiles, kSegTiles);
     const int64_t nb = p.nb[0] > p.nb[1] ? p.nb[0] : p.nb[1];
     size_t at = 0;
     p.off_cells = at;
     at += up256((size_t)(p.tiles * nb) * 4);
-    p.off_segs = at;
-    at += up256((size_t)(p.nseg * nb) * 4);
+    p.off_totals = at;
+    at += up256((size_t)nb * 4);
     p.off_starts = at;
     at += up256((size_t)(p.blocks > nb ? p.blocks : nb) * 4);
     p.off_first = at;
@@ -568,7 +580,7 @@ lak_status run(const Plan &p, int32_t *col_ptr, int32_t *row_idx, int32_t *perm,
                const int32_t *rp, const int32_t *ci, const E *vals, int64_t m, int64_t n,
                int64_t nnz, char *w, cudaStream_t st) {
     int32_t *cells = reinterpret_cast<int32_t *>(w + p.off_cells);
-    int32_t *segs = reinterpret_cast<int32_t *>(w + p.off_segs);
+    int32_t *totals = reinterpret_cast<int32_t *>(w + p.off_totals);
     int32_t *starts = reinterpret_cast<int32_t *>(w + p.off_starts);
     int32_t *first = reinterpret_cast<int32_t *>(w + p.off_first);
     Rec *rec[2];
@@ -592,26 +604,30 @@ lak_status run(const Plan &p, int32_t *col_ptr, int32_t *row_idx, int32_t *perm,
         const int nb = p.nb[i];
         const int shift = p.s + (i ? p.bits[0] : 0);
         const int mask = p.passes == 2 && i == 0 ? nb - 1 : 0x7fffffff;
-        const dim3 sgrid((unsigned)ceil_div(nb, 256), (unsigned)p.nseg);
-        const int32_t *keys = i == 0 ? ci : &rec[0]->col;
         const int bits = p.bits[i];
-        launch_k(part_count_kernel, (unsigned)p.tiles, kTileThreads, (size_t)nb * 4, st, cells,
-                 keys, i == 0 ? 1 : 4, nnz, shift, mask, nb);
-        launch_k(seg_sum_kernel, sgrid, 256, 0, st, segs, (const int32_t *)cells, p.tiles, nb);
-        launch_k(seg_scan_kernel, 1, 1024, 0, st, segs, starts, p.nseg, nb);
-        launch_k(seg_apply_kernel, sgrid, 256, 0, st, cells, (const int32_t *)segs, p.tiles, nb);
+        // the second pass counts digits that the first left where its own records will go
+        uint16_t *digits = p.passes == 2 ? reinterpret_cast<uint16_t *>(rec[1]) : nullptr;
+        if (i == 0)
+            launch_k(part_count_kernel<int32_t>, (unsigned)p.tiles, kTileThreads, (size_t)nb * 4,
+                     st, cells, ci, nnz, shift, mask, nb);
+        else
+            launch_k(part_count_kernel<uint16_t>, (unsigned)p.tiles, kTileThreads, (size_t)nb * 4,
+                     st, cells, (const uint16_t *)digits, nnz, shift, mask, nb);
+        launch_k(cell_scan_kernel, (unsigned)nb, 1024, 0, st, cells, totals, p.tiles);
+        launch_k(starts_kernel, 1, 1024, 0, st, starts, (const int32_t *)totals, nb);
         if (i == 0)
             launch_k(part_move_kernel<E, true>, (unsigned)p.tiles, kTileThreads, move_smem(nb),
-                     st, rec[0], rp, ci, vals, (const Rec *)nullptr, (const int32_t *)cells,
-                     (const int32_t *)first, m, nnz, shift, mask, nb, bits);
+                     st, rec[0], digits, p.s + p.bits[0], rp, ci, vals, (const Rec *)nullptr,
+                     (const int32_t *)cells, (const int32_t *)starts, (const int32_t *)first, m,
+                     nnz, shift, mask, nb, bits);
         else
             launch_k(part_move_kernel<E, false>, (unsigned)p.tiles, kTileThreads, move_smem(nb),
-                     st, rec[1], rp, ci, (const E *)nullptr, (const Rec *)rec[0],
-                     (const int32_t *)cells,
+                     st, rec[1], (uint16_t *)nullptr, 0, rp, ci, (const E *)nullptr,
+                     (const Rec *)rec[0], (const int32_t *)cells, (const int32_t *)starts,
                      (const int32_t *)first, m, nnz, shift, mask, nb, bits);
     }
     if (p.passes == 2)
-        launch_k(bounds_kernel, (unsigned)ceil_div(p.blocks, 128), 128, 0, st, starts,
+        launch_k(bounds_kernel, (unsigned)ceil_div(p.blocks, 4), 128, 0, st, starts,
                  (const Rec *)rec[1], nnz, p.blocks, p.s);
     launch_k(order_kernel<E>, (unsigned)p.blocks, 32 * kOrderWarps, order_smem(p.s), st,
              col_ptr, row_idx, perm, vals ? vals_t : (E *)nullptr, (const Rec *)rec[p.passes - 1],
