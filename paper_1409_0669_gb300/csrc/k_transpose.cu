@@ -29,7 +29,7 @@
 // 548 us, power law about equal).
 //
 // Measured (32 M entries of a power-law matrix, 2 M columns, FP32 values carried along):
-// 1.03 ms against 3.3 ms for the atomic scatter, the columns' sort and the gather; three
+// 1.00 ms against 3.3 ms for the atomic scatter, the columns' sort and the gather; three
 // passes of 0.9-1.0 GB each, 0.45 ms at the copy rate.  Blocks of a whole SM
 // (1024 threads, tiles of 8192) took 1.42 ms, ten-bit digits in one pass with column
 // blocks of 32 K entries gathered through L2 1.30 ms, per-warp fronts without the
