@@ -1080,8 +1080,10 @@ TRAFFIC_SOURCES = {
     "copy": ("paper_1409_0669_gb300/csrc/k_vec.cu",),
     "axpy": ("paper_1409_0669_gb300/csrc/k_vec.cu",),
     "dot": ("paper_1409_0669_gb300/csrc/k_vec.cu",),
-    "gemv_row": ("paper_1409_0669_gb300/csrc/k_gemv.cu", "paper_1409_0669_gb300/csrc/gemv_row.cuh"),
-    "gemv_col": ("paper_1409_0669_gb300/csrc/k_gemv.cu",),
+    "gemv_row": ("paper_1409_0669_gb300/csrc/k_gemv.cu", "paper_1409_0669_gb300/csrc/gemv_row.cuh",
+                 "paper_1409_0669_gb300/csrc/k_gemv_wide.cu"),
+    "gemv_col": ("paper_1409_0669_gb300/csrc/k_gemv.cu",
+                 "paper_1409_0669_gb300/csrc/k_gemv_wide.cu"),
     "spmv": ("paper_1409_0669_gb300/csrc/k_spmv.cu", "paper_1409_0669_gb300/csrc/spmv_seg.cuh"),
 }
 _COMMON_SOURCES = ("paper_1409_0669_gb300/csrc/lak_internal.cuh",)

@@ -723,7 +723,10 @@ __device__ __forceinline__ void staged_unit(StagedUnit &un, const T *xs, float *
 // ticket counter, brings the unit's x into shared memory, and its warps take the unit's
 // row blocks one by one.  Thread 0 looks the next unit up meanwhile.  The last block to
 // leave resets the counters.  24 warps of 80 registers and a step of 256 entries: longer
-// steps (512, 768) ran the same rows up to 10 % faster but left less room for x.
+// steps (512, 768) ran the same rows up to 10 % faster but left less room for x.  Bound
+// by the shared-memory pipe (83 % busy at 1000 x 20000 rows, DRAM 44 %), which gathers,
+// products and row sums share; sums by two lanes interleaved, four or eight lanes per row
+// were slower (1583 against 1590, 1743 and 2056 us).
 template <typename T>
 __global__ void __launch_bounds__(kStageThreads, 1)
 spmv_staged_kernel(const BatchHead *__restrict__ head, const int64_t *__restrict__ offs,
