@@ -29,7 +29,7 @@
 // 548 us, power law about equal).
 //
 // Measured (32 M entries of a power-law matrix, 2 M columns, FP32 values carried along):
-// 1.00 ms against 3.3 ms for the atomic scatter, the columns' sort and the gather; three
+// 0.89 ms against 3.3 ms for the atomic scatter, the columns' sort and the gather; three
 // passes of 0.9-1.0 GB each, 0.45 ms at the copy rate.  Blocks of a whole SM
 // (1024 threads, tiles of 8192) took 1.42 ms, ten-bit digits in one pass with column
 // blocks of 32 K entries gathered through L2 1.30 ms, per-warp fronts without the
@@ -273,29 +273,29 @@ part_move_kernel(Rec *__restrict__ out, uint16_t *__restrict__ digits, int above
 
     // 1. ranks within the warp; a lane keeps (digit, rank) and the row of its entries
     const int64_t w0 = t0 + (int64_t)warp * 32 * ITEMS;
+    const int have = (int)(t1 - w0) - lane;         // item i is there where 32 i < have
+    const int32_t k0 = (int32_t)w0 + lane;
     uint16_t *mine = count + warp * nb;
     uint32_t where[ITEMS];
     int32_t row[ITEMS];
     Rec rec[ITEMS];
 #pragma unroll
     for (int i = 0; i < ITEMS; ++i) {
-        const int64_t k = w0 + 32 * i + lane;
         rec[i].col = 0;
         rec[i].v = 0;
-        if (k < t1) {
+        if (32 * i < have) {
             if constexpr (CSR) {
-                rec[i].col = __ldg(ci + k);
-                if (vals) rec[i].v = __ldg(vals + k);
+                rec[i].col = __ldg(ci + w0 + lane + 32 * i);
+                if (vals) rec[i].v = __ldg(vals + w0 + lane + 32 * i);
             } else {
-                ld_raw<16, STREAM>(&rec[i], in + k);
+                ld_raw<16, STREAM>(&rec[i], in + w0 + lane + 32 * i);
             }
         }
     }
 #pragma unroll
     for (int i = 0; i < ITEMS; ++i) {
-        const int64_t k = w0 + 32 * i + lane;
         const int32_t d = (rec[i].col >> shift) & mask;
-        const int32_t r = warp_rank(mine, d, bits, k < t1, lane);
+        const int32_t r = warp_rank(mine, d, bits, 32 * i < have, lane);
         where[i] = (uint32_t)d << 16 | (uint32_t)r;
     }
     if constexpr (CSR) {
@@ -360,11 +360,10 @@ part_move_kernel(Rec *__restrict__ out, uint16_t *__restrict__ digits, int above
     // 3. records to their places in the tile
 #pragma unroll
     for (int i = 0; i < ITEMS; ++i) {
-        const int64_t k = w0 + 32 * i + lane;
-        if (k >= t1) break;
+        if (32 * i >= have) break;
         if constexpr (CSR) {
             rec[i].row = row[i];
-            rec[i].k = (int32_t)k;
+            rec[i].k = k0 + 32 * i;
         }
         const int place = (int)mine[where[i] >> 16] + (int)(where[i] & 0xffffu);
         stage[place] = rec[i];
@@ -448,17 +447,20 @@ order_kernel(int32_t *__restrict__ col_ptr, int32_t *__restrict__ row_idx,
     uint16_t *mine16 = half + warp * nc;
     int32_t *mine32 = full + warp * nc;
     uint32_t where[ITEMS];
+    // on chip: item i of this lane is from[32 i] where 32 i < have (32-bit counts: with
+    // 64-bit positions throughout, 32 M entries took 293 us here, now 271)
+    const Rec *from = recs + b0 + e0 + lane;
+    const int have = small ? (int)(e1 - e0) - lane : 0;
+    const int32_t first = (int32_t)c0;
     if (small) {
         int32_t c[ITEMS];
 #pragma unroll
-        for (int i = 0; i < ITEMS; ++i) {
-            const int64_t k = e0 + 32 * i + lane;
-            c[i] = k < e1 ? (int32_t)(__ldg(&recs[b0 + k].col) - c0) : 0;
-        }
+        for (int i = 0; i < ITEMS; ++i)
+            c[i] = 32 * i < have ? __ldg(&from[32 * i].col) - first : 0;
 #pragma unroll
         for (int i = 0; i < ITEMS; ++i) {
-            if (e0 + 32 * i >= e1) break;                   // warp-uniform
-            const int32_t r = warp_rank(mine16, c[i], s, e0 + 32 * i + lane < e1, lane);
+            if (32 * i >= have + lane) break;               // warp-uniform
+            const int32_t r = warp_rank(mine16, c[i], s, 32 * i < have, lane);
             where[i] = (uint32_t)c[i] << 16 | (uint32_t)r;
         }
     } else {
@@ -517,20 +519,24 @@ order_kernel(int32_t *__restrict__ col_ptr, int32_t *__restrict__ row_idx,
         uint32_t *sv = reinterpret_cast<uint32_t *>(sk + CAP);
 #pragma unroll
         for (int i = 0; i < ITEMS; ++i) {
-            const int64_t k = e0 + 32 * i + lane;
-            if (k >= e1) break;
+            if (32 * i >= have) break;
             Rec r;
-            ld_raw<16, CACHED>(&r, recs + b0 + k);
+            ld_raw<16, CACHED>(&r, from + 32 * i);
             const int place = (int)mine16[where[i] >> 16] + (int)(where[i] & 0xffffu);
             srow[place] = r.row;
             sk[place] = r.k;
             sv[place] = r.v;
         }
         __syncthreads();
+        row_idx += b0;
+        perm += b0;
         for (int q = tid; q < (int)len; q += 32 * kOrderWarps) {
-            row_idx[b0 + q] = srow[q];
-            perm[b0 + q] = sk[q];
-            if (vals_t) vals_t[b0 + q] = (E)sv[q];
+            row_idx[q] = srow[q];
+            perm[q] = sk[q];
+        }
+        if (vals_t) {
+            vals_t += b0;
+            for (int q = tid; q < (int)len; q += 32 * kOrderWarps) vals_t[q] = (E)sv[q];
         }
         return;
     }
