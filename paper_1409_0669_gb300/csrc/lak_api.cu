@@ -418,7 +418,8 @@ bool builtin_shape(lak_op op, lak_dtype dt, int bucket, const lak_cfg *cfg) {
 //     few rows of 32 KB and more: FP32 300 x 100000 158 -> 28, 300 x 4096 3.8 -> 4.8
 //     aligned rows from 8 MiB on: 4096^2 FP32 13.3 -> 12.5, BF16 9.7 -> 7.1, BF16
 //       16384^2 87.7 -> 80; FP32 16384^2 155 -> 156, so FP32 stops at 512 MiB;
-//       16384 x 256 FP32 5.1 -> 8.2
+//       16384 x 256 FP32 5.1 -> 8.2; FP32 1400 x 1500 6.0 -> 4.0, 800 x 8000 7.7 -> 7.2,
+//       1217 x 16384 26.6 -> 16.9, 1824 x 3000 6.2 -> 6.4; BF16 1400 x 8000 9.8 -> 8.4
 RowsLaunch plan_gemv_rows(lak_dtype dt, int64_t m, int64_t n, int64_t lda, const lak_cfg *cfg,
                           const void *A, const void *x) {
     RowsLaunch R{};
@@ -440,10 +441,8 @@ RowsLaunch plan_gemv_rows(lak_dtype dt, int64_t m, int64_t n, int64_t lda, const
     if (!di) return R;
     R.period = 1;
     while ((lda * es * R.period) % 16) R.period *= 2;
-    // one row per set where sets of four would leave SMs unevenly filled: FP32
-    // 1000 x 4096 4.5 against 8.2, 1000 x 16384 12.2 against 16; 2000 x 8000 13.0
-    // with four against 14.1
-    R.rows = f64 || (m > 600 && m < 1536) || m < 4 * R.period ? 1 : 4;
+    // FP64 takes one row per set (the FP64 pipe bounds it, not the reads of x)
+    R.rows = f64 || m < 4 * R.period ? 1 : 4;
     R.sets = ceil_div(m, (int64_t)R.rows * R.period) * R.period;
     // threads per set: a dozen packs or so per thread and row, more threads when the
     // sets alone would leave the SMs with few warps
@@ -451,7 +450,13 @@ RowsLaunch plan_gemv_rows(lak_dtype dt, int64_t m, int64_t n, int64_t lda, const
     const int lo = 32, hi = R.rows == 4 ? 256 : f64 ? 64 : 128;
     R.block = pow2_floor(g < lo ? lo : g > hi ? hi : g);
     const int64_t warps = R.rows == 4 ? 8LL * di->sms : 13LL * di->sms;
-    while (R.block < 256 && R.sets * (R.block / 32) < warps && nch >= 8LL * R.block) R.block *= 2;
+    // (FP32 1536 x 1500 4.9 -> 4.2 us with 128 threads, 1000 x 3000 5.2 -> 4.6 with 256;
+    // FP64 rows of up to 40 KB stay with one warp from 6.5 per SM on: 1400 x 2000 12.5
+    // against 19.0 with two)
+    const bool alone = f64 && nch < 2560 && 2 * R.sets >= 13LL * di->sms;
+    while (R.block < 256 && R.sets * (R.block / 32) < warps && !alone &&
+           nch >= (f64 ? 8LL : 5LL) * R.block)
+        R.block *= 2;
     // column splits where one wave of blocks leaves SMs idle; four waves of smaller
     // blocks where the rows are long enough (30 x 2097152 FP64: 130 -> 118 us)
     R.splits = 1;
