@@ -288,7 +288,9 @@ lak_status outer_t(void *dA, const void *dy, const void *x, int64_t m, int64_t n
         while ((ldd * (int64_t)sizeof(T) * P) % 16) P *= 2;
         const int64_t packs = (n + 16 / (int64_t)sizeof(T) - 2) / (16 / (int64_t)sizeof(T)) + 1;
         const int64_t bx = ceil_div(packs, 256), by = ceil_div(m, kOuterRows);
-        if (bx <= 0x7fffffff && by <= 65535) {
+        // the last block of a row at least four fifths full (8000 x 1501: 10.3 against 13.6),
+        // unless every row starts alike (20001 x 100: 4.5 -> 3.1; 100000 x 50: 8.8 -> 10.8)
+        if (bx <= 0x7fffffff && by <= 65535 && (P == 1 || packs * 5 >= bx * 256 * 4)) {
             launch_k(outer_off_kernel<T>, dim3((unsigned)bx, (unsigned)by), 256, 0, s,
                      static_cast<T *>(dA), static_cast<const T *>(dy), static_cast<const T *>(x), m,
                      n, ldd, P);

@@ -606,7 +606,13 @@ lak_status plan_spmv(lak_dtype dt, int64_t m, int64_t n, int64_t nnz, const lak_
         // (elasticity) FP64 4 lanes 107, 8 lanes 119; FP32 4 and 8 lanes 65, 16 lanes 79;
         // mean 130 (65..200) FP64 8 lanes 129, 4 lanes 141, 16 lanes 139; FP32 74, 88, 78;
         // mean 600 FP64 32 lanes 131, 16 lanes 144; FP32 99 and 111
-        const int G = mean > 320 ? 32 : mean > 160 ? 16 : mean > 100 || dt != LAK_F64 ? 8 : 4;
+        // With fewer rows more lanes, so that the chip has warps enough (elasticity of 3000
+        // rows FP64 8 lanes 2.9, 4 lanes 4.2; FP32 32 lanes 1.8, 8 lanes 2.3; 50000 rows of
+        // 66..130 random columns FP32 16 lanes 14.0, 8 lanes 17.0; FP64 8 lanes 21.0, 4
+        // lanes 25.4; elasticity of 41472 rows FP32 5.6 and 5.2, FP64 10.5 and 10.0)
+        int G = mean > 320 ? 32 : mean > 160 ? 16 : mean > 100 || dt != LAK_F64 ? 8 : 4;
+        const int least = m >= 262144 ? 4 : m >= 65536 || dt == LAK_F64 ? 8 : m >= 8192 ? 16 : 32;
+        if (G < least) G = least;
         int64_t blocks = ceil_div(m * G, kSpmvLongBlock);
         if (blocks <= 0x7fffffff) {
             out->L = Launch{kSpmvLongBlock, (int)blocks, 4, LAK_INC_GLOBAL};

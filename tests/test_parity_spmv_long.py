@@ -52,3 +52,29 @@ def test_long_rows(storage, kind, m):
         assert_reduced_sum(host(y), ref, absr, np.diff(rp.numpy()).astype(np.float64), storage,
                            f"{kind} {m}")
     assert_canary(buf, m)
+
+
+@pytest.mark.parametrize("storage", ["f32", "f64", "bf16"])
+@pytest.mark.parametrize("m", [8191, 8193, 65537, 262145])
+def test_lanes_by_rows(storage, m):
+    """Row counts on both sides of the lines between the numbers of lanes per row."""
+    import paper_1409_0669_gb300 as lak
+    g = np.random.default_rng(m)
+    lens = g.integers(60, 72, m)
+    lens[[0, m // 2, m - 1]] = 4001, 0, 777         # hub rows and an empty one
+    rp = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    assert rp[-1] > 64 * m
+    ci = g.integers(0, 6007, rp[-1]).astype(np.int32)
+    rp, ci = torch.from_numpy(rp), torch.from_numpy(ci)
+    v, x = synth.normal(ci.numel(), 5, storage), synth.uniform(6007, 6, storage)
+    ref = oracle.csr_spmv(rp, ci, v, x)
+    absr = oracle.csr_spmv(rp, ci, np.abs(oracle.widen(v)), np.abs(oracle.widen(x)))
+    buf, y = canary_buffer(m, v.dtype, "cuda")
+    lak.csr_spmv(rp.cuda(), ci.cuda(), v.cuda(), x.cuda(), y=y)
+    torch.cuda.synchronize()
+    if storage == "bf16":
+        assert_reduced_sum(host(y), ref, absr, np.diff(rp.numpy()).astype(np.float64), storage,
+                           f"{m}")
+    else:
+        assert_normwise_scaled(host(y), ref, absr, storage, f"{m}")
+    assert_canary(buf, m)
