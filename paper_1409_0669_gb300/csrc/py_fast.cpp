@@ -93,15 +93,22 @@ bool number(PyObject *o, double *v) {
     return true;
 }
 
-// the workspace of (device, stream) if it has `need` bytes
-bool workspace(const Where &w, size_t need, void **p, size_t *bytes) {
-    *p = nullptr;
-    *bytes = 0;
+// A call's hold on the workspace of its (device, stream).  LAK_CALL gives the GIL up, and
+// another thread on the same stream may then replace the kept workspace by a larger one:
+// without a reference of the call's own its memory would go back to the allocator, and
+// to another tensor of that stream, before the call has launched.
+struct Workspace {
+    Tensor hold;
+    void *ptr() const { return hold.defined() ? hold.data_ptr() : nullptr; }
+    size_t bytes() const { return hold.defined() ? (size_t)hold.numel() : 0; }
+};
+
+// False if the kept workspace has fewer than `need` bytes
+bool workspace(const Where &w, size_t need, Workspace *ws) {
     if (need == 0) return true;
     const auto it = workspaces().find({w.device, w.handle});
     if (it == workspaces().end() || (size_t)it->second.numel() < need) return false;
-    *p = it->second.data_ptr();
-    *bytes = (size_t)it->second.numel();
+    ws->hold = it->second;
     return true;
 }
 
@@ -199,15 +206,16 @@ LAK_FAST(fast_axpy_norm2, 5) {
         return none();
     const int dt = storage_of(*x);
     if (dt < 0) return none();
-    void *ws;
-    size_t bytes;
-    if (!workspace(w, vec_axpy_norm2_workspace(x->numel(), (lak_dtype)dt, nullptr), &ws, &bytes))
+    Workspace ws;
+    if (!workspace(w, vec_axpy_norm2_workspace(x->numel(), (lak_dtype)dt, nullptr), &ws))
         return none();
     Tensor made;
     const Tensor *out = result_of(a[4], w, acc_type(*x), *x, false, &made);
     if (!out) return none();
     void *px = x->data_ptr(), *py = y->data_ptr(), *pz = z->data_ptr(), *po = out->data_ptr();
-    LAK_CALL(vec_axpy_norm2(px, py, pz, alpha, po, x->numel(), (lak_dtype)dt, ws, bytes, nullptr, w.stream()));
+    void *pws = ws.ptr();
+    const size_t bytes = ws.bytes();
+    LAK_CALL(vec_axpy_norm2(px, py, pz, alpha, po, x->numel(), (lak_dtype)dt, pws, bytes, nullptr, w.stream()));
     return give(a[4], made);
 }
 
@@ -218,14 +226,15 @@ LAK_FAST(fast_dot, 4) {
     if (!same(x, y) || x->numel() != y->numel()) return none();
     const int dt = storage_of(*x);
     if (dt < 0) return none();
-    void *ws;
-    size_t bytes;
-    if (!workspace(w, vec_dot_workspace(x->numel(), (lak_dtype)dt, nullptr), &ws, &bytes)) return none();
+    Workspace ws;
+    if (!workspace(w, vec_dot_workspace(x->numel(), (lak_dtype)dt, nullptr), &ws)) return none();
     Tensor made;
     const Tensor *out = result_of(a[2], w, acc_type(*x), *x, a[3] == Py_True, &made);
     if (!out) return none();
     void *px = x->data_ptr(), *py = y->data_ptr(), *po = out->data_ptr();
-    LAK_CALL(vec_dot(po, px, py, x->numel(), (lak_dtype)dt, ws, bytes, nullptr, w.stream()));
+    void *pws = ws.ptr();
+    const size_t bytes = ws.bytes();
+    LAK_CALL(vec_dot(po, px, py, x->numel(), (lak_dtype)dt, pws, bytes, nullptr, w.stream()));
     return give(a[2], made);
 }
 
@@ -236,15 +245,16 @@ LAK_FAST(fast_dot_compensated, 3) {
     if (!same(x, y) || x->numel() != y->numel()) return none();
     const int dt = storage_of(*x);
     if (dt < 0 || dt == LAK_F64) return none();
-    void *ws;
-    size_t bytes;
-    if (!workspace(w, vec_dot_workspace(x->numel(), (lak_dtype)dt, nullptr), &ws, &bytes)) return none();
+    Workspace ws;
+    if (!workspace(w, vec_dot_workspace(x->numel(), (lak_dtype)dt, nullptr), &ws)) return none();
     Tensor made;
     const Tensor *out = result_of(a[2], w, at::kDouble, *x, false, &made);
     if (!out) return none();
     void *px = x->data_ptr(), *py = y->data_ptr();
     double *po = static_cast<double *>(out->data_ptr());
-    LAK_CALL(vec_dot_compensated(po, px, py, x->numel(), (lak_dtype)dt, ws, bytes, nullptr, w.stream()));
+    void *pws = ws.ptr();
+    const size_t bytes = ws.bytes();
+    LAK_CALL(vec_dot_compensated(po, px, py, x->numel(), (lak_dtype)dt, pws, bytes, nullptr, w.stream()));
     return give(a[2], made);
 }
 
@@ -280,18 +290,19 @@ LAK_FAST(fast_gemv, 6) {
         y = vec(a[2], w);
         if (!same(y, A) || y->numel() != rows) return none();
     }
-    void *ws;
-    size_t bytes;
-    if (!workspace(w, dense_gemv_workspace(rows, cols, as, (lak_dtype)dt, nullptr), &ws, &bytes))
+    Workspace ws;
+    if (!workspace(w, dense_gemv_workspace(rows, cols, as, (lak_dtype)dt, nullptr), &ws))
         return none();
     if (a[2] == Py_None) {
         made = at::empty({rows}, A->options());
         y = &made;
     }
     void *py = y->data_ptr(), *pA = A->data_ptr(), *px = x->data_ptr();
+    void *pws = ws.ptr();
+    const size_t bytes = ws.bytes();
     LAK_CALL(alpha == 1.0 && beta == 0.0
-                 ? dense_gemv(py, pA, px, rows, cols, lda, as, (lak_dtype)dt, ws, bytes, nullptr, w.stream())
-                 : dense_gemv_axpby(py, alpha, pA, px, beta, rows, cols, lda, as, (lak_dtype)dt, ws, bytes,
+                 ? dense_gemv(py, pA, px, rows, cols, lda, as, (lak_dtype)dt, pws, bytes, nullptr, w.stream())
+                 : dense_gemv_axpby(py, alpha, pA, px, beta, rows, cols, lda, as, (lak_dtype)dt, pws, bytes,
                                     nullptr, w.stream()));
     return give(a[2], made);
 }
