@@ -28,6 +28,12 @@
 // (beside the records they cost more than the gather: 3D Laplacian 128^3 666 against
 // 548 us, power law about equal).
 //
+// Patterns with far fewer entries than rows or columns take the same passes: the cost of
+// an empty row is its share of row_ptr (chunk_rows_kernel), that of a block of empty
+// columns its part of col_ptr.  Atomic scatter -> this (us): 1000 entries in 10 M x 10 M
+// 125 -> 71, 1 M in 50 M x 1 M 159 -> 144, 1 M in 64 M x 64 M 816 -> 613; 1000 in
+// 1000 x 1000 17 -> 22 (launches).
+//
 // Measured (32 M entries of a power-law matrix, 2 M columns, FP32 values carried along):
 // 0.89 ms against 3.3 ms for the atomic scatter, the columns' sort and the gather; three
 // passes of 0.9-1.0 GB each, 0.45 ms at the copy rate.  Blocks of a whole SM
@@ -42,13 +48,12 @@ namespace {
 
 constexpr int kDigitBits = 10;
 constexpr int kMaxBlocks = 1 << kDigitBits;     // digits of a partition pass, at most
-constexpr int kMaxColBits = 10;         // columns per block: at most 2^10
+constexpr int kMaxColBits = 10;         // columns per block: at most 2^10 (or 2^12, make_plan)
 constexpr int kTileWarps = 16;          // warps per block of the partition kernels
 constexpr int kTileThreads = 32 * kTileWarps;
 constexpr int kItems = 8;               // entries a lane takes of a tile
 constexpr int kTile = kTileThreads * kItems;
 constexpr int kOrderWarps = 16;         // warps per block of the ordering kernel
-constexpr int kBigWarps = 8;            // warps that work on a column block beyond that
 
 struct __align__(16) Rec {
     int32_t col, row, k;
@@ -76,7 +81,8 @@ __device__ __forceinline__ int32_t warp_rank(C *counter, int32_t d, int bits, bo
     if (bits > 4) split(4, 6);          // warp-uniform
     if (bits > 6) split(6, 7);
     if (bits > 7) split(7, 8);
-    if (bits > 8) split(8, 11);
+    if (bits > 8) split(8, 10);
+    if (bits > 10) split(10, 12);
     const int leader = __ffs((int)same) - 1;        // of an invalid lane: any
     int32_t base = 0;
     if (valid && lane == leader) {
@@ -88,28 +94,45 @@ __device__ __forceinline__ int32_t warp_rank(C *counter, int32_t d, int bits, bo
     return base + __popc(same & ((1u << lane) - 1u));
 }
 
-// first[c] = row of entry c * kChunk, by the rows (every non-empty row holds the chunk
-// starts that lie in it).  The whole warp fills in the chunks of a hub row (one thread's
+// first[c] = row of entry c << bits, by the rows (every non-empty row holds the chunk
+// starts that lie in it).  A warp reads kRowsPerLane rows per lane at a time; few of them
+// hold a chunk start.  The whole warp fills in the chunks of a hub row (one thread's
 // stores took 31 us for a power-law matrix of 2 M rows, all of it waiting for the longest).
-constexpr int kChunk = 128;
+constexpr int kChunkBits = 7, kChunk = 1 << kChunkBits;
+constexpr int kRowsPerLane = 8;
 __global__ void __launch_bounds__(256)
-chunk_rows_kernel(int32_t *__restrict__ first, const int32_t *__restrict__ rp, int64_t m) {
+chunk_rows_kernel(int32_t *__restrict__ first, const int32_t *__restrict__ rp, int64_t m,
+                  int bits) {
     LAK_PDL_ENTRY();
+    constexpr int N = kRowsPerLane;
     const int lane = threadIdx.x & 31;
-    for (int64_t r0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x - lane; r0 < m;
-         r0 += (int64_t)gridDim.x * blockDim.x) {           // warp-uniform
-        const int64_t r = r0 + lane;
-        const int64_t a = r < m ? __ldg(rp + r) : 0, b = r < m ? __ldg(rp + r + 1) : 0;
-        int32_t c = (int32_t)((a + kChunk - 1) / kChunk);
-        const int32_t e = (int32_t)((b + kChunk - 1) / kChunk);
-        for (unsigned hubs = __ballot_sync(0xffffffffu, e - c > 8); hubs; hubs &= hubs - 1) {
-            const int src = __ffs((int)hubs) - 1;
-            const int32_t c0 = __shfl_sync(0xffffffffu, c, src);
-            const int32_t e0 = __shfl_sync(0xffffffffu, e, src);
-            for (int32_t i = c0 + lane; i < e0; i += 32) first[i] = (int32_t)(r0 + src);
-            if (lane == src) c = e;
+    const int64_t warps = (int64_t)gridDim.x * blockDim.x / 32;
+    const int64_t up = (1LL << bits) - 1;
+    for (int64_t r0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32 * (32 * N); r0 < m;
+         r0 += warps * (32 * N)) {                          // warp-uniform
+        int32_t at[N + 1];
+#pragma unroll
+        for (int j = 0; j <= N; ++j) {
+            const int64_t r = r0 + 32 * j + (j < N ? lane : 0);
+            at[j] = __ldg(rp + (r < m ? r : m));
         }
-        for (; c < e; ++c) first[c] = (int32_t)r;
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+            const int32_t down = __shfl_down_sync(0xffffffffu, at[j], 1);
+            const int32_t over = __shfl_sync(0xffffffffu, at[j + 1], 0);
+            int32_t c = (int32_t)((at[j] + up) >> bits);
+            const int32_t e = (int32_t)(((lane < 31 ? down : over) + up) >> bits);
+            if (!__any_sync(0xffffffffu, c < e)) continue;
+            const int64_t r = r0 + 32 * j;
+            for (unsigned hubs = __ballot_sync(0xffffffffu, e - c > 8); hubs; hubs &= hubs - 1) {
+                const int src = __ffs((int)hubs) - 1;
+                const int32_t c0 = __shfl_sync(0xffffffffu, c, src);
+                const int32_t e0 = __shfl_sync(0xffffffffu, e, src);
+                for (int32_t i = c0 + lane; i < e0; i += 32) first[i] = (int32_t)(r + src);
+                if (lane == src) c = e;
+            }
+            for (; c < e; ++c) first[c] = (int32_t)(r + lane);
+        }
     }
 }
 
@@ -241,6 +264,11 @@ __device__ __forceinline__ int32_t sum_counts(const uint16_t *v, int ld, int n) 
     return s;
 }
 
+// Rows that a warp walks through to find those of its entries (32 a step, a step's loads
+// behind the one before); beyond that every entry searches for its own.  1 M entries in the
+// first and last of 16 M rows: 179 ms by walking only, 84 us.
+constexpr int kWalkRows = 512;
+
 constexpr size_t move_smem(int nb) {
     return (size_t)kTile * 16 + (size_t)nb * 4 + (size_t)kTileWarps * nb * 2;
 }
@@ -249,13 +277,16 @@ constexpr size_t move_smem(int nb) {
 // From the CSR arrays, or (CSR false) from the records of an earlier pass.
 // E: the values' type (uint16_t, uint32_t; vals may be null).
 // digits (may be null): the digit from bit `above` of the column on, for a later pass.
+// rows: the entries' rows; where null they are found from row_ptr, `first` giving that of
+// every kChunk-th entry.
 template <typename E, bool CSR>
 __global__ void __launch_bounds__(kTileThreads, 2)
 part_move_kernel(Rec *__restrict__ out, uint16_t *__restrict__ digits, int above,
                  const int32_t *__restrict__ rp,
                  const int32_t *__restrict__ ci, const E *__restrict__ vals,
                  const Rec *__restrict__ in, const int32_t *__restrict__ cells,
-                 const int32_t *__restrict__ starts, const int32_t *__restrict__ first, int64_t m, int64_t nnz, int shift, int mask,
+                 const int32_t *__restrict__ starts, const int32_t *__restrict__ first,
+                 const int32_t *__restrict__ rows, int64_t m, int64_t nnz, int shift, int mask,
                  int nb, int bits) {
     LAK_PDL_ENTRY();
     constexpr int ITEMS = kItems, TILE = kTile;
@@ -299,32 +330,51 @@ part_move_kernel(Rec *__restrict__ out, uint16_t *__restrict__ digits, int above
         where[i] = (uint32_t)d << 16 | (uint32_t)r;
     }
     if constexpr (CSR) {
-        // every non-empty row that begins inside the warp's entries leaves its number at
-        // its first entry; an entry's row is the last such number up to it
-        int32_t *marks = reinterpret_cast<int32_t *>(stage) + warp * 32 * ITEMS;
-#pragma unroll
-        for (int i = 0; i < ITEMS; ++i) marks[32 * i + lane] = 0;
-        __syncwarp();
-        int32_t run = 0;
-        if (w0 < t1) {
+        // the rows that the warp's entries lie in: run .. top
+        int32_t run = 0, top = 0;
+        const int64_t w1 = w0 + 32 * ITEMS < t1 ? w0 + 32 * ITEMS : t1;
+        if (w0 < t1 && !rows) {
             run = __ldg(first + w0 / kChunk);
-            const int64_t w1 = w0 + 32 * ITEMS < t1 ? w0 + 32 * ITEMS : t1;
-            for (int64_t rb = run + 1; rb < m; rb += 32) {
+            const int64_t c1 = (w1 + kChunk - 1) / kChunk;
+            top = c1 * kChunk < nnz ? __ldg(first + c1) : (int32_t)(m - 1);
+        }
+        if (rows) {                                         // grid-uniform
+#pragma unroll
+            for (int i = 0; i < ITEMS; ++i) row[i] = 32 * i < have ? __ldg(rows + k0 + 32 * i) : 0;
+        } else if (top - run <= kWalkRows) {                // warp-uniform
+            // every non-empty row that begins inside the warp's entries leaves its number
+            // at its first entry; an entry's row is the last such number up to it
+            int32_t *marks = reinterpret_cast<int32_t *>(stage) + warp * 32 * ITEMS;
+#pragma unroll
+            for (int i = 0; i < ITEMS; ++i) marks[32 * i + lane] = 0;
+            __syncwarp();
+            for (int64_t rb = run + 1; rb <= top; rb += 32) {
                 const int64_t r = rb + lane;
-                const int64_t a = r < m ? (int64_t)__ldg(rp + r) : w1;
-                const int64_t b = r < m ? (int64_t)__ldg(rp + r + 1) : w1;
+                const int64_t a = r <= top ? (int64_t)__ldg(rp + r) : w1;
+                const int64_t b = r <= top ? (int64_t)__ldg(rp + r + 1) : w1;
                 if (a < w1 && b > a) marks[a - w0] = (int32_t)r;
                 if (__any_sync(0xffffffffu, a >= w1)) break;
             }
-        }
-        __syncwarp();
+            __syncwarp();
 #pragma unroll
-        for (int i = 0; i < ITEMS; ++i) {
-            const int32_t v = marks[32 * i + lane];
-            const unsigned begun = __ballot_sync(0xffffffffu, v) & (0xffffffffu >> (31 - lane));
-            const int32_t r = __shfl_sync(0xffffffffu, v, begun ? 31 - __clz((int)begun) : 0);
-            row[i] = begun ? r : run;
-            run = __shfl_sync(0xffffffffu, row[i], 31);
+            for (int i = 0; i < ITEMS; ++i) {
+                const int32_t v = marks[32 * i + lane];
+                const unsigned begun = __ballot_sync(0xffffffffu, v) & (0xffffffffu >> (31 - lane));
+                const int32_t r = __shfl_sync(0xffffffffu, v, begun ? 31 - __clz((int)begun) : 0);
+                row[i] = begun ? r : run;
+                run = __shfl_sync(0xffffffffu, row[i], 31);
+            }
+        } else {
+            // runs of empty rows: the last row in run .. top that begins at or before the
+            // entry, by halving (all entries of the warp in step)
+#pragma unroll
+            for (int i = 0; i < ITEMS; ++i) row[i] = run;
+            for (int32_t len = top - run + 1; len > 1; len -= len / 2) {
+                const int32_t half = len / 2;
+#pragma unroll
+                for (int i = 0; i < ITEMS; ++i)
+                    if (32 * i < have && __ldg(rp + row[i] + half) <= k0 + 32 * i) row[i] += half;
+            }
         }
     }
     __syncthreads();
@@ -404,12 +454,15 @@ bounds_kernel(int32_t *__restrict__ bounds, const Rec *__restrict__ recs, int64_
     if (lane == 0) bounds[b] = (int32_t)lo;
 }
 
+// Warps that rank the records of a column block of 2^s columns, so that their counters
+// take 32 KB
+constexpr int rank_warps(int s) { return s > kMaxColBits ? kOrderWarps >> 2 : kOrderWarps; }
 // Records of a column block that are ordered on chip, 12 bytes each beside the counters
 constexpr int kOrderItems = 12;
-constexpr int kOrderCap = 32 * kOrderWarps * kOrderItems;
+constexpr int order_cap(int s) { return 32 * rank_warps(s) * kOrderItems; }
 
 constexpr size_t order_smem(int s) {
-    return (size_t)kOrderWarps * (1 << s) * 2 + 16 + (size_t)kOrderCap * 12;
+    return (size_t)rank_warps(s) * (1 << s) * 2 + 16 + (size_t)order_cap(s) * 12;
 }
 
 // One block per column block: orders its records by column and writes the CSC arrays.
@@ -417,30 +470,34 @@ constexpr size_t order_smem(int s) {
 // The usual column block fits on chip: its records are read, ranked, placed in shared
 // memory and written out consecutively.  A larger one (hub columns) is counted and
 // ranked in place, its entries stored one by one.
-template <typename E>
+template <typename E, int RW>
 __global__ void __launch_bounds__(32 * kOrderWarps, 2)
 order_kernel(int32_t *__restrict__ col_ptr, int32_t *__restrict__ row_idx,
              int32_t *__restrict__ perm, E *__restrict__ vals_t, const Rec *__restrict__ recs,
              const int32_t *__restrict__ bounds, int64_t n, int64_t nnz, int s) {
     LAK_PDL_ENTRY();
-    constexpr int ITEMS = kOrderItems, CAP = kOrderCap;
+    constexpr int ITEMS = kOrderItems, CAP = 32 * RW * ITEMS, BIG = RW / 2;
     extern __shared__ __align__(16) unsigned char order_raw[];
     __shared__ int32_t wtot[kOrderWarps];
-    __shared__ int64_t range[2];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nc = 1 << s;
     const int64_t c0 = (int64_t)blockIdx.x << s;
-    if (tid < 2) range[tid] = blockIdx.x + tid == gridDim.x ? nnz : bounds[blockIdx.x + tid];
+    const int64_t b0 = bounds[blockIdx.x];
+    const int64_t len = (blockIdx.x + 1 == gridDim.x ? nnz : bounds[blockIdx.x + 1]) - b0;
+    if (len == 0) {                                         // block-uniform
+        for (int j = tid; j < nc; j += 32 * kOrderWarps)
+            if (c0 + j < n) col_ptr[c0 + j] = (int32_t)b0;
+        if (blockIdx.x == gridDim.x - 1 && tid == 0) col_ptr[n] = (int32_t)nnz;
+        return;
+    }
     // counters per warp and column: 16 bits for the records on chip, 32 bits and half
     // the warps for more
+    const bool small = len <= CAP;
+    const int nw = small ? RW : BIG;
     uint16_t *half = reinterpret_cast<uint16_t *>(order_raw);
     int32_t *full = reinterpret_cast<int32_t *>(order_raw);
-    for (int i = tid; i < kOrderWarps * nc / 2; i += 32 * kOrderWarps) full[i] = 0;
+    for (int i = tid; i < RW * nc / 2; i += 32 * kOrderWarps) full[i] = 0;
     __syncthreads();
-    const int64_t b0 = range[0];
-    const int64_t len = range[1] - b0;
-    const bool small = len <= CAP;
-    const int nw = small ? kOrderWarps : kBigWarps;
     const int64_t per = (len + nw * 32 - 1) / (nw * 32) * 32;
     const int64_t e0 = warp < nw ? warp * per : len;
     const int64_t e1 = e0 + per < len ? e0 + per : len;
@@ -473,10 +530,10 @@ order_kernel(int32_t *__restrict__ col_ptr, int32_t *__restrict__ row_idx,
     int32_t total = 0;
     for (int j = tid * cpt; j < (tid + 1) * cpt && j < nc; ++j) {
         if (small) {
-#pragma unroll 8
-            for (int w = 0; w < kOrderWarps; ++w) total += half[w * nc + j];
+#pragma unroll(RW < 8 ? RW : 8)
+            for (int w = 0; w < RW; ++w) total += half[w * nc + j];
         } else {
-            for (int w = 0; w < kBigWarps; ++w) total += full[w * nc + j];
+            for (int w = 0; w < BIG; ++w) total += full[w * nc + j];
         }
     }
     int32_t incl = total;
@@ -493,7 +550,7 @@ order_kernel(int32_t *__restrict__ col_ptr, int32_t *__restrict__ row_idx,
         if (c0 + j < n) col_ptr[c0 + j] = (int32_t)(b0 + at);
         if (small) {
 #pragma unroll
-            for (int w = 0; w < kOrderWarps; w += 4) {
+            for (int w = 0; w < RW; w += 4) {
                 int32_t c[4];
 #pragma unroll
                 for (int u = 0; u < 4; ++u) c[u] = half[(w + u) * nc + j];
@@ -504,7 +561,7 @@ order_kernel(int32_t *__restrict__ col_ptr, int32_t *__restrict__ row_idx,
                 }
             }
         } else {
-            for (int w = 0; w < kBigWarps; ++w) {
+            for (int w = 0; w < BIG; ++w) {
                 const int32_t c = full[w * nc + j];
                 full[w * nc + j] = at;
                 at += c;
@@ -514,7 +571,7 @@ order_kernel(int32_t *__restrict__ col_ptr, int32_t *__restrict__ row_idx,
     if (blockIdx.x == gridDim.x - 1 && tid == 0) col_ptr[n] = (int32_t)nnz;
     __syncthreads();
     if (small) {
-        int32_t *srow = reinterpret_cast<int32_t *>(order_raw + ((size_t)kOrderWarps * nc * 2 + 15) / 16 * 16);
+        int32_t *srow = reinterpret_cast<int32_t *>(order_raw + ((size_t)RW * nc * 2 + 15) / 16 * 16);
         int32_t *sk = srow + CAP;
         uint32_t *sv = reinterpret_cast<uint32_t *>(sk + CAP);
 #pragma unroll
@@ -570,12 +627,19 @@ Plan make_plan(int64_t n, int64_t nnz) {
     // columns per block: as many as leave the mean column block three quarters of what
     // the ordering kernel holds on chip, and two blocks per SM or more where they would
     // still have 2048 entries
-    const int64_t mean = kOrderCap / 4 * 3;
+    const int64_t mean = order_cap(kMaxColBits) / 4 * 3;
     int s = kMaxColBits;
     auto blocks = [&](int bits) { return ((n - 1) >> bits) + 1; };
     while (s > 0 && blocks(s - 1) <= (int64_t)kMaxBlocks * kMaxBlocks &&
            (blocks(s) * mean < nnz || (blocks(s) < 304 && blocks(s) * 2048 < nnz)))
         --s;
+    // four columns and more per entry: blocks of four times the columns, two thirds of their
+    // room filled in the mean at most, where that saves the second pass or many blocks with
+    // little to do (us: 1 M entries 4 M columns 104 -> 89, 64 M 612 -> 514; 100,000 entries
+    // 1.6 M columns 53 -> 40)
+    if (s == kMaxColBits && ((n / 4 >= nnz && blocks(s) > kMaxBlocks) ||
+                             (n / 16 >= nnz && blocks(s) > 304)))
+        s = kMaxColBits + 2;
     p.s = s;
     p.blocks = ((n - 1) >> s) + 1;
     int bits = 0;
@@ -617,18 +681,24 @@ lak_status run(const Plan &p, int32_t *col_ptr, int32_t *row_idx, int32_t *perm,
         rec[i] = reinterpret_cast<Rec *>(w + p.off_rec[i < p.passes ? i : 0]);
     const int move_most = (int)move_smem(kMaxBlocks);
     const int order_most = (int)order_smem(kMaxColBits);
+    const bool wide = p.s > kMaxColBits;
+    auto *order = wide ? order_kernel<E, rank_warps(kMaxColBits + 2)>
+                       : order_kernel<E, rank_warps(kMaxColBits)>;
     cudaError_t e = cudaFuncSetAttribute(part_move_kernel<E, true>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, move_most);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(part_move_kernel<E, false>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, move_most);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(order_kernel<E>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 order_most);
+        e = cudaFuncSetAttribute(order, cudaFuncAttributeMaxDynamicSharedMemorySize, order_most);
     if (e != cudaSuccess)
         return fail(LAK_ECUDA, "csr_transpose: shared memory: %s", cudaGetErrorString(e));
-    launch_k(chunk_rows_kernel, (unsigned)(ceil_div(m, 256) < 65535 ? ceil_div(m, 256) : 65535), 256,
-             0, st, first, rp, m);
+    // more rows than entries: the rows of all entries, kept in row_idx until order_kernel
+    // writes it (64 M rows of 1 M entries, 1 M columns: 265 us where each entry searches)
+    int32_t *rows = m > nnz ? row_idx : nullptr;
+    const int64_t row_blocks = ceil_div(m, 256 * kRowsPerLane);
+    launch_k(chunk_rows_kernel, (unsigned)(row_blocks < 65535 ? row_blocks : 65535), 256, 0, st,
+             rows ? rows : first, rp, m, rows ? 0 : kChunkBits);
     for (int i = 0; i < p.passes; ++i) {
         const int nb = p.nb[i];
         const int shift = p.s + (i ? p.bits[0] : 0);
@@ -647,18 +717,18 @@ lak_status run(const Plan &p, int32_t *col_ptr, int32_t *row_idx, int32_t *perm,
         if (i == 0)
             launch_k(part_move_kernel<E, true>, (unsigned)p.tiles, kTileThreads, move_smem(nb),
                      st, rec[0], digits, p.s + p.bits[0], rp, ci, vals, (const Rec *)nullptr,
-                     (const int32_t *)cells, (const int32_t *)starts, (const int32_t *)first, m,
-                     nnz, shift, mask, nb, bits);
+                     (const int32_t *)cells, (const int32_t *)starts, (const int32_t *)first,
+                     (const int32_t *)rows, m, nnz, shift, mask, nb, bits);
         else
             launch_k(part_move_kernel<E, false>, (unsigned)p.tiles, kTileThreads, move_smem(nb),
                      st, rec[1], (uint16_t *)nullptr, 0, rp, ci, (const E *)nullptr,
                      (const Rec *)rec[0], (const int32_t *)cells, (const int32_t *)starts,
-                     (const int32_t *)first, m, nnz, shift, mask, nb, bits);
+                     (const int32_t *)first, (const int32_t *)nullptr, m, nnz, shift, mask, nb, bits);
     }
     if (p.passes == 2)
         launch_k(bounds_kernel, (unsigned)ceil_div(p.blocks, 4), 128, 0, st, starts,
                  (const Rec *)rec[1], nnz, p.blocks, p.s);
-    launch_k(order_kernel<E>, (unsigned)p.blocks, 32 * kOrderWarps, order_smem(p.s), st,
+    launch_k(order, (unsigned)p.blocks, 32 * kOrderWarps, order_smem(p.s), st,
              col_ptr, row_idx, perm, vals ? vals_t : (E *)nullptr, (const Rec *)rec[p.passes - 1],
              (const int32_t *)starts, n, nnz, p.s);
     return check_launch("csr_transpose");
