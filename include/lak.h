@@ -330,9 +330,9 @@ LAK_API lak_status vec_dot_noalloc(void *out, const void *x, const void *y, int6
  * Workspace bytes dense_gemv (Sec. 2's matrix-vector product) needs
  * on the current device: column-major split-K partials and per-tile counters;
  * row-major the same for a few very long rows, where the columns are split over
- * blocks -- there the workspace is optional (without one, or with a smaller one,
- * the call runs unsplit, which leaves most of the GPU idle); 0 for other row-major
- * shapes.
+ * blocks, enough for any lda and alignment -- there the workspace is optional (a
+ * smaller one gets fewer splits, none at all one, which leaves most of the GPU
+ * idle); 0 for other row-major shapes.
  */
 LAK_API size_t dense_gemv_workspace(int64_t m, int64_t n, lak_layout layout,
                                     lak_dtype dtype, const lak_cfg *cfg);

@@ -15,6 +15,7 @@ allocated, which is the state the kernels require and leave behind.
 """
 from __future__ import annotations
 
+import contextlib
 import ctypes
 from typing import Optional, Sequence, Union
 
@@ -140,16 +141,35 @@ def _same_storage(*ts):
 _workspaces = {}
 
 
-def _workspace(nbytes: int, stream_handle: int, device: torch.device) -> torch.Tensor:
+def _on_stream(stream, device: torch.device):
+    """Context in which tensors are made on `stream` (None: the current one), so that their
+    memory and what fills it belong to it."""
+    if stream is None:
+        return contextlib.nullcontext()
+    if not isinstance(stream, torch.cuda.Stream):
+        stream = torch.cuda.ExternalStream(int(stream), device=device)
+    return torch.cuda.stream(stream)
+
+
+def _workspace(nbytes: int, stream_handle: int, device: torch.device, stream=None,
+               per_graph: bool = False) -> torch.Tensor:
     """Zero-filled scratch kept per (device, stream); grown (and re-zeroed)
-    when a call needs more.  Kernels leave their counters at zero."""
+    when a call needs more.  Kernels leave their counters at zero.  What is made
+    while the stream is being captured belongs to the graph, which fills it with
+    zeros in every replay, and is not kept; with per_graph a captured call always
+    gets such scratch, independent of the kept one's later growth."""
     key = (device.index, stream_handle)
     ws = _workspaces.get(key)
-    if ws is None or ws.numel() < nbytes:
-        ws = torch.zeros(max(nbytes, 256), dtype=torch.uint8, device=device)
-        _workspaces[key] = ws
-        if _fast is not None:
-            _fast.keep_workspace(device.index, stream_handle, ws)
+    if ws is not None and ws.numel() >= nbytes and not per_graph:
+        return ws
+    with _on_stream(stream, device):
+        captured = torch.cuda.is_current_stream_capturing()
+        if ws is None or ws.numel() < nbytes or captured:
+            ws = torch.zeros(max(nbytes, 256), dtype=torch.uint8, device=device)
+            if not captured:
+                _workspaces[key] = ws
+                if _fast is not None:
+                    _fast.keep_workspace(device.index, stream_handle, ws)
     return ws
 
 
@@ -314,7 +334,7 @@ def vec_axpy_norm2(x: torch.Tensor, y: torch.Tensor, z: torch.Tensor, alpha: flo
     sh = _stream(stream)
     need = int(_lib.vec_axpy_norm2_workspace(n, DTYPES[s], _cfg_ptr(cfg)))
     if workspace is None:
-        workspace = _workspace(need, sh, x.device)
+        workspace = _workspace(need, sh, x.device, stream)
     st = _lib.vec_axpy_norm2(_vec_arg(x, "x"), _vec_arg(y, "y"), _vec_arg(z, "z"), float(alpha),
                              _dev_ptr(out, "out"), n, DTYPES[s], _dev_ptr(workspace, "workspace"),
                              workspace.numel(), _cfg_ptr(cfg), sh)
@@ -350,7 +370,7 @@ def vec_dot(x: torch.Tensor, y: torch.Tensor, out: Optional[torch.Tensor] = None
         raise TypeError(f"out must be a {odt} tensor with at least one element")
     sh = _stream(stream)
     if workspace is None:
-        workspace = _workspace(_dot_ws_need(n, s, cfg), sh, x.device)
+        workspace = _workspace(_dot_ws_need(n, s, cfg), sh, x.device, stream)
     st = _lib.vec_dot(_dev_ptr(out, "out"), _vec_arg(x, "x"), _vec_arg(y, "y"), n, DTYPES[s],
                       _dev_ptr(workspace, "workspace"), workspace.numel() * workspace.element_size(),
                       _cfg_ptr(cfg), sh)
@@ -382,7 +402,7 @@ def vec_dot_sparse(vals: torch.Tensor, idx: torch.Tensor, y: torch.Tensor,
     sh = _stream(stream)
     need = vec_dot_sparse_workspace(nnz, s, cfg)
     if workspace is None:
-        workspace = _workspace(need, sh, y.device)
+        workspace = _workspace(need, sh, y.device, stream)
     st = _lib.vec_dot_sparse(_dev_ptr(out, "out"), _vec_arg(vals, "vals") if nnz else None,
                              _vec_arg(idx, "idx") if nnz else None,
                              _vec_arg(y, "y") if y.numel() else None, nnz, y.numel(), DTYPES[s],
@@ -412,7 +432,7 @@ def vec_dot_compensated(x: torch.Tensor, y: torch.Tensor, out: Optional[torch.Te
         raise TypeError("out must be a float64 tensor with at least one element")
     sh = _stream(stream)
     if workspace is None:
-        workspace = _workspace(_dot_ws_need(n, s, cfg), sh, x.device)
+        workspace = _workspace(_dot_ws_need(n, s, cfg), sh, x.device, stream)
     st = _lib.vec_dot_compensated(_dev_ptr(out, "out"), _vec_arg(x, "x"), _vec_arg(y, "y"), n,
                                   DTYPES[s], _dev_ptr(workspace, "workspace"),
                                   workspace.numel() * workspace.element_size(), _cfg_ptr(cfg), sh)
@@ -492,8 +512,8 @@ def dense_gemv(A: torch.Tensor, x: torch.Tensor, y: Optional[torch.Tensor] = Non
     need = dense_gemv_workspace(m, n, layout, s, cfg)
     ws_ptr, ws_bytes = None, 0
     if need > 0:
-        if workspace is None or layout == "row":      # the caller's serves column-major calls
-            workspace = _workspace(need, sh, A.device)
+        if workspace is None:
+            workspace = _workspace(need, sh, A.device, stream, per_graph=layout == "row")
         ws_ptr = _dev_ptr(workspace, "workspace")
         ws_bytes = workspace.numel() * workspace.element_size()
     if alpha == 1.0 and beta == 0.0:
@@ -529,8 +549,8 @@ def dense_gemv_trans(A: torch.Tensor, x: torch.Tensor, y: Optional[torch.Tensor]
     need = dense_gemv_workspace(n, m, other, s, cfg)
     ws_ptr, ws_bytes = None, 0
     if need > 0:
-        if workspace is None or other == "row":
-            workspace = _workspace(need, sh, A.device)
+        if workspace is None:
+            workspace = _workspace(need, sh, A.device, stream, per_graph=other == "row")
         ws_ptr, ws_bytes = _dev_ptr(workspace, "workspace"), workspace.numel()
     st = _lib.dense_gemv_trans(_vec_arg(y, "y"), _dev_ptr(A, "A"), _vec_arg(x, "x"), m, n, lda,
                                LAYOUTS[layout], DTYPES[s], ws_ptr, ws_bytes, _cfg_ptr(cfg), sh)
@@ -614,11 +634,7 @@ def csr_sampled_outer(row_ptr: torch.Tensor, col_idx: torch.Tensor, dy: torch.Te
 def _stream_scratch(nbytes: int, device: torch.device, stream) -> torch.Tensor:
     """Scratch for one call on `stream` (None: the current one), owned by that stream,
     so that the allocator hands it on only behind the call's kernels."""
-    if stream is None:
-        return torch.empty(max(nbytes, 256), dtype=torch.uint8, device=device)
-    if not isinstance(stream, torch.cuda.Stream):
-        stream = torch.cuda.ExternalStream(int(stream), device=device)
-    with torch.cuda.stream(stream):
+    with _on_stream(stream, device):
         return torch.empty(max(nbytes, 256), dtype=torch.uint8, device=device)
 
 

@@ -475,6 +475,24 @@ size_t rows_ws_bytes(const RowsLaunch &R, lak_dtype dt, int64_t m) {
     return (size_t)LAK_WS_COUNTER_BYTES + (size_t)R.splits * (size_t)m * (dt == LAK_F64 ? 8 : 4);
 }
 
+// What a row-major product of these sizes can use, whatever its lda and alignment: the
+// rows' period and with it the sets and splits follow from lda.
+size_t rows_ws_most(lak_dtype dt, int64_t m, int64_t n, const lak_cfg *cfg) {
+    const int es = esize(dt), v = 16 / es;
+    const DeviceInfo *di = device_info();
+    // no splits below 4096 packs a row, or where the sets fill the GPU (plan_gemv_rows)
+    if (!di || n / v < 4096 || m > 8LL * di->sms) return 0;
+    size_t most = 0;
+    for (int period = 1; period <= v; period *= 2)
+        for (int off = 0; off < 2; ++off) {
+            const int64_t lda = (n + v - 1) / v * v + (period > 1 ? v / period : 0);
+            const void *x = reinterpret_cast<const void *>((uintptr_t)(off * es));
+            const size_t b = rows_ws_bytes(plan_gemv_rows(dt, m, n, lda, cfg, nullptr, x), dt, m);
+            if (b > most) most = b;
+        }
+    return most;
+}
+
 // Column-major products with very many rows and few columns, a thread per 16 bytes
 // of rows (gemv_tall_kernel): from 768 threads per SM on.  Timed against the
 // tile-per-block kernel (us): 2097152 x 30 FP64 134 -> 122, FP32 56 -> 39; 999983 x 17
@@ -1013,9 +1031,7 @@ LAK_API size_t dense_gemv_workspace(int64_t m, int64_t n, lak_layout layout, lak
     if (!valid_dtype(dtype) || m < 0 || n < 0 || check_cfg(cfg, "dense_gemv_workspace") != LAK_OK)
         return 0;
     if (layout == LAK_COL_MAJOR && use_gemv_tall(dtype, m, n, cfg)) return 0;
-    if (layout != LAK_COL_MAJOR)
-        return rows_ws_bytes(plan_gemv_rows(dtype, m, n, n > 1 ? n : 1, cfg, nullptr, nullptr),
-                             dtype, m);
+    if (layout != LAK_COL_MAJOR) return rows_ws_most(dtype, m, n, cfg);
     // the widest vec the call could pick gives the fewest tiles; narrower vecs
     // (forced by alignment) only add tiles, so size for vec = 1 as well
     size_t best = col_off_ws_bytes(dtype, m, plan_gemv_col_off(dtype, m, n, cfg));
@@ -1057,10 +1073,14 @@ lak_status gemv_impl(const char *who, void *y, const void *A, const void *x, int
     if (layout == LAK_ROW_MAJOR) {
         RowsLaunch R = plan_gemv_rows(dtype, m, n, lda, cfg, A, x);
         if (R.rows > 0) {
-            // the workspace is optional here: without one the columns stay unsplit
+            // the workspace is optional here: as many splits as it has room for
             const size_t need = rows_ws_bytes(R, dtype, m);
-            if (need > 0 && (!workspace || ws_bytes < need || (uintptr_t)workspace % 256))
-                R.splits = 1;
+            if (need > 0 && (!workspace || ws_bytes < need || (uintptr_t)workspace % 256)) {
+                const size_t one = (size_t)m * (dtype == LAK_F64 ? 8 : 4);
+                const bool any = workspace && (uintptr_t)workspace % 256 == 0 &&
+                                 ws_bytes >= (size_t)LAK_WS_COUNTER_BYTES + 2 * one;
+                R.splits = any ? (int)((ws_bytes - (size_t)LAK_WS_COUNTER_BYTES) / one) : 1;
+            }
             return launch_gemv_rows(dtype, y, A, x, m, n, lda, R, workspace, alpha, beta, s);
         }
         RowPlan p;

@@ -14,6 +14,7 @@
 
 #include <ATen/ATen.h>
 #include <c10/cuda/CUDAFunctions.h>
+#include <c10/cuda/CUDAGraphsC10Utils.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/autograd/python_variable.h>
 
@@ -291,8 +292,12 @@ LAK_FAST(fast_gemv, 6) {
         if (!same(y, A) || y->numel() != rows) return none();
     }
     Workspace ws;
-    if (!workspace(w, dense_gemv_workspace(rows, cols, as, (lak_dtype)dt, nullptr), &ws))
+    const size_t need = dense_gemv_workspace(rows, cols, as, (lak_dtype)dt, nullptr);
+    // a row-major product in a graph has scratch of the graph's own (Python path)
+    if (need > 0 && as == LAK_ROW_MAJOR &&
+        c10::cuda::currentStreamCaptureStatusMayInitCtx() != c10::cuda::CaptureStatus::None)
         return none();
+    if (!workspace(w, need, &ws)) return none();
     if (a[2] == Py_None) {
         made = at::empty({rows}, A->options());
         y = &made;
