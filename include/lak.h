@@ -532,9 +532,9 @@ LAK_API lak_status vec_scale_dev(void *out, const void *v, const void *alpha, in
  * for F32/BF16/F16, double for F64), LAK_OP_GEMV_ROW (lak_gemv_desc, row-major
  * instances), LAK_OP_SPMV (lak_csr_desc, warp-segmented rows; its warps take
  * 32-row blocks in order from a ticket counter in the workspace, so cfg.increment
- * does not apply to it; plans without a cfg give FP32 and 16-bit instances whose x
- * fits in shared memory to a second kernel of the same run, which reads all n
- * values of x).  The dot and CSR batches keep counters in the
+ * does not apply to it; plans for which the caller gave neither a cfg nor a default
+ * (lak_set_batch_default_cfg) give FP32 and 16-bit instances whose x fits in shared
+ * memory to a second kernel of the same run, which reads all n values of x).  The dot and CSR batches keep counters in the
  * workspace: one run of a batch at a time per workspace.  Per instance
  * the results equal those of the single-instance calls up to the order of
  * floating-point summation (axpy: identical).  The dot keeps at most
@@ -585,6 +585,12 @@ LAK_API lak_status lak_batch_run(const lak_batch_info *info, const void *dev_tab
  * plans made earlier keep their configuration.
  */
 LAK_API lak_status lak_set_batch_default_cfg(lak_op op, lak_dtype dtype, const lak_cfg *cfg);
+
+/* The same for an entry that was measured on the library's behalf (the Python package
+ * installs those it ships): it shapes the persistent launch, and the library still chooses
+ * the kernels, so CSR plans keep their second one.  The two calls replace each other's
+ * entry.  (Sec. 3.4, as above.) */
+LAK_API lak_status lak_set_batch_tuned_cfg(lak_op op, lak_dtype dtype, const lak_cfg *cfg);
 
 /* ------------------------------------------------------------------------
  * Measurement aid (no counterpart in the paper, whose roofs are the devices'

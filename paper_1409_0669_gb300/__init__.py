@@ -216,6 +216,11 @@ def _apply_batch_default(op: str, storage: str, cfg: CfgLike):
                   _lib.lak_set_batch_default_cfg(OPS[op], DTYPES[storage], _cfg_ptr(cfg)))
 
 
+def _apply_batch_tuned(op: str, storage: str, cfg: CfgLike):
+    _native.check("lak_set_batch_tuned_cfg",
+                  _lib.lak_set_batch_tuned_cfg(OPS[op], DTYPES[storage], _cfg_ptr(cfg)))
+
+
 def set_batch_default_cfg(op: str, storage: str, cfg: CfgLike):
     """Replace (or with cfg=None restore the built-in shape of) the launch
     configuration that batched launches of `op` take when planned without one.

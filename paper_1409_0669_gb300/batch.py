@@ -47,7 +47,7 @@ def install_tuned_defaults(path: str = TUNED_DEFAULTS) -> int:
         return 0
     import json
 
-    from . import _apply_batch_default, _user_batch_defaults
+    from . import _apply_batch_tuned, _user_batch_defaults
     from .autotune import cache_key
     with open(path) as fh:
         entries = json.load(fh).get(cache_key(), {})
@@ -56,7 +56,7 @@ def install_tuned_defaults(path: str = TUNED_DEFAULTS) -> int:
         parts = key.split(":")
         if parts[0] != "batch" or (parts[1], parts[2]) in _user_batch_defaults:
             continue
-        _apply_batch_default(parts[1], parts[2], tuple(cfg))
+        _apply_batch_tuned(parts[1], parts[2], tuple(cfg))
         done += 1
     return done
 

@@ -75,7 +75,7 @@ struct CsrItem {
 };
 
 // CSR instances (FP32 and 16-bit storage) whose x fits in one SM's shared memory are taken
-// by spmv_staged_kernel, in plans with the default shape.  spmv_batch_kernel is bound by
+// by spmv_staged_kernel, in plans without a configuration of the caller's.  spmv_batch_kernel is bound by
 // its gathers through L1 (one lane per clock and SM: 262 G entries/s) and, on short rows,
 // by the walk over their ends; shared memory serves about nine random lanes per clock.
 // Measured in G entries/s, spmv_batch_kernel against the staged one:
@@ -933,8 +933,7 @@ LAK_API lak_status lak_batch_plan(lak_op op, lak_dtype dtype, const void *host_d
         return it;
     };
     const size_t isz = item_size(op);
-    // rows of a unit where spmv_staged_kernel takes the instance, else 0; only in plans
-    // with the default shape
+    // rows of a unit where spmv_staged_kernel takes the instance, else 0
     auto stage_rows = [&](const lak_csr_desc &d) -> int64_t {
         if (es == 8 || d.m <= 0 || d.n <= 0 || d.n * es > kStageBytes ||
             d.nnz < kStageMinEntries || d.nnz < (es == 4 ? 16 : 2) * d.m || d.nnz < 2 * d.n ||
@@ -981,7 +980,7 @@ LAK_API lak_status lak_batch_plan(lak_op op, lak_dtype dtype, const void *host_d
         }
         total += units;
     }
-    const bool stage = op == LAK_OP_SPMV && !(cfg && cfg->block != 0) && staged_units >= kStageMinUnits;
+    const bool stage = op == LAK_OP_SPMV && staged_units >= kStageMinUnits && batch_own_kernels(op, dtype, cfg);
     const size_t base = base_bytes(op, count);
     const size_t need = stage ? base + 2 * offsets_bytes(count) : items_offset(count) + isz * (size_t)count;
     info->count = count;

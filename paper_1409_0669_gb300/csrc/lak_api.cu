@@ -234,8 +234,10 @@ std::mutex g_cfg_mu;
 
 // Batched defaults installed with lak_set_batch_default_cfg (axpy, dot,
 // row-major GEMV, CSR), per storage type.
+// g_batch_shape: installed with lak_set_batch_tuned_cfg, which leaves the choice of kernels
+// to the library.
 lak_cfg g_batch_override[4][4];
-bool g_has_batch_override[4][4];
+bool g_has_batch_override[4][4], g_batch_shape[4][4];
 
 int batch_op_index(lak_op op) {
     switch (op) {
@@ -684,6 +686,13 @@ lak_cfg batch_config(lak_op op, lak_dtype dt, const lak_cfg *cfg) {
     return c;
 }
 
+bool batch_own_kernels(lak_op op, lak_dtype dt, const lak_cfg *cfg) {
+    if (cfg && cfg->block != 0) return false;
+    std::lock_guard<std::mutex> lk(g_cfg_mu);
+    const int bi = batch_op_index(op);
+    return bi < 0 || !g_has_batch_override[bi][dt] || g_batch_shape[bi][dt];
+}
+
 lak_status plan_dot(const char *who, lak_dtype dt, int64_t n, const lak_cfg *cfg, const void *x,
                     const void *y, Launch *L, int64_t *head) {
     lak_status st = check_cfg(cfg, who);
@@ -773,23 +782,32 @@ LAK_API lak_status lak_set_default_cfg(lak_op op, lak_dtype dtype, const lak_cfg
     return lak_set_default_cfg_bucket(op, dtype, -1, cfg);
 }
 
-LAK_API lak_status lak_set_batch_default_cfg(lak_op op, lak_dtype dtype, const lak_cfg *cfg) {
+static lak_status set_batch_cfg(const char *who, lak_op op, lak_dtype dtype, const lak_cfg *cfg,
+                                bool shape) {
     const int bi = batch_op_index(op);
-    if (bi < 0) return fail(LAK_EINVAL, "lak_set_batch_default_cfg: op %d has no batched form", (int)op);
-    if (!valid_dtype(dtype))
-        return fail(LAK_EDTYPE, "lak_set_batch_default_cfg: unknown dtype %d", (int)dtype);
+    if (bi < 0) return fail(LAK_EINVAL, "%s: op %d has no batched form", who, (int)op);
+    if (!valid_dtype(dtype)) return fail(LAK_EDTYPE, "%s: unknown dtype %d", who, (int)dtype);
     if (cfg && cfg->block != 0) {
         const int max_block = op == LAK_OP_GEMV_ROW ? kGemvBatchMaxBlock : 512;
         if (cfg->block < 32 || cfg->block > max_block || cfg->block % 32 || cfg->grid < 0 ||
             (cfg->vec != 0 && !pow2_vec(cfg->vec)) ||
             (cfg->increment != LAK_INC_GLOBAL && cfg->increment != LAK_INC_LOCAL))
-            return fail(LAK_EINVAL, "lak_set_batch_default_cfg: invalid cfg (%d, %d, %d, %d)",
-                        cfg->block, cfg->grid, cfg->vec, cfg->increment);
+            return fail(LAK_EINVAL, "%s: invalid cfg (%d, %d, %d, %d)", who, cfg->block, cfg->grid,
+                        cfg->vec, cfg->increment);
     }
     std::lock_guard<std::mutex> lk(g_cfg_mu);
     g_has_batch_override[bi][dtype] = cfg && cfg->block != 0;
+    g_batch_shape[bi][dtype] = shape;
     if (g_has_batch_override[bi][dtype]) g_batch_override[bi][dtype] = *cfg;
     return LAK_OK;
+}
+
+LAK_API lak_status lak_set_batch_default_cfg(lak_op op, lak_dtype dtype, const lak_cfg *cfg) {
+    return set_batch_cfg("lak_set_batch_default_cfg", op, dtype, cfg, false);
+}
+
+LAK_API lak_status lak_set_batch_tuned_cfg(lak_op op, lak_dtype dtype, const lak_cfg *cfg) {
+    return set_batch_cfg("lak_set_batch_tuned_cfg", op, dtype, cfg, true);
 }
 
 LAK_API int32_t lak_size_bucket(lak_op op, lak_dtype dtype, int64_t m, int64_t n, int64_t nnz) {

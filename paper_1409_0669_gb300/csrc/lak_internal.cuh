@@ -118,6 +118,10 @@ constexpr int kGemvBatchMaxBlock = 128;
 // call; grid left as given.
 lak_cfg batch_config(lak_op op, lak_dtype dt, const lak_cfg *cfg);
 
+// Whether the library chooses the kernels of a batch: neither an explicit cfg nor a default
+// that the caller installed names its launch.
+bool batch_own_kernels(lak_op op, lak_dtype dt, const lak_cfg *cfg);
+
 // Largest vec <= want (power of two) whose access width divides the byte
 // offsets of every pointer in `ptrs` modulo the access width identically, so
 // that one scalar prologue aligns all of them at once.  Also returns the
