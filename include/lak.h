@@ -99,7 +99,10 @@ typedef enum {
  * A NULL cfg, or one whose block is 0, takes the library default for the op,
  * storage type and size bucket (set by lak_set_default_cfg[_bucket], e.g. from
  * an autotuning cache, else built in); a zero grid or vec in an otherwise
- * explicit cfg is filled in by the library.
+ * explicit cfg is filled in by the library.  A configuration, given or installed,
+ * names the launch of the op's general kernel; the kernels for special shapes
+ * (dense_gemv by row sets, on tall and on unaligned columns, long CSR rows, the
+ * fused update and norm's own shape) run only in calls without one.
  */
 typedef struct {
     int32_t block;
@@ -158,7 +161,9 @@ LAK_API lak_status lak_set_default_cfg(lak_op op, lak_dtype dtype, const lak_cfg
  * ops m = n = the vector length; for dense_gemv the matrix is m-by-n; for
  * csr_spmv m rows, n columns and nnz stored entries (nnz is ignored by the
  * other ops).  `vec` in *out is the vector width the call would actually use
- * for aligned pointers.  Writes *out; returns LAK_OK or a negative status.
+ * for aligned pointers.  Where the call takes a kernel for a special shape, *out
+ * describes that kernel's launch; given back as a cfg it names one of the general
+ * kernel.  Writes *out; returns LAK_OK or a negative status.
  */
 LAK_API lak_status lak_resolve_cfg(lak_op op, lak_dtype dtype, int64_t m, int64_t n,
                                    int64_t nnz, const lak_cfg *cfg, lak_cfg *out);

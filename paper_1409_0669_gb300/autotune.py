@@ -32,6 +32,10 @@ increments (the CSR batch schedules dynamically, so only one) -- searched by
 `tune_batch` on the batching workload itself (4096 uneven instances of one
 family, synth.batch_workload), one run of the whole batch per timing.
 
+A configuration names the general kernel's launch; the kernels the library has for
+special shapes run only in calls without one.  So the bucket and batch searches time the
+call without a configuration too, and keep nothing where that is the fastest.
+
 The winners can be saved as a JSON cache keyed by GPU name and SM count and
 installed as the library's per-op defaults (lak_set_default_cfg;
 "batch:<op>:<storage>" entries: lak_set_batch_default_cfg).  The cache this
@@ -51,6 +55,7 @@ from __future__ import annotations
 
 import argparse
 import json
+import os
 import statistics
 from typing import Callable, Dict, List, Optional
 
@@ -430,14 +435,20 @@ def problem_bucket(prob: Problem) -> int:
     return lib.lak_size_bucket(_OP_CODES[prob.op], DTYPES[prob.storage], *prob.dims)
 
 
-def choose_per_bucket(results: Dict[object, List[Dict]], buckets: Dict[object, int]) -> Dict[int, Dict]:
+def choose_per_bucket(results: Dict[object, List[Dict]], buckets: Dict[object, int],
+                      own: Optional[Dict[object, float]] = None) -> Dict[int, Dict]:
     """results: size -> tune() output; buckets: size -> bucket.  Per bucket,
     the configuration (timed at every size of the bucket) whose worst ratio
-    of the size's best time to its own time is largest."""
+    of the size's best time to its own time is largest.  own: size -> time of the
+    call without a configuration; a bucket where the library's own choice is the
+    best of all gets "cfg": None (nothing to install there)."""
     out = {}
     for b in sorted(set(buckets.values())):
         sizes = [sz for sz, bb in buckets.items() if bb == b]
         tables = {sz: {tuple(r["cfg"]): r["us"] for r in results[sz]} for sz in sizes}
+        if own is not None:
+            for sz in sizes:
+                tables[sz][()] = own[sz]        # the empty tuple sorts first: it wins a tie
         common = set.intersection(*(set(t) for t in tables.values()))
         best_cfg, best_score = None, -1.0
         for c in sorted(common):
@@ -445,20 +456,29 @@ def choose_per_bucket(results: Dict[object, List[Dict]], buckets: Dict[object, i
             if score > best_score:
                 best_cfg, best_score = c, score
         if best_cfg is not None:
-            out[b] = {"cfg": list(best_cfg), "worst_ratio": best_score, "sizes": sizes}
+            out[b] = {"cfg": list(best_cfg) or None, "worst_ratio": best_score, "sizes": sizes}
     return out
 
 
+def own_choice_us(prob, reps: int) -> float:
+    """Time of the call without a configuration, as often as refine_top times a candidate."""
+    return statistics.median(prob.time_cfg(None, reps) for _ in range(1 + REFINE_ROUNDS))
+
+
 def tune_buckets(op: str, storage: str, sizes, reps: int = 15) -> Dict[int, Dict]:
-    """Tune `op` at every size and keep one configuration per size bucket."""
-    results, buckets = {}, {}
+    """Tune `op` at every size and keep one configuration per size bucket, none where the
+    library's own choice is faster: a configuration names the general kernel's launch, so
+    the kernels for special shapes (row sets, long CSR rows, ...) run only without one.
+    Run it without installed defaults, which are what a call without a configuration takes."""
+    results, buckets, own = {}, {}, {}
     for sz in sizes:
         prob = Problem(op, storage, sz)
+        own[sz] = own_choice_us(prob, reps)
         results[sz] = tune(op, storage, sz, reps, problem=prob)
         buckets[sz] = problem_bucket(prob)
         del prob
         torch.cuda.empty_cache()
-    return choose_per_bucket(results, buckets)
+    return choose_per_bucket(results, buckets, own)
 
 
 def _default_point(prob: Problem, reps: int) -> Dict:
@@ -473,13 +493,17 @@ def cache_key() -> str:
 
 def save_cache(path: str, entries: Dict[str, List[int]]):
     """entries: {"<op>:<storage>": [block, grid, vec, increment]} for every
-    size bucket, or {"<op>:<storage>:<bucket>": [...]} for one."""
+    size bucket, or {"<op>:<storage>:<bucket>": [...]} for one; None in the place of a
+    configuration removes an entry (the library's own choice is faster)."""
     try:
         with open(path) as fh:
             data = json.load(fh)
     except (OSError, ValueError):
         data = {}
-    data.setdefault(cache_key(), {}).update(entries)
+    kept = data.setdefault(cache_key(), {})
+    kept.update(entries)
+    for key in [k for k, cfg in kept.items() if cfg is None]:
+        del kept[key]
     with open(path, "w") as fh:
         json.dump(data, fh, indent=1, sort_keys=True)
 
@@ -532,28 +556,33 @@ def _main(argv=None):
     cache_entries = {}
     if args.batch:
         res = tune_batch(args.op, args.storage, args.count, reps=min(args.reps, 5))
-        # the built-in shape: time a plan without a cfg with any installed entry
+        # a plan without a cfg: with the shipped entry, and with any installed entry
         # removed (the batched runner installs the shipped cache on first use)
         from . import _apply_batch_default
         from . import batch as _B
         prob_default = BatchProblem(args.op, args.storage, args.count)
         _B.install_tuned_defaults()
+        own_us = own_choice_us(prob_default, 5)
         _apply_batch_default(args.op, args.storage, None)
         default_us = prob_default.time_cfg(None)
         del prob_default
         _B._installed.discard(torch.cuda.current_device())
         _B.install_tuned_defaults()
-        cache_entries[f"batch:{args.op}:{args.storage}"] = res[0]["cfg"]
+        # an entry of the package's own file only shapes the launch; elsewhere it names it,
+        # and is not worth having where the library's own choice is faster
+        shipped = bool(args.save_cache) and os.path.realpath(args.save_cache) == os.path.realpath(_B.TUNED_DEFAULTS)
+        cache_entries[f"batch:{args.op}:{args.storage}"] = \
+            res[0]["cfg"] if shipped or res[0]["us"] < own_us else None
         text = json.dumps({"op": args.op, "storage": args.storage, "count": args.count,
                            "top": res[:args.top], "worst": res[-3:], "count_cfgs": len(res),
-                           "builtin_default_us": default_us}, indent=1)
+                           "builtin_default_us": default_us, "own_choice_us": own_us}, indent=1)
     elif args.buckets:
         sizes = [int(v) if v.isdigit() else v for v in args.size.split(",")]
         per = tune_buckets(args.op, args.storage, sizes, args.reps)
         text = json.dumps({"op": args.op, "storage": args.storage,
                            "buckets": {str(b): v for b, v in per.items()},
                            "cache": {f"{args.op}:{args.storage}:{b}": v["cfg"]
-                                     for b, v in per.items()}}, indent=1)
+                                     for b, v in per.items() if v["cfg"]}}, indent=1)
     elif args.study:
         label = "paper" if args.paper_sizes else "large"
         rep = copy_first_study(args.storage, STUDY_SIZES[label], reps=args.reps)
