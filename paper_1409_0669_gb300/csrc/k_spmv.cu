@@ -104,24 +104,27 @@ __device__ __forceinline__ typename Acc<T>::type group_row(const int32_t *__rest
                                                            int32_t longest, int lg) {
     using Ac = typename Acc<T>::type;
     constexpr int S = sizeof(Ac) == 8 ? 1 : 2;              // partial sums
+    using Step = uint32_t;
     Ac acc[S];
 #pragma unroll
     for (int i = 0; i < S; ++i) acc[i] = Ac(0);
-    for (int32_t base = 0; base < longest; base += G * U) {
+    // unsigned: the step past a row of nearly 2^31 entries must not wrap
+    static_assert((Step)0x7fffffff + 32 * U > (Step)0x7fffffff, "the last step of the longest row");
+    for (Step base = 0; base < (Step)longest; base += G * U) {
         int32_t col[U];
         T val[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int32_t k = base + u * G + lg;
-            if (k < len) {
+            const Step k = base + u * G + lg;
+            if (k < (Step)len) {
                 ld_raw<4, P>(&col[u], c + k);
                 ld_raw<(int)sizeof(T), P>(&val[u], v + k);
             }
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int32_t k = base + u * G + lg;
-            if (base + u * G < longest && k < len) {        // the first part is uniform
+            const Step k = base + u * G + lg;
+            if (base + u * G < (Step)longest && k < (Step)len) {    // the first part is uniform
                 Ac &a = acc[u % S];
                 a = fma_acc(widen(val[u]), widen(ld_cached(x + col[u])), a);
             }
