@@ -305,8 +305,10 @@ gemv_tall_kernel(T *__restrict__ y, const T *__restrict__ A, const T *__restrict
 // aligned 16-byte ones, and its sums are added to the block's rows at that shift.  A
 // block owns 31 V rows, which every window covers; the rows read twice (1 / 32) are the
 // neighbouring block's, in L2.  No load leaves a column's rows.  Splits over columns
-// and their combine as in the tile-per-block kernel.  FP32 7999 x 8000 117 -> 49 us
-// (5.2 TB/s), BF16 74 -> 33, FP64 211 -> 139.
+// as in the tile-per-block kernel.  Tile-per-block -> this (us, back to back, L2 cold):
+// FP32 7999 x 8000 117 -> 50 (5.1 TB/s), 3001 x 5000 39.6 -> 15.5; BF16 74 -> 33 and 26.5
+// -> 13.1; FP64 208 -> 139 and 54.4 -> 40.4.  With the matrix in L2: FP32 3001 x 5000 20 ->
+// 9.9, BF16 15.2 -> 9.9.
 template <typename T>
 __global__ void __launch_bounds__(kGemvOffBlock)
 gemv_col_off_kernel(T *__restrict__ y, const T *__restrict__ A, const T *__restrict__ x, int64_t m,
@@ -376,10 +378,22 @@ gemv_col_off_kernel(T *__restrict__ y, const T *__restrict__ A, const T *__restr
     for (int rr = threadIdx.x; rr < OWN; rr += kGemvOffBlock) {
         const int64_t row = tile0 + rr;
         if (row >= m) break;
-        double t = 0.0;                                      // many splits of few columns each
-#pragma unroll 4
-        for (int q = 0; q < nsplit; ++q) t += (double)__ldcg(partials + (int64_t)q * m + row);
-        y[row] = epilogue<T>((Ac)t, alpha, beta, beta != Ac(0) ? widen(y[row]) : Ac(0));
+        // eight splits at a time, their loads together: one by one and in FP64 this tail was
+        // a third of a product of 46 splits
+        const Ac *p = partials + row;
+        Ac t = Ac(0);
+        int q = 0;
+        for (; q + 8 <= nsplit; q += 8) {
+            Ac u[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) u[i] = __ldcg(p + (int64_t)(q + i) * m);
+            t += ((u[0] + u[1]) + (u[2] + u[3])) + ((u[4] + u[5]) + (u[6] + u[7]));
+        }
+        Ac u[7];
+#pragma unroll
+        for (int i = 0; i < 7; ++i) u[i] = q + i < nsplit ? __ldcg(p + (int64_t)(q + i) * m) : Ac(0);
+        t += ((u[0] + u[1]) + (u[2] + u[3])) + ((u[4] + u[5]) + u[6]);
+        y[row] = epilogue<T>(t, alpha, beta, beta != Ac(0) ? widen(y[row]) : Ac(0));
     }
 }
 

@@ -510,15 +510,17 @@ bool use_gemv_tall(lak_dtype dt, int64_t m, int64_t n, const lak_cfg *cfg) {
 
 // Column-major products with columns off 16 bytes (gemv_col_off_kernel): the column
 // splits, 0 where the tile-per-block kernel keeps the call.  The lines lie where both
-// were timed (us, L2 cold, tile-per-block -> this):
-//   FP32 from 1 MiB on, six blocks per SM: 1001^2 9.5 -> 7.5, 3001 x 5000 39 -> 16,
-//     7999 x 8000 117 -> 49, 16383 x 16384 541 -> 195; 301 x 300 3.8 -> 4.5
-//   16 bits from 2000 rows on: BF16 3001 x 5000 26 -> 15, 7999 x 8000 74 -> 33; 1001^2
-//     6.6 -> 7.8
-//   FP64 from 2000 rows and 700 columns up to 512 MiB, eight blocks per SM: 3001 x 5000
-//     55 -> 40, 7999 x 8000 211 -> 139; 16383 x 500 20 -> 23, 16383 x 16384 554 -> 568;
-//     and where the tiles alone fill the GPU (1216): 100003 x 200 55 -> 44
-// Eight columns per warp and split at least: the last block adds the splits one by one.
+// were timed (us, back to back, L2 cold and, in brackets, the matrix in L2):
+//   FP32 from 1 MiB on, six blocks per SM: 1001^2 9.0 -> 6.7 (5.8 -> 5.3), 3001 x 5000
+//     39.6 -> 15.5 (20 -> 9.9), 7999 x 8000 117 -> 50, 301 x 3000 8.6 -> 7.4 (6.0, 6.1);
+//     301 x 300 3.8 -> 4.5
+//   16 bits from 2000 rows on: BF16 2001 x 2000 13.3 -> 8.9 (7.9 -> 6.8), 3001 x 5000 26.5
+//     -> 13.1 (15.2 -> 9.9), 7999 x 8000 74 -> 33
+//   FP64 from 2000 rows and 700 columns up to 512 MiB, eight blocks per SM: 2001 x 2000
+//     18.8, 18.8 (19.0 -> 16.2), 3001 x 5000 54.4 -> 40.4, 7999 x 8000 209 -> 139; 16383 x
+//     500 20 -> 23, 16383 x 16384 554 -> 568; and where the tiles alone fill the GPU
+//     (1216): 100003 x 200 55 -> 44
+// Eight columns per warp and split at least, for the last block's sums over the splits.
 int plan_gemv_col_off(lak_dtype dt, int64_t m, int64_t n, const lak_cfg *cfg) {
     const int es = esize(dt), v = 16 / es;
     const int64_t bytes = op_bytes(LAK_OP_GEMV_COL, dt, m, n, 0);
