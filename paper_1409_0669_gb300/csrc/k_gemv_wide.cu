@@ -222,19 +222,25 @@ gemv_rows_kernel(T *__restrict__ y, const T *__restrict__ A, const T *__restrict
 // A thread owns V consecutive rows and walks all columns: every warp load is 32 V
 // consecutive entries of one column, and nothing is combined between threads (the
 // tile-per-block kernel splits its columns over the block's warps and adds their sums
-// in shared memory, which for 30 FP64 columns was a quarter of its FP64 work).
+// in shared memory).  Sums of kGemvTallOneSum columns are added to a running one, so that the
+// chains of roundings are no longer than the tile-per-block kernel's (one chain over 30
+// FP32 columns was 22 % further off, over 64 columns 64 %).  FP64 is bound by its pipe, on
+// which those additions cost what the form saves (2097152 x 30: 118 us with one chain, 134
+// with sums, 125 by tiles), so it comes here only with one such sum.
 // SHIFT: columns start at other offsets than a multiple of 16 bytes; each pack is
 // then read through two aligned loads and shifted by the column's offset (uniform
 // over the grid; the second load hits L1).  The first and the last column, whose
-// windows could leave the matrix, are read one element at a time.  Measured (us): FP64
-// 2097152 x 30 134 -> 121 (FP64 pipe: 107 with the epilogue), FP32 1000000 x 8 16.1 ->
-// 6.8, odd 999983 x 17 90 -> 15.5 (4.4 TB/s).
+// windows could leave the matrix, are read one element at a time.  FP32 is held to 32
+// registers there, for a full SM (999983 x 17 20.6 -> 15.8 us).
+// Tile-per-block -> this (us, L2 cold): FP32 1000000 x 8 16.0 -> 6.2, 2000000 x 30 49.9 ->
+// 36.8 (6.5 TB/s), odd 999983 x 17 82 -> 15.8; BF16 2000000 x 30 34.5 -> 19.2; FP64 odd
+// 700001 x 8 63 -> 18.5.
 template <typename T, int V, bool SHIFT>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kGemvTallBlock, SHIFT && sizeof(T) == 4 ? 8 : 4)
 gemv_tall_kernel(T *__restrict__ y, const T *__restrict__ A, const T *__restrict__ x, int64_t m,
                  int64_t n, int64_t lda, typename Acc<T>::type alpha,
                  typename Acc<T>::type beta, bool y_ok) {
-    LAK_PDL_ENTRY();
+    LAK_PDL_WAIT();
     using Ac = typename Acc<T>::type;
     const int64_t r0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * V;
     if (r0 >= m) return;
@@ -262,20 +268,58 @@ gemv_tall_kernel(T *__restrict__ y, const T *__restrict__ A, const T *__restrict
         j = 1;
         j1 = n - 1;
     }
-#pragma unroll(SHIFT ? 4 : 8)
-    for (; j < j1; ++j) {
-        Pack<T, V> pa;
-        const T *p = a + j * lda;
-        if constexpr (SHIFT)
-            load_window<T, CACHED>(pa, p, (uint32_t)((uintptr_t)p % 16));
-        else
-            load_pack<T, V, STREAM>(pa, p);
-        const T xj = ld_cached(x + j);
+    if constexpr (sizeof(T) == 2 || !SHIFT) {
+        // K columns' loads together, then their sum
+        constexpr int K = SHIFT ? 4 : kGemvTallOneSum;
+        auto columns = [&](int64_t j, int count, auto whole) {
+            Pack<T, V> pa[K];
+            T xj[K];
 #pragma unroll
-        for (int v = 0; v < V; ++v) acc[v] = fma_wide(pa.e[v], xj, acc[v]);
+            for (int i = 0; i < K; ++i) {
+                if (!whole.value && i >= count) break;
+                const T *p = a + (j + i) * lda;
+                xj[i] = ld_cached(x + j + i);
+                if constexpr (SHIFT)
+                    load_window<T, CACHED>(pa[i], p, (uint32_t)((uintptr_t)p % 16));
+                else
+                    load_pack<T, V, STREAM>(pa[i], p);
+            }
+            Ac t[V];
+#pragma unroll
+            for (int v = 0; v < V; ++v) t[v] = Ac(0);
+#pragma unroll
+            for (int i = 0; i < K; ++i) {
+                if (!whole.value && i >= count) break;
+#pragma unroll
+                for (int v = 0; v < V; ++v) t[v] = fma_wide(pa[i].e[v], xj[i], t[v]);
+            }
+#pragma unroll
+            for (int v = 0; v < V; ++v) acc[v] += t[v];
+        };
+        for (; j + K <= j1; j += K) columns(j, K, Flag<true>{});
+        if (j < j1) columns(j, (int)(j1 - j), Flag<false>{});
+    } else {
+        while (j < j1) {
+            const int64_t je = j + kGemvTallOneSum < j1 ? j + kGemvTallOneSum : j1;
+            Ac t[V];
+#pragma unroll
+            for (int v = 0; v < V; ++v) t[v] = Ac(0);
+#pragma unroll 4
+            for (; j < je; ++j) {
+                Pack<T, V> pa;
+                const T *p = a + j * lda;
+                load_window<T, CACHED>(pa, p, (uint32_t)((uintptr_t)p % 16));
+                const T xj = ld_cached(x + j);
+#pragma unroll
+                for (int v = 0; v < V; ++v) t[v] = fma_wide(pa.e[v], xj, t[v]);
+            }
+#pragma unroll
+            for (int v = 0; v < V; ++v) acc[v] += t[v];
+        }
     }
     if constexpr (SHIFT)
         if (n > 1) scalar_column(n - 1);
+    LAK_PDL_TRIGGER();
     Pack<T, V> py;
     if (beta != Ac(0)) {
         if (y_ok) {

@@ -497,11 +497,12 @@ size_t rows_ws_most(lak_dtype dt, int64_t m, int64_t n, const lak_cfg *cfg) {
 
 // Column-major products with very many rows and few columns, a thread per 16 bytes
 // of rows (gemv_tall_kernel): from 768 threads per SM on.  Timed against the
-// tile-per-block kernel (us): 2097152 x 30 FP64 134 -> 122, FP32 56 -> 39; 999983 x 17
-// FP32 (odd) 90 -> 15.5; 500000 x 50 FP32 (820 threads per SM) 21.8 -> 17.9; 300000 x
-// 1000 FP32 (490) 173 -> 235.  With more columns the tiles' combine no longer shows.
+// tile-per-block kernel (us): 2000000 x 30 FP32 50 -> 37, BF16 34 -> 19; 999983 x 17 FP32
+// (odd) 82 -> 15.8; 500000 x 50 FP32 (820 threads per SM) 22.7 -> 16.3; 300000 x 1000 FP32
+// (490) 173 -> 235.  With more columns the tiles' combine no longer shows.  FP64 as far as
+// its columns are one sum: 700001 x 8 63 -> 18.5, 1000000 x 8 27.5 -> 22.9.
 bool use_gemv_tall(lak_dtype dt, int64_t m, int64_t n, const lak_cfg *cfg) {
-    if (n < 1 || n > 64 || m < 65536) return false;
+    if (n < 1 || n > (dt == LAK_F64 ? kGemvTallOneSum : 64) || m < 65536) return false;
     const DeviceInfo *di = device_info();
     if (!di || m * esize(dt) / 16 < 768LL * di->sms) return false;
     return builtin_shape(LAK_OP_GEMV_COL, dt, bucket_of(op_bytes(LAK_OP_GEMV_COL, dt, m, n, 0)),
@@ -519,7 +520,8 @@ bool use_gemv_tall(lak_dtype dt, int64_t m, int64_t n, const lak_cfg *cfg) {
 //   FP64 from 2000 rows and 700 columns up to 512 MiB, eight blocks per SM: 2001 x 2000
 //     18.8, 18.8 (19.0 -> 16.2), 3001 x 5000 54.4 -> 40.4, 7999 x 8000 209 -> 139; 16383 x
 //     500 20 -> 23, 16383 x 16384 554 -> 568; and where the tiles alone fill the GPU
-//     (1216): 100003 x 200 55 -> 44
+//     (1216): 100003 x 200 55 -> 44, 130001 x 17 17.0 -> 10.4; with few columns up to
+//     64 MiB: 999983 x 17 47 -> 75
 // Eight columns per warp and split at least, for the last block's sums over the splits.
 int plan_gemv_col_off(lak_dtype dt, int64_t m, int64_t n, const lak_cfg *cfg) {
     const int es = esize(dt), v = 16 / es;
@@ -527,7 +529,7 @@ int plan_gemv_col_off(lak_dtype dt, int64_t m, int64_t n, const lak_cfg *cfg) {
     const int bucket = bucket_of(bytes);
     if (bytes < (1 << 20) || m < (es == 4 ? 8 * v : 2000) || n < 8) return 0;
     const int64_t tiles = ceil_div(m, 31LL * v);
-    if (es == 8 && tiles < 1216 && (n < 700 || bucket > 2)) return 0;
+    if (es == 8 && (tiles < 1216 ? n < 700 || bucket > 2 : n <= 64 && bucket > 1)) return 0;
     if (!builtin_shape(LAK_OP_GEMV_COL, dt, bucket, cfg)) return 0;
     const DeviceInfo *di = device_info();
     if (!di) return 0;

@@ -172,8 +172,10 @@ struct RowsLaunch {
 lak_status launch_gemv_rows(lak_dtype dt, void *y, const void *A, const void *x, int64_t m,
                             int64_t n, int64_t lda, const RowsLaunch &L, void *ws, double alpha,
                             double beta, cudaStream_t s);
-// Column-major product with very many rows: a thread per 16 bytes of rows.
+// Column-major product with very many rows: a thread per 16 bytes of rows; columns that
+// it takes as one sum.
 constexpr int kGemvTallBlock = 256;
+constexpr int kGemvTallOneSum = 8;
 lak_status launch_gemv_tall(lak_dtype dt, void *y, const void *A, const void *x, int64_t m,
                             int64_t n, int64_t lda, double alpha, double beta, cudaStream_t s);
 // Column-major product whose columns start off 16 bytes; splits > 1 as above.
