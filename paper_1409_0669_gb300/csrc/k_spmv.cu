@@ -95,15 +95,16 @@ spmv_kernel(T *__restrict__ y, const int32_t *__restrict__ rp, const int32_t *__
 // One lane group's row: the G lanes of a group stride through its entries U at a time,
 // `longest` (uniform over the warp) bounding the steps so that slots no row of the warp
 // fills are not issued -- in FP64 a predicated-off FMA costs as much as a full one.
-// FP32 keeps two partial sums, FP64 one chain.  All 32 lanes call it; every lane of a
-// group returns the row's sum.
+// FP32 keeps two partial sums; FP64 as many as leave its chains no longer than those of
+// the one-row form, which has more lanes per row (with one chain in 4 lanes rows of 81 were
+// 30 % further off).  All 32 lanes call it; every lane of a group returns the row's sum.
 template <typename T, int G, int U, int P>
 __device__ __forceinline__ typename Acc<T>::type group_row(const int32_t *__restrict__ c,
                                                            const T *__restrict__ v,
                                                            const T *__restrict__ x, int32_t len,
                                                            int32_t longest, int lg) {
     using Ac = typename Acc<T>::type;
-    constexpr int S = sizeof(Ac) == 8 ? 1 : 2;              // partial sums
+    constexpr int S = sizeof(Ac) != 8 ? 2 : G <= 8 ? 4 : G == 16 ? 2 : 1;   // partial sums
     using Step = uint32_t;
     Ac acc[S];
 #pragma unroll
@@ -130,7 +131,11 @@ __device__ __forceinline__ typename Acc<T>::type group_row(const int32_t *__rest
             }
         }
     }
-    if constexpr (S == 2) acc[0] += acc[1];
+#pragma unroll
+    for (int w = 1; w < S; w <<= 1) {
+#pragma unroll
+        for (int i = 0; i + w < S; i += 2 * w) acc[i] += acc[i + w];
+    }
     return group_sum(acc[0], G);
 }
 
@@ -138,10 +143,11 @@ __device__ __forceinline__ typename Acc<T>::type group_row(const int32_t *__rest
 // whose longest row is far from the mean of its rows takes them one by one with all
 // its lanes instead.  FP64 is bound by the pipe's warp instructions, so fewer lanes per
 // row than the one-row form's serve it: 81 entries in 16 lanes took 8 FMAs (2 of them
-// for slots no row fills) and 4 adds for two rows, in 4 lanes 21 and 2 for eight.
-// Measured (us, one-row groups -> this; 41 M entries of a 3D elasticity matrix, L2 cold):
-// FP64 196 -> 108 (4.7 TB/s; FP64 pipe 78), FP32 90 -> 66, BF16 111 -> 59; rows with a
-// heavy tail (up to 50000 entries, mean 76) as before (FP64 899 -> 865, FP32 441 -> 411).
+// for slots no row fills) and 4 adds for two rows, in 4 lanes 21 and 5 for eight.
+// Measured (us, one-row groups -> this; 41 M entries in rows of 81 near the diagonal, L2
+// cold): FP64 187 -> 116, FP32 88 -> 70, BF16 106 -> 62; random columns FP64 186 -> 190;
+// rows with a heavy tail (up to 50000 entries, mean 76) as before (FP64 899 -> 865, FP32
+// 441 -> 411).
 template <typename T, int G>
 __global__ void __launch_bounds__(kSpmvLongBlock)
 spmv_long_kernel(T *__restrict__ y, const int32_t *__restrict__ rp,

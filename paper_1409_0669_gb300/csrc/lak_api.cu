@@ -628,17 +628,30 @@ lak_status plan_spmv(lak_dtype dt, int64_t m, int64_t n, int64_t nnz, const lak_
     if (mean > 64 && !seg && builtin_shape(LAK_OP_SPMV, dt, bucket, cfg)) {
         // lanes per row by the mean row length, where they were timed (us): mean 81
         // (elasticity) FP64 4 lanes 107, 8 lanes 119; FP32 4 and 8 lanes 65, 16 lanes 79;
-        // mean 130 (65..200) FP64 8 lanes 129, 4 lanes 141, 16 lanes 139; FP32 74, 88, 78;
-        // mean 600 FP64 32 lanes 131, 16 lanes 144; FP32 99 and 111
+        // mean 130 (65..200) FP64 8 lanes 129, 4 lanes 141, 16 lanes 139; FP32 74, 88, 78
+        // (16 lanes taken: two sums in 8 lanes are further off than the general kernel);
+        // mean 600 FP64 32 lanes 131, 16 lanes 144
         // With fewer rows more lanes, so that the chip has warps enough (elasticity of 3000
         // rows FP64 8 lanes 2.9, 4 lanes 4.2; FP32 32 lanes 1.8, 8 lanes 2.3; 50000 rows of
         // 66..130 random columns FP32 16 lanes 14.0, 8 lanes 17.0; FP64 8 lanes 21.0, 4
         // lanes 25.4; elasticity of 41472 rows FP32 5.6 and 5.2, FP64 10.5 and 10.0)
-        int G = mean > 320 ? 32 : mean > 160 ? 16 : mean > 100 || dt != LAK_F64 ? 8 : 4;
+        int G = mean > 320 ? 32 : mean > 160 ? 16 : dt != LAK_F64 ? (mean > 100 ? 16 : 8)
+                                                                  : mean > 100 ? 8 : 4;
         const int least = m >= 262144 ? 4 : m >= 65536 || dt == LAK_F64 ? 8 : m >= 8192 ? 16 : 32;
         if (G < least) G = least;
+        // FP32 rows beyond a mean of 160 stay with the general kernel, which is as fast and
+        // more accurate on its 128 chains (mean 550 45.0, here 45.4; 2500 45.6, 47.0); 16-bit
+        // ones beyond 700 (2500 41, 47) and with fewer than 50000 rows (300 x 20000 11.5, 13.4)
+        bool take = dt == LAK_F64 || mean <= 160 || (dt != LAK_F32 && mean <= 700 && m >= 50000);
+        // FP64 with too few warps to hide a row's steps behind other rows: three steps of four
+        // entries per lane at most, or the general kernel with its eight (3000 rows of 128: 8
+        // lanes 7.2, 16 lanes 4.3, general 4.8; 1000 of 750: 11.8, general 9.8)
+        if (dt == LAK_F64 && m * G < 32LL * 32 * di->sms) {
+            while (G < 32 && mean > 12LL * G) G *= 2;
+            if (mean > 12LL * G) take = false;
+        }
         int64_t blocks = ceil_div(m * G, kSpmvLongBlock);
-        if (blocks <= 0x7fffffff) {
+        if (take && blocks <= 0x7fffffff) {
             out->L = Launch{kSpmvLongBlock, (int)blocks, 4, LAK_INC_GLOBAL};
             out->group = G;
             out->long_rows = true;

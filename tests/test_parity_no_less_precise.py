@@ -28,6 +28,44 @@ def rms(y, exact):
     return float(d.square().mean().sqrt())
 
 
+def csr(lo, hi, m, seed=5):
+    g = gen(seed)
+    lens = torch.randint(lo, hi, (m,), device="cuda", generator=g)
+    rp = torch.zeros(m + 1, dtype=torch.int32, device="cuda")
+    rp[1:] = torch.cumsum(lens, 0)
+    ci = torch.randint(0, m, (int(rp[-1]),), device="cuda", generator=g).int()
+    return rp, ci, torch.repeat_interleave(torch.arange(m, device="cuda"), lens)
+
+
+@pytest.mark.parametrize("lo, hi, m", [(81, 82, 300_000), (66, 100, 270_000), (81, 82, 20_000),
+                                       (105, 150, 70_000), (170, 256, 40_000)])
+def test_long_rows_f64(lo, hi, m):
+    rp, ci, row = csr(lo, hi, m)
+    g = gen(6)
+    # products of up to 2^54, 256 of them within 63 bits
+    v = torch.randint(-2 ** 30, 2 ** 30, ci.shape, device="cuda", generator=g)
+    x = torch.randint(-2 ** 24, 2 ** 24, (m,), device="cuda", generator=g)
+    exact = torch.zeros(m, dtype=torch.int64, device="cuda").index_add_(0, row, v * x[ci.long()])
+    args = (rp, ci, v.double(), x.double())
+    err = rms(lak().csr_spmv(*args), exact)
+    general = rms(lak().csr_spmv(*args, cfg=(64, 16 * SMS, 8, 0)), exact)
+    assert 0 < err <= SLACK * general, (err, general)
+
+
+@pytest.mark.parametrize("lo, hi, m", [(81, 82, 300_000), (105, 150, 100_000), (140, 181, 70_000),
+                                       (400, 700, 20_000), (2000, 3000, 20_000)])
+def test_long_rows_f32(lo, hi, m):
+    rp, ci, row = csr(lo, hi, m)
+    g = gen(6)
+    v = torch.randn(ci.shape, device="cuda", generator=g)
+    x = torch.rand(m, device="cuda", generator=g) * 2 - 1
+    exact = torch.zeros(m, dtype=torch.float64, device="cuda").index_add_(
+        0, row, v.double() * x.double()[ci.long()])
+    err = rms(lak().csr_spmv(rp, ci, v, x), exact)
+    general = rms(lak().csr_spmv(rp, ci, v, x, cfg=(128, 16 * SMS, 4, 0)), exact)
+    assert 0 < err <= SLACK * general, (err, general)
+
+
 def dense(m, n, layout):
     g = gen(7)
     A = torch.randn(m * n, device="cuda", generator=g)
