@@ -312,10 +312,12 @@ struct VecPlan {
 };
 
 lak_status plan_vector(lak_op op, lak_dtype dt, int64_t n, const lak_cfg *cfg,
-                       const void *const *ptrs, int nptrs, VecPlan *out) {
+                       const void *const *ptrs, int nptrs, VecPlan *out,
+                       bool compensated = false) {
     const DeviceInfo *di = device_info();
     if (!di) return LAK_ECUDA;
-    const int bucket = bucket_of(op_bytes(op, dt, n, n, 0));
+    const int64_t bytes = op_bytes(op, dt, n, n, 0);
+    const int bucket = bucket_of(bytes);
     lak_cfg c = base_cfg(op, dt, bucket, cfg);
     const int es = esize(dt);
     int want = c.vec ? c.vec : builtin_default(op, dt, bucket).vec;
@@ -325,9 +327,13 @@ lak_status plan_vector(lak_op op, lak_dtype dt, int64_t n, const lak_cfg *cfg,
     // entries, L2 cold): BF16 update 44.8 -> 22.3, copy 22.3 -> 15.1, inner product 28.2 ->
     // 19.4; FP32 update 56.0 -> 41.9, copy 31.4 -> 27.8.  The FP32 inner product keeps its
     // one-element accesses (1e8 entries: 121 against 146 us), and FP64, whose warps read
-    // whole lines that way, too (update 86.0 against 88.5 us).
+    // whole lines that way, too (update 86.0 against 88.5 us).  So do calls too small for
+    // the windows' longer way to a result (FP32 update of 30,000 entries 1.7 against 2.2),
+    // and the compensated inner product below 64 MiB, where a thread's eight sums cost more
+    // to join than they save (BF16, 2,097,152 entries 9.1 against 15.7; 6e7 70 -> 55).
     const bool unlike = ptrs && vec * es < 16 && want * es >= 16;
-    const bool shifted = unlike && es <= (op == LAK_OP_DOT ? 2 : 4) &&
+    const bool pays = op != LAK_OP_DOT ? bytes >= 1 << 20 : !compensated || bucket >= 2;
+    const bool shifted = unlike && pays && es <= (op == LAK_OP_DOT ? 2 : 4) &&
                          shifted_head(es, ptrs, nptrs, n, &head);
     if (shifted) vec = 16 / es;
     const int64_t nchunks = vec > 0 ? (n - head) / vec : n;
@@ -337,8 +343,9 @@ lak_status plan_vector(lak_op op, lak_dtype dt, int64_t n, const lak_cfg *cfg,
         const int per_sm = default_grid_per_sm(op, dt, bucket);
         int64_t cap = per_sm > 0 ? (int64_t)per_sm * di->sms : waves_grid(di, c.block);
         // the table's caps go with its pack widths: narrower accesses take as many more
-        // blocks, up to a full SM (FP32 dot of 21.5 M entries 49.9 -> 29.7 us)
-        if (unlike && es <= 4) {
+        // blocks, up to a full SM (FP32 dot of 21.5 M entries 49.9 -> 29.7 us; one-element
+        // accesses from 64 MiB on, 8 M entries in L2 8.8 against 10.5)
+        if (unlike && es <= 4 && (shifted || bucket >= 2)) {
             const int64_t more = cap * (want * es / 16);
             const int64_t most = waves_grid(di, c.block);
             cap = more < most ? more : cap > most ? cap : most;
@@ -1050,7 +1057,7 @@ LAK_API lak_status vec_dot_compensated(double *out, const void *x, const void *y
         return fail(LAK_EINVAL, "vec_dot_compensated: pointers not aligned to the element size");
     const void *ptrs[2] = {x, y};
     VecPlan p;
-    st = plan_vector(LAK_OP_DOT, dtype, n, cfg, ptrs, 2, &p);
+    st = plan_vector(LAK_OP_DOT, dtype, n, cfg, ptrs, 2, &p, true);
     if (st != LAK_OK) return st;
     const size_t need = (size_t)LAK_WS_COUNTER_BYTES + 8 * (size_t)p.L.grid;
     if (!workspace || ws_bytes < need)
