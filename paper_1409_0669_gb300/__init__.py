@@ -30,8 +30,10 @@ try:
     # direct calls for the common forms (csrc/py_fast.cpp); each returns None where the
     # Python path has to take the call
     from . import _fast
-except ImportError:             # built against another torch: the Python paths serve all
+except ImportError:             # not built: the Python paths serve all
     _fast = None
+if _fast is not None and _fast.torch_version != torch.__version__:
+    _fast = None                # it reads tensors as the torch that it was compiled for lays them out
 
 __all__ = ["vec_copy", "vec_axpy", "vec_axpby", "vec_axpy_norm2", "vec_axpy_norm2_workspace",
            "dense_gemv_trans", "vec_dot", "vec_dot_workspace", "vec_dot_sparse",

@@ -5,18 +5,22 @@ Each translation unit under ``csrc/`` is compiled by nvcc in parallel into
 ``_build/`` and linked (static CUDA runtime) into a shared library beside this
 file; the extension (``csrc/py_fast.cpp``) is compiled by g++ against the
 installed torch's headers and linked against that library.  A rebuild happens
-only when a source or header is newer than the results, unless ``force`` is
-set.
+only when a source or header is newer than the results, or the installed torch is
+another one than the extension was compiled for, unless ``force`` is set.  An
+extension that cannot be compiled is left out with a warning: the package works
+without it, through ctypes.
 """
 from __future__ import annotations
 
 import concurrent.futures
 import importlib.util
 import os
+import re
 import shutil
 import subprocess
 import sysconfig
 import tempfile
+import warnings
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
@@ -25,6 +29,7 @@ INCLUDE = os.path.join(ROOT, "include")
 OBJDIR = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "liblak_gb300.so")
 FAST = os.path.join(PKG, "_fast" + sysconfig.get_config_var("EXT_SUFFIX"))
+FAST_STAMP = os.path.join(OBJDIR, "py_fast.torch")    # torch it was last compiled (or tried) for
 ARCH = "-gencode=arch=compute_103a,code=sm_103a"
 SOURCES = ["lak_api.cu", "k_vec.cu", "k_gemv.cu", "k_gemv_wide.cu", "k_spmv.cu", "k_dot_noalloc.cu", "k_batch.cu", "k_grad.cu", "k_transpose.cu", "k_vec_ext.cu", "k_sell.cu", "k_csr_bin.cu", "k_probe.cu"]
 
@@ -47,9 +52,13 @@ def _deps():
 
 
 def up_to_date() -> bool:
-    if not os.path.exists(LIB) or not os.path.exists(FAST):
+    if not os.path.exists(LIB) or not os.path.exists(FAST_STAMP):
         return False
-    t = min(os.path.getmtime(LIB), os.path.getmtime(FAST))
+    with open(FAST_STAMP) as fh:
+        version, _, failed = fh.read().partition(" ")
+    if version != torch_version() or (not failed and not os.path.exists(FAST)):
+        return False
+    t = min(os.path.getmtime(f) for f in ([LIB, FAST_STAMP] if failed else [LIB, FAST_STAMP, FAST]))
     return all(os.path.getmtime(f) <= t for f in _deps())
 
 
@@ -65,12 +74,22 @@ def torch_dir() -> str:
     return list(spec.submodule_search_locations)[0]
 
 
+def torch_version() -> str:
+    """The installed torch's version, read without importing it."""
+    with open(os.path.join(torch_dir(), "version.py")) as fh:
+        found = re.search(r"""^__version__\s*=\s*['"]([^'"]+)""", fh.read(), re.M)
+    if not found:
+        raise RuntimeError("torch/version.py names no version")
+    return found.group(1)
+
+
 def compile_fast() -> str:
     """Object file of the Python extension."""
     inc = os.path.join(torch_dir(), "include")
     cuda = os.path.join(os.path.dirname(os.path.dirname(nvcc_path())), "include")
     obj = os.path.join(OBJDIR, "py_fast.o")
-    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-fvisibility=hidden", "-I", INCLUDE, "-I", inc,
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-fvisibility=hidden",
+           f'-DLAK_TORCH_VERSION="{torch_version()}"', "-I", INCLUDE, "-I", inc,
            "-I", os.path.join(inc, "torch", "csrc", "api", "include"), "-I", cuda, "-I",
            sysconfig.get_paths()["include"], "-c", os.path.join(CSRC, "py_fast.cpp"), "-o", obj]
     r = subprocess.run(cmd, capture_output=True, text=True)
@@ -110,7 +129,6 @@ def build(force: bool = False, verbose: bool = False, ptxas_verbose: bool = Fals
     with concurrent.futures.ThreadPoolExecutor(max_workers=len(SOURCES) + 1) as ex:
         fast = ex.submit(compile_fast)
         results = list(ex.map(one, SOURCES))
-        fast_obj = fast.result()
     if verbose or ptxas_verbose:
         for _, log in results:
             if log:
@@ -123,7 +141,16 @@ def build(force: bool = False, verbose: bool = False, ptxas_verbose: bool = Fals
         os.unlink(tmp)
         raise RuntimeError(f"link failed:\n{r.stderr}")
     os.replace(tmp, LIB)
-    link_fast(fast_obj)
+    stamp = torch_version()
+    try:
+        link_fast(fast.result())
+    except Exception as e:              # g++, torch's headers or its libraries
+        warnings.warn(f"built without the Python extension: {e}")
+        stamp += " failed"
+        if os.path.exists(FAST):        # of other sources or another torch
+            os.unlink(FAST)
+    with open(FAST_STAMP, "w") as fh:
+        fh.write(stamp)
     return LIB
 
 

@@ -423,4 +423,8 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_fast", nullptr, -1, methods, null
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__fast(void) { return PyModule_Create(&module); }
+PyMODINIT_FUNC PyInit__fast(void) {
+    PyObject *m = PyModule_Create(&module);
+    if (m && PyModule_AddStringConstant(m, "torch_version", LAK_TORCH_VERSION) < 0) Py_CLEAR(m);
+    return m;
+}
