@@ -75,20 +75,24 @@ struct CsrItem {
 };
 
 // CSR instances (FP32 and 16-bit storage) whose x fits in one SM's shared memory are taken
-// by spmv_staged_kernel, in plans without a configuration of the caller's.  spmv_batch_kernel is bound by
-// its gathers through L1 (one lane per clock and SM: 262 G entries/s) and, on short rows,
-// by the walk over their ends; shared memory serves about nine random lanes per clock.
-// Measured in G entries/s, spmv_batch_kernel against the staged one:
-//   1000 x 20000 rows of 5..64, random columns   FP32 267 -> 438   BF16 303 -> 471
-//   the same, columns within 64 of the diagonal  FP32 369 -> 447   BF16 427 -> 497
-//   300 x 30000 rows of 150..250                 FP32 301 -> 513   BF16 394 -> 563
-//   4096 x 4000 rows of 8..10                    FP32 142 -> 280   BF16 163 -> 297
-//   2000 x 20000 rows of 2                       FP32  53 ->  81   BF16  57 ->  82
-// 1024 instances of 1000..200000 rows of 5..64: FP32 5076 -> 4640 us (26 % of the rows
-// staged), BF16 4533 -> 3741 us (51 %).  FP32 rows of fewer than 16 entries stay with
-// spmv_batch_kernel all the same: the staged kernel rounds a product before it adds it,
-// which costs 1 % of accuracy at 9 entries and 17 % at 2 (from 16 on its shorter chains
-// more than make up for it; products of 16-bit values are exact in FP32).  FP64 stays
+// by spmv_staged_kernel, in plans without a configuration of the caller's.
+// spmv_batch_kernel is bound by its gathers through L1 (one lane per clock and SM: 262 G
+// entries/s) and, on short rows, by the walk over their ends; shared memory serves about
+// nine random lanes per clock.  Measured in G entries/s, spmv_batch_kernel against the
+// staged one:
+//   1000 x 20000 rows of 5..64, random columns   FP32 272 -> 412   BF16 309 -> 477
+//   the same, columns within 64 of the diagonal  FP32 377 -> 420   BF16 437 -> 500
+//   300 x 30000 rows of 150..250                 FP32 331 -> 497   BF16 396 -> 574
+//   4096 x 4000 rows of 8..10                    FP32 stay, 149    BF16 170 -> 339
+//   2000 x 20000 rows of 2                       FP32 stay, 56     BF16  61 ->  96
+// 1024 instances of 1000..200000 rows of 5..64: FP32 5056 -> 4679 us (26 % of the rows
+// staged), BF16 4533 -> 3741 us (51 %).  The staged kernel rounds a product before it adds
+// it (products of 16-bit values are exact in FP32), which would cost 17 % of accuracy on
+// FP32 rows of 2 entries and 1 % on rows of 9; from 16 on its shorter chains more than make
+// up for it.  So FP32 instances of fewer than 16 entries a row stay with spmv_batch_kernel,
+// and rows of up to kStageShort entries inside the others are taken by FMAs (7 % of the
+// time at 5..64).  Both factors of every entry in the buffer instead, one FMA each, took 36
+// to 42 % more (700 x 20000 rows of 5..64 1082 -> 1467 us).  FP64 stays
 // there too: one multiplication and one addition per entry in place of an FMA, the latter
 // with few lanes at work, made it 1.3 to 3.1 times slower.  Instances of fewer than
 // kStageMinEntries do not pay for looking up their unit (16000 of 5000 entries: 499 ->
@@ -98,6 +102,7 @@ constexpr int kStageBlock = 16;                       // rows that a warp takes 
 constexpr int kStageQuads = 2;                        // 4 entries each, per lane and step
 constexpr int kStageStep = 128 * kStageQuads;         // entries of a warp's step
 constexpr int kStageLong = 96;                        // a row's part that the whole warp sums
+constexpr int kStageShort = 8;                        // FP32 rows taken as one chain of FMAs
 constexpr int64_t kStageEntries = 131072;             // of a unit, about
 constexpr int64_t kStageMinEntries = 32768;           // of an instance
 constexpr int64_t kStageMinUnits = 152 * 4;
@@ -611,6 +616,28 @@ __device__ __forceinline__ void staged_load(StagedStep<T> &st, const StagedUnit 
     }
 }
 
+// An FP32 row of kStageShort entries at most, as one chain of FMAs from its own entries:
+// products rounded before they are added cost up to 17 % of accuracy on such rows.
+__device__ __forceinline__ float staged_short(const StagedUnit &un, const float *xs, uint32_t k0,
+                                              uint32_t k1) {
+    const float *vals = static_cast<const float *>(un.vals);
+    float acc = 0.0f;
+    for (; k0 < k1; k0 += 4) {
+        int32_t col[4];
+        float val[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t)
+            if (k0 + t < k1) {
+                col[t] = __ldg(un.ci + k0 + t);
+                val[t] = __ldg(vals + k0 + t);
+            }
+#pragma unroll
+        for (int t = 0; t < 4; ++t)
+            if (k0 + t < k1) acc = fma_acc(val[t], xs[col[t]], acc);
+    }
+    return acc;
+}
+
 // A warp's share of a unit, blocks of kStageBlock rows taken one by one: the products of
 // kStageStep entries at a time go to `buf`; two lanes then sum the part of a row that lies
 // there, in four chains each (the whole warp, where that part is longer than kStageLong).
@@ -709,6 +736,8 @@ __device__ __forceinline__ void staged_unit(StagedUnit &un, const T *xs, float *
         } while (!last);
         acc += __shfl_xor_sync(0xffffffffu, acc, 1);
         const int64_t row = (int64_t)b * kStageBlock + (lane >> 1);
+        if constexpr (sizeof(T) == 4)
+            if ((lane & 1) == 0 && k1 - k0 - 2 <= kStageShort - 2) acc = staged_short(un, xs, k0, k1);
         if ((lane & 1) == 0 && row < m) static_cast<T *>(un.y)[row] = narrow<T>(acc);
         if (!more) return;
         b = b2;
