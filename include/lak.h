@@ -490,8 +490,9 @@ LAK_API lak_status csr_transpose(int32_t *col_ptr, int32_t *row_idx, int32_t *pe
                                  int64_t n, int64_t nnz, void *workspace, size_t ws_bytes,
                                  void *stream);
 
-/* Workspace bytes csr_transpose_vals needs: a 16-byte record per entry (two beyond about
- * 1024 blocks of columns) and the partition's counts.  No counterpart in the paper. */
+/* Workspace bytes csr_transpose_vals needs: a 16-byte record per entry (two beyond
+ * 1024 blocks of columns) and the partition's counts, a byte per entry at most.
+ * No counterpart in the paper. */
 LAK_API size_t csr_transpose_vals_workspace(int64_t n, int64_t nnz, lak_dtype dtype);
 
 /* csr_transpose with the values carried along: vals_t[q] = vals[perm[q]], bit copies of

@@ -9,7 +9,7 @@
 //   gemv_col_off_kernel  column-major, columns off 16 bytes: every warp takes columns
 //                      of one offset and shifts its rows by it
 //
-// Both compute y = alpha * A x + beta * y (y is not read when beta == 0).
+// All compute y = alpha * A x + beta * y (y is not read when beta == 0).
 #include "lak_internal.cuh"
 
 namespace lak {

@@ -315,13 +315,7 @@ lak_status outer_t(void *dA, const void *dy, const void *x, int64_t m, int64_t n
     return check_launch("dense_outer");
 }
 
-bool valid_dt(lak_dtype dt) { return dt == LAK_F32 || dt == LAK_F64 || dt == LAK_BF16 || dt == LAK_F16; }
-
-}  // namespace
-}  // namespace lak
-
-namespace lak {
-
+// Inclusive scan of v[0..len) in place; sums: scan_scratch_ints(len) ints.
 int64_t scan_scratch_ints(int64_t len) {
     const int64_t tiles = (len + kScanTile - 1) / kScanTile;
     const int64_t tiles2 = (tiles + kScanTile - 1) / kScanTile;
@@ -343,6 +337,9 @@ void launch_scan_i32(int32_t *v, int64_t len, int32_t *sums, cudaStream_t s) {
     }
 }
 
+bool valid_dt(lak_dtype dt) { return dt == LAK_F32 || dt == LAK_F64 || dt == LAK_BF16 || dt == LAK_F16; }
+
+}  // namespace
 }  // namespace lak
 
 using namespace lak;

@@ -527,7 +527,7 @@ bool use_gemv_tall(lak_dtype dt, int64_t m, int64_t n, const lak_cfg *cfg) {
 //   FP64 from 2000 rows and 700 columns up to 512 MiB, eight blocks per SM: 2001 x 2000
 //     18.8, 18.8 (19.0 -> 16.2), 3001 x 5000 54.4 -> 40.4, 7999 x 8000 209 -> 139; 16383 x
 //     500 20 -> 23, 16383 x 16384 554 -> 568; and where the tiles alone fill the GPU
-//     (1216): 100003 x 200 55 -> 44, 130001 x 17 17.0 -> 10.4; with few columns up to
+//     (eight per SM): 100003 x 200 55 -> 44, 130001 x 17 17.0 -> 10.4; with few columns up to
 //     64 MiB: 999983 x 17 47 -> 75
 // Eight columns per warp and split at least, for the last block's sums over the splits.
 int plan_gemv_col_off(lak_dtype dt, int64_t m, int64_t n, const lak_cfg *cfg) {
@@ -536,10 +536,10 @@ int plan_gemv_col_off(lak_dtype dt, int64_t m, int64_t n, const lak_cfg *cfg) {
     const int bucket = bucket_of(bytes);
     if (bytes < (1 << 20) || m < (es == 4 ? 8 * v : 2000) || n < 8) return 0;
     const int64_t tiles = ceil_div(m, 31LL * v);
-    if (es == 8 && (tiles < 1216 ? n < 700 || bucket > 2 : n <= 64 && bucket > 1)) return 0;
-    if (!builtin_shape(LAK_OP_GEMV_COL, dt, bucket, cfg)) return 0;
     const DeviceInfo *di = device_info();
     if (!di) return 0;
+    if (es == 8 && (tiles < 8LL * di->sms ? n < 700 || bucket > 2 : n <= 64 && bucket > 1)) return 0;
+    if (!builtin_shape(LAK_OP_GEMV_COL, dt, bucket, cfg)) return 0;
     const int64_t per_sm = es == 8 || (es == 2 && bucket == 3) ? 8 : es == 4 ? 6 : 4;
     int64_t splits = per_sm * di->sms / tiles;
     const int64_t most = n / (8 * (kGemvOffBlock / 32));

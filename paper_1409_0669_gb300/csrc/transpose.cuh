@@ -1,13 +1,9 @@
-// Shared by the CSR transpose's two forms (k_grad.cu, k_transpose.cu).
+// The CSR transpose's stable partition (k_transpose.cu) for its entry points (k_grad.cu).
 #pragma once
 
 #include "lak_internal.cuh"
 
 namespace lak {
-
-// Inclusive scan of v[0..len) in place; sums: scan_scratch_ints(len) ints.
-int64_t scan_scratch_ints(int64_t len);
-void launch_scan_i32(int32_t *v, int64_t len, int32_t *sums, cudaStream_t s);
 
 // Columns the stable partition takes (two passes over column blocks of 2^10).
 constexpr int64_t kTransposeMaxCols = 1LL << 30;
