@@ -753,7 +753,7 @@ __device__ __forceinline__ void staged_unit(StagedUnit &un, const T *xs, float *
 // row blocks one by one.  Thread 0 looks the next unit up meanwhile.  The last block to
 // leave resets the counters.  24 warps of 80 registers and a step of 256 entries: longer
 // steps (512, 768) ran the same rows up to 10 % faster but left less room for x.  Bound
-// by the shared-memory pipe (83 % busy at 1000 x 20000 rows, DRAM 44 %), which gathers,
+// by the shared-memory pipe (83 % busy at 700 x 20000 rows, DRAM 41 %), which gathers,
 // products and row sums share; sums by two lanes interleaved, four or eight lanes per row
 // were slower (1583 against 1590, 1743 and 2056 us).
 template <typename T>
