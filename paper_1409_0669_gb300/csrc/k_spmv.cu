@@ -21,6 +21,8 @@
 // per-warp shared accumulator with one writer per row per chunk -- no atomics,
 // deterministic (the body lives in spmv_seg.cuh, shared with the batched
 // kernel).
+#include <type_traits>
+
 #include "lak_internal.cuh"
 #include "spmv_seg.cuh"
 
@@ -95,41 +97,45 @@ spmv_kernel(T *__restrict__ y, const int32_t *__restrict__ rp, const int32_t *__
 // One lane group's row: the G lanes of a group stride through its entries U at a time,
 // `longest` (uniform over the warp) bounding the steps so that slots no row of the warp
 // fills are not issued -- in FP64 a predicated-off FMA costs as much as a full one.
-// FP32 keeps two partial sums; FP64 as many as leave its chains no longer than those of
-// the one-row form, which has more lanes per row (with one chain in 4 lanes rows of 81 were
-// 30 % further off).  All 32 lanes call it; every lane of a group returns the row's sum.
-template <typename T, int G, int U, int P>
+// S partial sums per lane, at most U: FP32 two, FP64 as many as leave its chains no longer
+// than those of the one-row form, which has more lanes per row (with one chain in 4 lanes
+// rows of 81 were 30 % further off).  All 32 lanes call it; every lane of a group returns
+// the row's sum.
+// Pos, of positions in the row: the step past a row of nearly 2^31 entries must not wrap, so
+// signed ones leave the loop before it and unsigned ones have the room.
+template <typename T, int G, int U, int P, int S, typename Pos>
 __device__ __forceinline__ typename Acc<T>::type group_row(const int32_t *__restrict__ c,
                                                            const T *__restrict__ v,
                                                            const T *__restrict__ x, int32_t len,
                                                            int32_t longest, int lg) {
     using Ac = typename Acc<T>::type;
-    constexpr int S = sizeof(Ac) != 8 ? 2 : G <= 8 ? 4 : G == 16 ? 2 : 1;   // partial sums
-    using Step = uint32_t;
+    constexpr bool wide = std::is_unsigned_v<Pos>;
+    static_assert(wide ? (Pos)0x7fffffff + 32u * U > 0x7fffffffu : 0x80000000u % (G * U) == 0,
+                  "no position of the last step wraps");
     Ac acc[S];
 #pragma unroll
     for (int i = 0; i < S; ++i) acc[i] = Ac(0);
-    // unsigned: the step past a row of nearly 2^31 entries must not wrap
-    static_assert((Step)0x7fffffff + 32 * U > (Step)0x7fffffff, "the last step of the longest row");
-    for (Step base = 0; base < (Step)longest; base += G * U) {
+    for (Pos base = 0; base < (Pos)longest; base += G * U) {
         int32_t col[U];
         T val[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const Step k = base + u * G + lg;
-            if (k < (Step)len) {
+            const Pos k = base + u * G + lg;
+            if (k < (Pos)len) {
                 ld_raw<4, P>(&col[u], c + k);
                 ld_raw<(int)sizeof(T), P>(&val[u], v + k);
             }
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const Step k = base + u * G + lg;
-            if (base + u * G < (Step)longest && k < (Step)len) {    // the first part is uniform
+            const Pos k = base + u * G + lg;
+            if (base + u * G < (Pos)longest && k < (Pos)len) {    // the first part is uniform
                 Ac &a = acc[u % S];
                 a = fma_acc(widen(val[u]), widen(ld_cached(x + col[u])), a);
             }
         }
+        if constexpr (!wide)
+            if (longest - base <= G * U) break;
     }
 #pragma unroll
     for (int w = 1; w < S; w <<= 1) {
@@ -145,16 +151,19 @@ __device__ __forceinline__ typename Acc<T>::type group_row(const int32_t *__rest
 // row than the one-row form's serve it: 81 entries in 16 lanes took 8 FMAs (2 of them
 // for slots no row fills) and 4 adds for two rows, in 4 lanes 21 and 5 for eight.
 // Measured (us, one-row groups -> this; 41 M entries in rows of 81 near the diagonal, L2
-// cold): FP64 187 -> 116, FP32 88 -> 70, BF16 106 -> 62; random columns FP64 186 -> 190;
-// rows with a heavy tail (up to 50000 entries, mean 76) as before (FP64 899 -> 865, FP32
+// cold): FP64 187 -> 116, FP32 87 -> 65, BF16 106 -> 56; random columns FP64 186 -> 190,
+// FP32 167 -> 166; rows with a heavy tail (up to 50000 entries, mean 76) as before (FP64 899 -> 865, FP32
 // 441 -> 411).
-template <typename T, int G>
+template <typename T, int G, int S>
 __global__ void __launch_bounds__(kSpmvLongBlock)
 spmv_long_kernel(T *__restrict__ y, const int32_t *__restrict__ rp,
                  const int32_t *__restrict__ ci, const T *__restrict__ vals,
                  const T *__restrict__ x, int64_t m) {
     LAK_PDL_WAIT();
     using Ac = typename Acc<T>::type;
+    // FP64 in less than a warp measured faster with unsigned positions (500000 rows of 81:
+    // 116 against 120 us), the others with signed ones (FP32 65, 75; FP64 rows of 2500 68, 70)
+    using Pos = std::conditional_t<sizeof(Ac) == 8 && G < 32, uint32_t, int32_t>;
     constexpr int U = 4, rows = 32 / G;
     const int lane = threadIdx.x & 31, lg = lane % G;
     const int64_t row0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * rows;
@@ -170,13 +179,13 @@ spmv_long_kernel(T *__restrict__ y, const int32_t *__restrict__ rp,
     const int64_t total = (int64_t)__ldg(rp + last) - __ldg(rp + row0);
     constexpr int F = rows == 2 ? 3 : 4;                    // twice the factor on the mean
     if (2 * (int64_t)longest * rows <= F * total + 64 * rows) {
-        const Ac t = group_row<T, G, U, CACHED>(ci + k0, vals + k0, x, len, longest, lg);
+        const Ac t = group_row<T, G, U, CACHED, S, Pos>(ci + k0, vals + k0, x, len, longest, lg);
         if (lg == 0 && row < m) y[row] = narrow<T>(t);
     } else {
         for (int r = 0; r < rows && row0 + r < m; ++r) {
             const int32_t a = __shfl_sync(0xffffffffu, k0, r * G);
             const int32_t n = __shfl_sync(0xffffffffu, len, r * G);
-            const Ac t = group_row<T, 32, U, STREAM>(ci + a, vals + a, x, n, n, lane);
+            const Ac t = group_row<T, 32, U, STREAM, sizeof(Ac) == 8 ? 1 : 2, Pos>(ci + a, vals + a, x, n, n, lane);
             if (lane == 0) y[row0 + r] = narrow<T>(t);
         }
     }
@@ -291,18 +300,27 @@ namespace {
 
 template <typename T>
 lak_status spmv_long_t(void *y, const int32_t *rp, const int32_t *ci, const void *vals,
-                       const void *x, int64_t m, int G, cudaStream_t s) {
+                       const void *x, int64_t m, int G, bool longer, cudaStream_t s) {
     T *yp = static_cast<T *>(y);
     const T *vp = static_cast<const T *>(vals);
     const T *xp = static_cast<const T *>(x);
     const unsigned grid = (unsigned)ceil_div(m * G, kSpmvLongBlock);
-#define LAK_LONG(GG)                                                                        \
-    launch_k(spmv_long_kernel<T, GG>, grid, kSpmvLongBlock, 0, s, yp, rp, ci, vp, xp, m)
-    switch (G) {
-    case 4: LAK_LONG(4); break;
-    case 8: LAK_LONG(8); break;
-    case 16: LAK_LONG(16); break;
-    default: LAK_LONG(32); break;
+#define LAK_LONG(GG, SS)                                                                    \
+    launch_k(spmv_long_kernel<T, GG, SS>, grid, kSpmvLongBlock, 0, s, yp, rp, ci, vp, xp, m)
+    if constexpr (sizeof(T) == 8) {
+        // chains as long as the general kernel's: 8 lanes of rows up to 100 need two of them
+        switch (G) {
+        case 4: LAK_LONG(4, 4); break;
+        case 8: if (longer) LAK_LONG(8, 4); else LAK_LONG(8, 2); break;
+        case 16: LAK_LONG(16, 2); break;
+        default: LAK_LONG(32, 1); break;
+        }
+    } else {
+        switch (G) {
+        case 8: LAK_LONG(8, 2); break;
+        case 16: LAK_LONG(16, 2); break;
+        default: LAK_LONG(32, 2); break;
+        }
     }
 #undef LAK_LONG
     return check_launch("csr_spmv (long rows)");
@@ -312,12 +330,12 @@ lak_status spmv_long_t(void *y, const int32_t *rp, const int32_t *ci, const void
 
 lak_status launch_spmv_long(lak_dtype dt, void *y, const int32_t *rp, const int32_t *ci,
                             const void *vals, const void *x, int64_t m, int group,
-                            cudaStream_t s) {
+                            bool longer, cudaStream_t s) {
     switch (dt) {
-    case LAK_F32: return spmv_long_t<float>(y, rp, ci, vals, x, m, group, s);
-    case LAK_F64: return spmv_long_t<double>(y, rp, ci, vals, x, m, group, s);
-    case LAK_BF16: return spmv_long_t<__nv_bfloat16>(y, rp, ci, vals, x, m, group, s);
-    case LAK_F16: return spmv_long_t<__half>(y, rp, ci, vals, x, m, group, s);
+    case LAK_F32: return spmv_long_t<float>(y, rp, ci, vals, x, m, group, longer, s);
+    case LAK_F64: return spmv_long_t<double>(y, rp, ci, vals, x, m, group, longer, s);
+    case LAK_BF16: return spmv_long_t<__nv_bfloat16>(y, rp, ci, vals, x, m, group, longer, s);
+    case LAK_F16: return spmv_long_t<__half>(y, rp, ci, vals, x, m, group, longer, s);
     }
     return fail(LAK_EDTYPE, "csr_spmv: unknown dtype %d", (int)dt);
 }

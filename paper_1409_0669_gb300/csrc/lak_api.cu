@@ -599,6 +599,7 @@ struct SpmvPlan {
     Launch L;
     int group;     // lanes per row; 0 = warp-segmented variant
     bool long_rows = false;    // spmv_long_kernel
+    bool longer = false;       // of a mean beyond 100
 };
 
 // Mean row lengths between which the warp-segmented variant is used; below
@@ -662,6 +663,7 @@ lak_status plan_spmv(lak_dtype dt, int64_t m, int64_t n, int64_t nnz, const lak_
             out->L = Launch{kSpmvLongBlock, (int)blocks, 4, LAK_INC_GLOBAL};
             out->group = G;
             out->long_rows = true;
+            out->longer = mean > 100;
             return LAK_OK;
         }
     }
@@ -1308,7 +1310,7 @@ LAK_API lak_status csr_spmv(void *y, const int32_t *row_ptr, const int32_t *col_
     if (st != LAK_OK) return st;
     if (p.long_rows)
         return launch_spmv_long(dtype, y, row_ptr, col_idx, vals, x, m, p.group,
-                                (cudaStream_t)stream);
+                                p.longer, (cudaStream_t)stream);
     return launch_spmv(dtype, y, row_ptr, col_idx, vals, x, m, p.L, p.group, (cudaStream_t)stream);
 }
 

@@ -183,10 +183,11 @@ constexpr int kGemvOffBlock = 256;
 lak_status launch_gemv_col_off(lak_dtype dt, void *y, const void *A, const void *x, int64_t m,
                                int64_t n, int64_t lda, int splits, void *ws, double alpha,
                                double beta, cudaStream_t s);
-// Long rows: `group` lanes per row (4, 8, 16 or 32).
+// Long rows: `group` lanes per row (FP64 4, 8, 16 or 32, else 8, 16 or 32); longer: of a
+// mean beyond 100.
 constexpr int kSpmvLongBlock = 128;
 lak_status launch_spmv_long(lak_dtype dt, void *y, const int32_t *rp, const int32_t *ci,
-                            const void *vals, const void *x, int64_t m, int group,
+                            const void *vals, const void *x, int64_t m, int group, bool longer,
                             cudaStream_t s);
 lak_status launch_spmv(lak_dtype dt, void *y, const int32_t *rp, const int32_t *ci,
                        const void *vals, const void *x, int64_t m, const Launch &L, int group,
